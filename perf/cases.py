@@ -3,8 +3,8 @@
 ``listed()`` names the cases, ``draw(rng)`` gives further ones of the same ranges.  For a case,
 ``prepare`` makes what a caller holds in hand (activations, filled caches, weights, workspaces),
 ``run`` is one pass through the public entry points, ``work`` the bytes and operations the pass
-cannot do without, and ``tolerance`` how far another correct implementation of the same precision
-may be off.  Sizes are those of the benchmark workloads of ``synth.CONFIGS`` and generic ones.
+cannot do without, ``tolerance`` how far another correct implementation of the same precision
+may be off, and ``exact`` what the pass returns in plain 64-bit arithmetic.  Sizes are those of the benchmark workloads of ``synth.CONFIGS`` and generic ones.
 
 Kinds of pass:
   decode    one denoising pass of a stream's newest chunk in one layer: rotate q and k (with the
@@ -353,3 +353,189 @@ def run(state):
     B.ll_clip_attn_backward(cache.h, 0, s["q_out"], s["out"], s["d_out"], s["lse"], s["start"], s["frames"], c["attn_window"],
                             c["grid_h"], c["grid_w"], THETA, s["dq"], s["dk"], s["dv"], s["ws"])
     return [s["dq"], s["dk"], s["dv"]]
+
+
+# ---- the same passes in plain torch, 64 bits ---------------------------------------------------
+#
+# What the library stores in 16 or 8 bits on the way (rotated q and k, cache rows, the forward's
+# output that the backward is handed) is rounded here as well, so that what is left is the error
+# of the arithmetic and of the last rounding.
+
+MAX_SCORES = 1 << 26                                         # score entries held at a time
+
+
+def _round(x):
+    return x.to(BF16).double()
+
+
+def _rotation(c, start, frames):
+    """(cos, sin) [tokens, 1, pairs] of the frames' tokens: the pairs of a head row go to t, then h, then w."""
+    n_h = c["head_dim"] // 6
+    n_t = c["head_dim"] // 2 - 2 * n_h
+
+    def axis(n, pairs):
+        i = torch.arange(pairs, device="cuda", dtype=torch.float64)
+        return n.double()[:, None] * THETA ** (-i / pairs)
+
+    at = torch.arange(frames * c["grid_h"] * c["grid_w"], device="cuda")
+    p = c["grid_h"] * c["grid_w"]
+    angle = torch.cat([axis(start + at // p, n_t), axis(at % p // c["grid_w"], n_h), axis(at % c["grid_w"], n_h)], 1)
+    return angle.cos()[:, None], angle.sin()[:, None]
+
+
+def _rotate(x, cos, sin):
+    a, b = x[..., 0::2], x[..., 1::2]
+    return torch.stack([a * cos - b * sin, a * sin + b * cos], -1).flatten(-2)
+
+
+class _PlainCache:
+    """Sink and ring of one layer, [row, head, dim]."""
+
+    def __init__(self, c):
+        self.c, self.W = c, c["window"]
+        self.p = c["grid_h"] * c["grid_w"]
+        shape = ((c["sink"] + self.W) * self.p, c["heads"], c["head_dim"])
+        self.k, self.v = (torch.zeros(*shape, device="cuda", dtype=torch.float64) for _ in range(2))
+
+    def rows(self, frames):
+        s = self.c["sink"]
+        first = torch.tensor([f if f < s else s + (f - s) % self.W for f in frames], device="cuda")
+        return (first[:, None] * self.p + torch.arange(self.p, device="cuda")).flatten()
+
+    def _stored(self, x):
+        if self.c.get("kv") != "e4m3":
+            return _round(x)
+        scale = torch.tensor(6.0 / 448.0, dtype=torch.float32, device="cuda").double()
+        return (x / scale).clamp(-448, 448).float().to(torch.float8_e4m3fn).double() * scale
+
+    def put(self, k, v, start):
+        """Rows that are rotated already."""
+        at = self.rows(range(start, start + len(k) // self.p))
+        self.k[at], self.v[at] = self._stored(k), self._stored(v)
+
+    def rope_append_kv(self, layer, q, k, v, start, grid_h, grid_w, theta):
+        self.put(_rotate(k.double(), *_rotation(self.c, start, self.c["chunk"])), v.double(), start)
+
+    def visible(self, end, window, first=0):
+        return self.rows(list(range(min(self.c["sink"], end))) + list(range(max(self.c["sink"], end - window, first), end)))
+
+    def stored(self):
+        if self.c.get("kv") == "e4m3":
+            return {"k": None, "v": None}                    # codes: whole values
+        return {"k": self.k.transpose(0, 1), "v": self.v.transpose(0, 1)}
+
+
+def _attend(q, k, v):
+    """softmax(q k^T / sqrt(D)) v and the log of the sums, [rows, heads, D] and [heads, rows]."""
+    out, lse = torch.empty_like(q), torch.empty(q.shape[1], q.shape[0], device="cuda", dtype=torch.float64)
+    step = max(1, MAX_SCORES // len(k))
+    for h in range(q.shape[1]):
+        for i in range(0, len(q), step):
+            s = q[i:i + step, h] @ k[:, h].T * q.shape[2] ** -0.5
+            lse[h, i:i + step] = s.logsumexp(1)
+            out[i:i + step, h] = (s - lse[h, i:i + step, None]).exp_() @ v[:, h]
+    return out, lse
+
+
+def _attend_groups(cache, q, starts, window, first=0):
+    n = cache.c["chunk"] * cache.p
+    parts = []
+    for g, start in enumerate(starts):
+        at = cache.visible(start + cache.c["chunk"], window, first)
+        parts.append(_attend(q[g * n:(g + 1) * n], cache.k[at], cache.v[at]))
+    return torch.cat([o for o, _ in parts]), torch.cat([x for _, x in parts], 1)
+
+
+def _gradients(cache, q, out, d_out, lse, starts, window):
+    c, n = cache.c, cache.c["chunk"] * cache.p
+    dq, dk, dv = torch.zeros_like(q), torch.zeros_like(cache.k), torch.zeros_like(cache.v)
+    delta, scale = (out * d_out).sum(2), c["head_dim"] ** -0.5
+    for g, start in enumerate(starts):
+        at = cache.visible(start + c["chunk"], window)
+        step = max(1, MAX_SCORES // len(at))
+        for h in range(c["heads"]):
+            k, v = cache.k[at, h], cache.v[at, h]
+            dk_h, dv_h = torch.zeros_like(k), torch.zeros_like(v)
+            for i in range(g * n, (g + 1) * n, step):
+                rows = slice(i, min(i + step, (g + 1) * n))
+                w = (q[rows, h] @ k.T * scale - lse[h, rows, None]).exp_()
+                ds = w * (d_out[rows, h] @ v.T - delta[rows, h, None])
+                dq[rows, h] = ds @ k * scale
+                dk_h += ds.T @ q[rows, h] * scale
+                dv_h += w.T @ d_out[rows, h]
+            dk[at, h] += dk_h
+            dv[at, h] += dv_h
+    own = cache.rows(range(starts[0], starts[-1] + c["chunk"]))
+    cos, sin = _rotation(c, starts[0], len(starts) * c["chunk"])
+    return [_rotate(dq, cos, -sin), _rotate(dk[own], cos, -sin), dv[own]]
+
+
+def _rms(x, eps=1e-6):
+    return (x.flatten(1).square().mean(1) + eps).rsqrt()
+
+
+def exact(case, seed):
+    """What `run` returns on `prepare(case, seed)`: draws the inputs in the same order."""
+    c, kind = case, case["kind"]
+    inputs = _Inputs(seed)
+    if kind == "cross":
+        q = inputs.normal(c["n_q"], c["heads"], c["head_dim"])
+        k, v = (inputs.normal(c["n_k"], c["heads"], c["head_dim"]) for _ in range(2))
+        return _attend(q.double(), k.double(), v.double())[0]
+    p, n, heads, dim = c["grid_h"] * c["grid_w"], c["chunk"], c["heads"], c["head_dim"]
+
+    def activations(frames, outliers=0.0):
+        return tuple(inputs.normal(frames * p, heads, dim, outliers=outliers).double() for _ in range(3))
+
+    if kind == "batched":
+        outs = []
+        for pos in _positions(c):
+            cache = _PlainCache(c)
+            _fill(cache, c, inputs, pos + 1, c["outliers"])
+            q, k, v = activations(n, c["outliers"])
+            turn = _rotation(c, pos * n, n)
+            cache.put(_rotate(k, *turn), v, pos * n)
+            q = _rotate(q, *turn)
+            outs.append([_attend_groups(cache, _round(q), [pos * n], c["window"])[0], q, cache.stored()])
+        return outs
+
+    cache = _PlainCache(c)
+    _fill(cache, c, inputs, c["filled"])
+    start = (c["filled"] - 1) * n
+    if kind == "project":
+        width = heads * dim
+        x = inputs.normal(n * p, c["d_model"]).double()
+        w = inputs.normal(3 * width, c["d_model"], scale=c["d_model"] ** -0.5).double()
+        y = x @ w.T + inputs.floats(3 * width, std=0.1).double()
+        q, k, v = (t.reshape(n * p, heads, dim) for t in y.chunk(3, 1))
+        row_scale = None
+        if c["norm"]:
+            gain_q, gain_k = (inputs.floats(width, mean=1.0, std=0.1).double().reshape(heads, dim) for _ in range(2))
+            row_scale, k_scale = _rms(q), _rms(k)
+            q, k = q * gain_q, k * gain_k * k_scale[:, None, None]
+        turn = _rotation(c, start, n)
+        cache.put(_rotate(k, *turn), v, start)
+        return [_rotate(q, *turn), row_scale, cache.stored()]
+    frames = n
+    if kind == "recache":
+        frames = _recached_frames(c)
+        start = c["filled"] * n - frames
+    elif kind in ("clip", "backward"):
+        frames, start = c["clip_chunks"] * n, c["filled"] * n
+    q, k, v = activations(frames)
+    if c.get("norm"):
+        gain_q, gain_k = (inputs.floats(heads * dim, mean=1.0, std=0.1).double().reshape(heads, dim) for _ in range(2))
+        q, k = q * gain_q * _rms(q)[:, None, None], k * gain_k * _rms(k)[:, None, None]
+    turn = _rotation(c, start, frames)
+    cache.put(_rotate(k, *turn), v, start)
+    q = _rotate(q, *turn)
+    if kind == "append":
+        return [q, cache.stored()]
+    starts = range(start, start + frames, n)
+    window, first = c.get("attn_window", c["window"]), start if kind == "recache" else 0
+    out, lse = _attend_groups(cache, _round(q), starts, window, first)
+    if kind == "clip":
+        return [out, lse, q, cache.stored()]
+    if kind == "backward":
+        return _gradients(cache, _round(q), _round(out), inputs.normal(frames * p, heads, dim).double(), lse, starts, window)
+    return [out, q, cache.stored()]
