@@ -70,13 +70,15 @@ constexpr int kMmaWarp = 17;
 // clamped range) on the polynomial path.
 constexpr float kSafeSum = 128.f;
 // Register reallocation draws on what the CTA was launched with: 640 threads x 96
-// registers = (16 softmax warps x 104 + 4 producer-group warps x 64) x 32.  A
-// request beyond that total would block forever.
+// registers = (16 softmax warps x kSoftmaxRegs + 4 producer-group warps x kProducerRegs) x 32.  A
+// request beyond that total would block forever.  At head_dim 64 the softmax warps hold a whole
+// score tile (64 registers), which spills at 104.
 constexpr int kLaunchRegs = 96;
-constexpr int kSoftmaxRegs = 104;
-constexpr int kProducerRegs = 64;
-static_assert(kSoftmaxWarps * kSoftmaxRegs + (kThreads / 32 - kSoftmaxWarps) * kProducerRegs <= (kThreads / 32) * kLaunchRegs,
-              "setmaxnreg targets exceed the CTA's register allocation");
+template <int D> constexpr int kSoftmaxRegs = D == 64 ? 112 : 104;
+template <int D> constexpr int kProducerRegs = D == 64 ? 32 : 64;
+template <int D> constexpr bool kRegsFit =
+    kSoftmaxWarps * kSoftmaxRegs<D> + (kThreads / 32 - kSoftmaxWarps) * kProducerRegs<D> <= (kThreads / 32) * kLaunchRegs;
+static_assert(kRegsFit<64> && kRegsFit<128>, "setmaxnreg targets exceed the CTA's register allocation");
 // 8-key groups (bit k of 16 per 128-key tile) whose exponentials use the cubic instead of the
 // special-function unit.  head_dim 128: none - the special-function unit is not what a step
 // waits for, and the cubic's ten instructions per pair cost time and power (0.4027 ms against
@@ -252,9 +254,9 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
     };
 
     if (warp >= kSoftmaxWarps) {
-        // Register reallocation: the softmax warps hold half an S row pair per thread,
+        // Register reallocation: the softmax warps hold 32 or 64 scores per thread,
         // the producer warpgroup (TMA, MMA and two idle warps) needs little.
-        setmaxnreg_dec<kProducerRegs>();
+        setmaxnreg_dec<kProducerRegs<D>>();
         if (skip) {
             // an earlier CTA gave up: nothing to do
         } else if (warp == kTmaWarp && lane == 0) {
@@ -410,7 +412,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
         }
     } else {
         // ============================= softmax warps =============================
-        setmaxnreg_inc<kSoftmaxRegs>();
+        setmaxnreg_inc<kSoftmaxRegs<D>>();
         if (!skip) [&]() {
             const int q = warp & 3;                        // TMEM lane quarter this warp may touch
             const int w = warp >> 3;                       // lane (query tile) of the column
@@ -450,7 +452,25 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                     if (!__all_sync(0xffffffffu, wait(kSFull + w, sc, j))) return;
                     tc_fence_after_sync();
                     const int nvalid = kit.valid();
-                    // The tile is taken in two 64-key pieces.  A piece's exponentials are computed
+                    // head_dim 64: the whole tile goes to registers at once and the S buffer back to the
+                    // MMA warp, so that the next QK and its hand-overs run under all of this step's
+                    // weights (2480 -> 2350 clk per step; 24 heads of 64: 0.744 -> 0.707 ms at the power
+                    // limit).  At head_dim 128 it is taken 64 columns at a time: there the early release
+                    // costs cycles and energy (0.478 ms against 0.514 ms; 455 mJ against 488 mJ per call).
+                    constexpr bool kWholeTile = D == 64;
+                    uint32_t s_tile[kWholeTile ? 64 : 32];
+                    auto release_s = [&]() {
+                        tmem_wait_ld();
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(kSEmpty + w));
+                    };
+                    if (kWholeTile) {
+                        tmem_ld_16x256b_x8(t_s, s_tile);
+                        tmem_ld_16x256b_x8(t_s + 64, s_tile + (kWholeTile ? 32 : 0));
+                        release_s();
+                    }
+                    // The tile is worked through in two 64-key pieces.  A piece's exponentials are computed
                     // against the rows' current reference maxima straight away; its sums then tell
                     // whether that was safe (no weight can exceed the sum).  Only when some sum in
                     // the warp is large or not finite - always on a column's first piece, where the
@@ -458,15 +478,11 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                     // what has been accumulated rescaled, and the piece redone.
 #pragma unroll
                     for (int piece = 0; piece < 2; ++piece) {
-                        uint32_t v[32];
+                        uint32_t *v = s_tile + (kWholeTile ? 32 * piece : 0);
                         uint32_t pp[16];                           // the piece's P: 16 rows x 64 keys per warp
-                        tmem_ld_16x256b_x8(t_s + 64 * piece, v);
-                        tmem_wait_ld();
-                        if (piece == 1) {
-                            // the whole tile is in registers now: the S buffer may take the next QK
-                            tc_fence_before_sync();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(bar(kSEmpty + w));
+                        if (!kWholeTile) {
+                            tmem_ld_16x256b_x8(t_s + 64 * piece, v);
+                            if (piece == 0) tmem_wait_ld(); else release_s();
                         }
                         if (nvalid < kKeyTile) mask_piece(v, 64 * piece, cq, nvalid);
                         uint64_t ts_a = 0ull, ts_b = 0ull;         // the piece's sums, two partials per row
