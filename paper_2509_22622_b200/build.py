@@ -10,7 +10,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libllattn.so")
 SOURCES = ["ll_host.cu", "rope_append.cu", "attn_sm100.cu", "attn_simt.cu", "rope_static.cu", "qkv_gemm.cu", "attn_bwd.cu"]
-HEADERS = ["ll_internal.h", "ptx.cuh", "bounded_wait.cuh", "rope_math.cuh", os.path.join(ROOT, "include", "llattn.h"),
+HEADERS = ["ll_internal.h", "ptx.cuh", "bounded_wait.cuh", "exp2_poly.cuh", "rope_math.cuh", os.path.join(ROOT, "include", "llattn.h"),
            os.path.join(ROOT, "include", "llattn_debug.h")]
 
 NVCC_FLAGS = [

@@ -50,11 +50,6 @@ __device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_
                  : "memory");
 }
 
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
 // delta[h][i] = sum_d d_out[i][h][d] * out[i][h][d]: one warp per (row, head).
 template <int D>
 __global__ void __launch_bounds__(256) bwd_delta_kernel(const __grid_constant__ BwdParams p)

@@ -67,7 +67,9 @@ constexpr int kMmaWarp = 17;
 // A piece's 16 weights per thread and row were safe to compute if they sum to less than this:
 // no weight can exceed the sum, and a score too far above the row's reference shows up as a
 // weight of at least 2^127 on the special-function unit and of just under 256 (the top of its
-// clamped range) on the polynomial path.
+// clamped range) on the polynomial path.  (A limit of 2^32 moves the references less often and makes
+// eight streams with outliers 6 % faster, but the largest weight of a row is then hardly ever exactly
+// 1, and its rounding shows: relative error 1.8e-3 instead of 1.6e-3.)
 constexpr float kSafeSum = 128.f;
 // Register reallocation draws on what the CTA was launched with: 640 threads x 96
 // registers = (16 softmax warps x kSoftmaxRegs + 4 producer-group warps x kProducerRegs) x 32.  A
@@ -122,7 +124,6 @@ struct KeyIter {
         }
     }
     __device__ int row() const { return g->k_start[r] + off; }
-    __device__ int valid() const { return min(kKeyTile, g->k_len[r] - off); }
     __device__ void next()
     {
         off += kKeyTile;
@@ -201,6 +202,150 @@ __device__ __forceinline__ void mask_piece(uint32_t *v, int col0, int cq, int nv
         if (col0 + 8 * k + cq >= nvalid) v[4 * k] = v[4 * k + 2] = 0xff800000u;
         if (col0 + 8 * k + cq + 1 >= nvalid) v[4 * k + 1] = v[4 * k + 3] = 0xff800000u;
     }
+}
+
+// Where a softmax warp's 16 rows sit: q = TMEM lane quarter, w = lane (query tile) of the column, h = half
+// of the quarter.
+struct WarpRows {
+    int lane, q, w, h;
+    __device__ WarpRows(int warp, int lane_) : lane(lane_), q(warp & 3), w(warp >> 3), h((warp >> 2) & 1) {}
+    __device__ int first() const { return 32 * q + 16 * h; }              // inside the lane's 128-row tile
+    __device__ int row_a() const { return first() + (lane >> 2); }        // row of registers 4k+{0,1}; 4k+{2,3} are row_a + 8
+    __device__ int slab() const { return w * 8 + q * 2 + h; }
+};
+
+// 64 columns (chunk ch) of the warp's rows, packed as pp of a softmax piece, to the output.  They go through
+// the lane's P tile (its last PV has completed; every warp uses its own 16 rows), so that eight
+// threads store 128 contiguous bytes of a row instead of four storing 16: 30.0 -> 26.7 us for a launch of
+// two columns of four steps per CTA (4680 queries, 512 keys, 12 heads of 128).
+template <int D>
+__device__ __forceinline__ void store_rows(const AttnParams &p, const AttnItem &item, const Segment &s, const WarpRows &wr, uint32_t p_smem,
+                                           uint32_t p_at, int ch, const uint32_t (&pk)[16])
+{
+    using C = Cfg<D>;
+    const uint32_t at = p_at + ch * C::kAtomBytes;
+    stmatrix_x4(at, pk[0], pk[2], pk[4], pk[6]);                       // rows a, chunks 0..3
+    stmatrix_x4(at ^ 64u, pk[8], pk[10], pk[12], pk[14]);               // rows a, chunks 4..7
+    stmatrix_x4(at + 8 * 128, pk[1], pk[3], pk[5], pk[7]);              // rows a + 8
+    stmatrix_x4((at ^ 64u) + 8 * 128, pk[9], pk[11], pk[13], pk[15]);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {                                      // rows 4 i + lane / 8 of the warp's 16, 16-byte chunk lane % 8
+        const int r = 4 * i + (wr.lane >> 3), row = 128 * wr.w + wr.first() + r;
+        const uint4 x = ld_shared_v4(p_smem + wr.w * C::kPBytes + ch * C::kAtomBytes + (uint32_t)(wr.first() + r) * 128 +
+                                     ((uint32_t)((wr.lane ^ r) & 7) << 4));
+        if (row < s.rows_valid)
+            *reinterpret_cast<uint4 *>(item.out + ((size_t)(s.q0 + row) * p.heads + s.head) * D + 64 * ch + 8 * (wr.lane & 7)) = x;
+    }
+}
+
+// The log of the rows' sums (reference maxima m, sums l of rows a and a + 8), when the caller wants it.
+__device__ __forceinline__ void store_lse(const AttnItem &item, const Segment &s, const WarpRows &wr, float m_a, float m_b, float l_a, float l_b)
+{
+    if (!item.lse || (wr.lane & 3)) return;
+    const int row = 128 * wr.w + wr.row_a();
+    float *lse = item.lse + (size_t)s.head * item.nq_total + s.q0 + row;
+    if (row < s.rows_valid) lse[0] = (m_a + log2f(l_a)) * 0.6931471805599453f;
+    if (row + 8 < s.rows_valid) lse[8] = (m_b + log2f(l_b)) * 0.6931471805599453f;
+}
+
+// The shares that hold parts of a split column: the first one, and how many (they are consecutive).
+__device__ __forceinline__ void parts_of(const AttnParams &p, const Segment &s, int own, int &i0, int &n_parts)
+{
+    int i1 = own;
+    i0 = own;
+    while (p.share_begin[i0] > s.col_begin) --i0;
+    while (p.share_begin[i1 + 1] < s.col_begin + p.g[s.g].n_kt) ++i1;
+    n_parts = i1 - i0 + 1;
+}
+
+// Merges the parts of a split column for the warp's rows: reference maxima and sums first, then the O rows,
+// always from the slots and in the order of the parts, so the result does not depend on
+// which part happened to arrive last.  Bound by the latency of its loads, which therefore go out kBatch
+// parts at a time (columns of three parts: 6.5 -> 3 us).
+template <int D>
+__device__ __forceinline__ void merge_column(const AttnParams &p, const Segment &s, int own, const WarpRows &wr, uint32_t p_smem, uint32_t p_at)
+{
+    constexpr int kBatch = D == 64 ? 2 : 4;
+    constexpr size_t kSlotFloats = (size_t)kQTileRows * (D + 2);
+    int i0, n_parts;
+    parts_of(p, s, own, i0, n_parts);
+    const AttnItem &item = p.item[p.g[s.g].item];
+    const int last = i0 + n_parts - 1, slab = wr.slab(), lane = wr.lane;
+    auto part_slot = [&](int i) -> const float * { return p.partial + (size_t)(2 * i + (i == i0 ? 1 : 0)) * kSlotFloats; };
+    float2 pa[kBatch], pb[kBatch];                     // (reference, sum) of a batch of parts, rows a and a + 8
+    auto load_ml = [&](int first) {
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const float2 *ml = reinterpret_cast<const float2 *>(part_slot(min(first + u, last)) + (size_t)kQTileRows * D) + slab * 16 + (lane >> 2);
+            pa[u] = __ldcg(ml);
+            pb[u] = __ldcg(ml + 8);
+        }
+    };
+    float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
+    for (int i = i0; i <= last; i += kBatch) {
+        load_ml(i);                                    // (the last part again behind the last: no new maximum)
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            m_a = fmaxf(m_a, pa[u].x);
+            m_b = fmaxf(m_b, pb[u].x);
+        }
+    }
+    for (int i = i0; i <= last; i += kBatch) {
+        if (n_parts > kBatch) load_ml(i);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            if (i + u > last) break;
+            l_a = fmaf(pa[u].y, ex2(pa[u].x - m_a), l_a);
+            l_b = fmaf(pb[u].y, ex2(pb[u].x - m_b), l_b);
+        }
+    }
+    const float v_scale = item.v_scale ? __ldg(item.v_scale + s.head) : 1.f;   // 8-bit caches: value codes x scale
+    const float inv_a = v_scale / l_a, inv_b = v_scale / l_b;
+#pragma unroll 1
+    for (int ch = 0; ch < D / 64; ++ch) {
+        uint32_t pk[16];
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            float o[16];                               // 32 columns: of each 16, this thread's four of row a, then of row a + 8
+#pragma unroll
+            for (int k = 0; k < 16; ++k) o[k] = 0.f;
+            for (int i = i0; i <= last; i += kBatch) {
+                float4 x[kBatch][4];
+                if (n_parts > kBatch) load_ml(i);
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    const float4 *src = reinterpret_cast<const float4 *>(part_slot(min(i + u, last))) +
+                                        (size_t)(slab * (D / 16) + 4 * ch + 2 * half) * 64 + lane;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) x[u][k] = __ldcg(src + 32 * k);
+                }
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    if (i + u > last) break;
+                    const float wa = ex2(pa[u].x - m_a) * inv_a, wb = ex2(pb[u].x - m_b) * inv_b;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float wk = (k & 1) ? wb : wa;
+                        o[4 * k] = fmaf(x[u][k].x, wk, o[4 * k]);
+                        o[4 * k + 1] = fmaf(x[u][k].y, wk, o[4 * k + 1]);
+                        o[4 * k + 2] = fmaf(x[u][k].z, wk, o[4 * k + 2]);
+                        o[4 * k + 3] = fmaf(x[u][k].w, wk, o[4 * k + 3]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {          // 8-column group 4 half + 2 k + g
+                    pk[2 * (4 * half + 2 * k + g)] = cvt_bf16x2(o[8 * k + 2 * g], o[8 * k + 2 * g + 1]);
+                    pk[2 * (4 * half + 2 * k + g) + 1] = cvt_bf16x2(o[8 * k + 4 + 2 * g], o[8 * k + 5 + 2 * g]);
+                }
+        }
+        store_rows<D>(p, item, s, wr, p_smem, p_at, ch, pk);
+    }
+    store_lse(item, s, wr, m_a, m_b, l_a, l_b);
+    __syncwarp();                                      // the P rows are read before another column's are staged
 }
 
 template <int D>
@@ -414,27 +559,32 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
         // ============================= softmax warps =============================
         setmaxnreg_inc<kSoftmaxRegs<D>>();
         if (!skip) [&]() {
-            const int q = warp & 3;                        // TMEM lane quarter this warp may touch
-            const int w = warp >> 3;                       // lane (query tile) of the column
-            const int h = (warp >> 2) & 1;                 // which 16 rows of the quarter
-            const uint32_t lane_off = (uint32_t)(32 * q + 16 * h) << 16;
+            const WarpRows wr(warp, lane);
+            const int w = wr.w;
+            const uint32_t lane_off = (uint32_t)wr.first() << 16;   // the TMEM lanes this warp reads
             const uint32_t t_s = tmem + lane_off + C::kColS + 128 * w;
             const uint32_t t_o = tmem + lane_off + C::kColO + D * w;
-            const int row_a = 32 * q + 16 * h + (lane >> 2);   // row of registers 4k+{0,1}; 4k+{2,3} are row_a + 8
             const int cq = 2 * (lane & 3);                     // first of this thread's two columns in each group of 8
-            const int slab = w * 8 + q * 2 + h;
             // P goes to shared memory with stmatrix: of the warp's 16 rows x 64 keys, one call
             // stores four 8-row x 8-key blocks (a block row = one 16-byte chunk); lane 8m + r gives the
             // address of row r of the block holding chunk m, which sits at chunk position m ^ r.
             // Chunks 4..7 are at the same address ^ 64, the second eight rows 1024 bytes on.
-            const uint32_t p_at = p_smem + w * C::kPBytes + (uint32_t)(32 * q + 16 * h + (lane & 7)) * 128 +
+            const uint32_t p_at = p_smem + w * C::kPBytes + (uint32_t)(wr.first() + (lane & 7)) * 128 +
                                   ((uint32_t)((lane >> 3) ^ (lane & 7)) << 4);
             uint32_t sc = 0, oc = 0;
+            constexpr bool kMergeLate = D == 64;
+            uint32_t to_merge = 0;                             // which of the CTA's two parts complete a column here
             Segment s;
             for (WorkIter it(p, cta); it.next(s);) {
                 if (w >= s.n_sub) continue;
                 const AttnGroup &G = p.g[s.g];
-                KeyIter kit(&G, s.kt0);
+                // keys left in the current run of the visible set (its last tile may be ragged)
+                int run, left;
+                {
+                    const KeyIter first(&G, s.kt0);
+                    run = first.r;
+                    left = G.k_len[run] - first.off;
+                }
                 // log2(e)/sqrt(D), times the head's key scale when the cache holds 8-bit codes
                 const float *k_scale = p.item[G.item].k_scale;
                 const float c = k_scale ? p.scale_log2 * __ldg(k_scale + s.head) : p.scale_log2;
@@ -442,16 +592,18 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 // per-token factor was left out of the stored q)
                 float c_a = c, c_b = c;
                 if (const float *q_scale = p.item[G.item].q_scale) {
-                    const int r = 128 * w + row_a;
+                    const int r = 128 * w + wr.row_a();
                     if (r < s.rows_valid) c_a *= __ldg(q_scale + s.q0 + r);
                     if (r + 8 < s.rows_valid) c_b *= __ldg(q_scale + s.q0 + r + 8);
                 }
                 float m_a = -INFINITY, m_b = -INFINITY;
                 uint64_t acc_a = 0ull, acc_b = 0ull;       // two partial sums per row
-                for (int j = s.kt0; j < s.kt1; ++j, kit.next(), ++sc) {
+                for (int j = s.kt0; j < s.kt1; ++j, ++sc) {
                     if (!__all_sync(0xffffffffu, wait(kSFull + w, sc, j))) return;
                     tc_fence_after_sync();
-                    const int nvalid = kit.valid();
+                    const int nvalid = min(left, kKeyTile);
+                    left -= kKeyTile;
+                    if (left <= 0 && j + 1 < s.kt1) left = G.k_len[++run];
                     // head_dim 64: the whole tile goes to registers at once and the S buffer back to the
                     // MMA warp, so that the next QK and its hand-overs run under all of this step's
                     // weights (2480 -> 2350 clk per step; 24 heads of 64: 0.744 -> 0.707 ms at the power
@@ -473,9 +625,9 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                     // The tile is worked through in two 64-key pieces.  A piece's exponentials are computed
                     // against the rows' current reference maxima straight away; its sums then tell
                     // whether that was safe (no weight can exceed the sum).  Only when some sum in
-                    // the warp is large or not finite - always on a column's first piece, where the
-                    // references are -inf - are the exact row maxima taken, the references moved,
-                    // what has been accumulated rescaled, and the piece redone.
+                    // the warp is too large or not finite - and on a column's first piece, which has
+                    // no references yet - are the exact row maxima taken, the references moved,
+                    // what has been accumulated rescaled, and the piece computed against them.
 #pragma unroll
                     for (int piece = 0; piece < 2; ++piece) {
                         uint32_t *v = s_tile + (kWholeTile ? 32 * piece : 0);
@@ -486,7 +638,8 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                         }
                         if (nvalid < kKeyTile) mask_piece(v, 64 * piece, cq, nvalid);
                         uint64_t ts_a = 0ull, ts_b = 0ull;         // the piece's sums, two partials per row
-                        {
+                        const bool fresh = piece == 0 && j == s.kt0;   // nothing accumulated yet, no references
+                        if (!fresh) {
                             const uint64_t na2 = pack2(-m_a, -m_a), nb2 = pack2(-m_b, -m_b);
                             const uint64_t c2a = pack2(c_a, c_a), c2b = pack2(c_b, c_b);
                             const PolyRow ra{c_a * (1.f / 128.f), ((float)kPolyLow - m_a) * (1.f / 128.f)};
@@ -528,15 +681,14 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                                 }
                             }
                         }
-                        float sa, sb;
-                        {
-                            float x0, x1;
+                        bool move = fresh;
+                        if (!fresh) {
+                            float x0, x1, y0, y1;
                             unpack2(ts_a, x0, x1);
-                            sa = x0 + x1;
-                            unpack2(ts_b, x0, x1);
-                            sb = x0 + x1;
+                            unpack2(ts_b, y0, y1);
+                            move = __any_sync(0xffffffffu, !(x0 + x1 < kSafeSum) || !(y0 + y1 < kSafeSum));
                         }
-                        if (__any_sync(0xffffffffu, !(sa < kSafeSum) || !(sb < kSafeSum))) {
+                        if (move) {
                             // exact maxima of the piece's rows: 16 columns per thread, then across the quad
                             float ta = fmaxf(as_f(v[0]), as_f(v[1])), tb = fmaxf(as_f(v[2]), as_f(v[3]));
 #pragma unroll
@@ -548,7 +700,6 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                             tb = fmaxf(tb, __shfl_xor_sync(0xffffffffu, tb, 1));
                             ta = fmaxf(ta, __shfl_xor_sync(0xffffffffu, ta, 2)) * c_a;
                             tb = fmaxf(tb, __shfl_xor_sync(0xffffffffu, tb, 2)) * c_b;
-                            const bool fresh = j == s.kt0 && piece == 0;     // nothing accumulated yet
                             const float new_a = fresh ? ta : fmaxf(m_a, ta), new_b = fresh ? tb : fmaxf(m_b, tb);
                             const float al_a = fresh ? 0.f : ex2(m_a - new_a), al_b = fresh ? 0.f : ex2(m_b - new_b);
                             m_a = new_a;
@@ -581,23 +732,23 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                                 if (!__all_sync(0xffffffffu, wait(kPEmpty + w, sc - 1, (int)sc))) return;
                                 tc_fence_after_sync();
 #pragma unroll 1
-                                for (int ch = 0; ch < C::kOChunks; ++ch) {
-                                    uint32_t o[32];
-                                    tmem_ld_16x256b_x8(t_o + 64 * ch, o);
+                                for (int ch = 0; ch < D / 32; ++ch) {
+                                    uint32_t o[16];
+                                    tmem_ld_16x256b_x4(t_o + 32 * ch, o);
                                     tmem_wait_ld();
 #pragma unroll
-                                    for (int k = 0; k < 8; ++k) {
+                                    for (int k = 0; k < 4; ++k) {
                                         o[4 * k] = as_u(as_f(o[4 * k]) * al_a);
                                         o[4 * k + 1] = as_u(as_f(o[4 * k + 1]) * al_a);
                                         o[4 * k + 2] = as_u(as_f(o[4 * k + 2]) * al_b);
                                         o[4 * k + 3] = as_u(as_f(o[4 * k + 3]) * al_b);
                                     }
-                                    tmem_st_16x256b_x8(t_o + 64 * ch, o);
+                                    tmem_st_16x256b_x4(t_o + 32 * ch, o);
                                 }
                                 tmem_wait_st();
                                 tc_fence_before_sync();
                             }
-                            // the piece again, against the new references
+                            // the piece against the new references
                             const uint64_t na2 = pack2(-m_a, -m_a), nb2 = pack2(-m_b, -m_b);
                             const uint64_t c2a = pack2(c_a, c_a), c2b = pack2(c_b, c_b);
                             ts_a = ts_b = 0ull;
@@ -650,128 +801,65 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                     l_a += __shfl_xor_sync(0xffffffffu, l_a, 2);
                     l_b += __shfl_xor_sync(0xffffffffu, l_b, 2);
                 }
-                const int row = 128 * w + row_a;               // row inside the column
-                const bool live_a = row < s.rows_valid, live_b = row + 8 < s.rows_valid;
                 const AttnItem &item = p.item[G.item];
-                ll_bf16 *dst_a = item.out + ((size_t)(s.q0 + row) * p.heads + s.head) * D;
-                ll_bf16 *dst_b = dst_a + (size_t)8 * p.heads * D;
-                float *lse_a = item.lse ? item.lse + (size_t)s.head * item.nq_total + s.q0 + row : nullptr;
-
-                bool finish = true;            // this warp writes the output rows
-                int i0 = 0, n_parts = 1;
-                const bool whole = s.kt0 == 0 && s.kt1 == G.n_kt;
-                const size_t slot_floats = (size_t)kQTileRows * (D + 2);
-                if (!whole) {
-                    // leave this part in its slot and count the arrival
-                    // (the parts of a column sit in consecutive shares; i0 = the share with its first step)
-                    const int own = p.share_of_cta[cta];
-                    int i1 = own;
-                    i0 = own;
-                    while (p.share_begin[i0] > s.col_begin) --i0;
-                    while (p.share_begin[i1 + 1] < s.col_begin + G.n_kt) ++i1;
-                    n_parts = i1 - i0 + 1;
-                    float *slot = p.partial + (size_t)(2 * own + (s.kt0 == 0 ? 1 : 0)) * slot_floats;
+                if (s.kt0 == 0 && s.kt1 == G.n_kt) {
+                    // a whole column: normalise and store
+                    const float v_scale = item.v_scale ? __ldg(item.v_scale + s.head) : 1.f;   // 8-bit caches: value codes x scale
+                    const float inv_a = v_scale / l_a, inv_b = v_scale / l_b;
+#pragma unroll 1
+                    for (int ch = 0; ch < C::kOChunks; ++ch) {
+                        uint32_t o[32], pk[16];
+                        tmem_ld_16x256b_x8(t_o + 64 * ch, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            pk[2 * k] = cvt_bf16x2(as_f(o[4 * k]) * inv_a, as_f(o[4 * k + 1]) * inv_a);
+                            pk[2 * k + 1] = cvt_bf16x2(as_f(o[4 * k + 2]) * inv_b, as_f(o[4 * k + 3]) * inv_b);
+                        }
+                        store_rows<D>(p, item, s, wr, p_smem, p_at, ch, pk);
+                    }
+                    store_lse(item, s, wr, m_a, m_b, l_a, l_b);
+                } else {
+                    // a part of a column: into its slot, and count the arrival; the warp that arrives last
+                    // merges the parts.  At head_dim 64 it does so when the CTA's steps are done (a CTA has at
+                    // most two parts: the end of its share's first column and the beginning of the last
+                    // one): with the merge inside the column loop the softmax of a whole tile does not fit the
+                    // registers (0.710 -> 0.815 ms, 24 heads of 64); at 128 it fits, and the loop
+                    // is faster with it (0.484 against 0.490 ms).
+                    const int own = p.share_of_cta[cta], which = s.kt0 == 0 ? 1 : 0;
+                    int i0, n_parts;
+                    parts_of(p, s, own, i0, n_parts);
+                    float *slot = p.partial + (size_t)(2 * own + which) * kQTileRows * (D + 2);
 #pragma unroll 1
                     for (int ch = 0; ch < C::kOChunks; ++ch) {
                         uint32_t o[32];
                         tmem_ld_16x256b_x8(t_o + 64 * ch, o);
                         tmem_wait_ld();
+                        uint4 *dst = reinterpret_cast<uint4 *>(slot) + (size_t)(wr.slab() * (D / 16) + 4 * ch) * 64 + lane;
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            float2 *dst = reinterpret_cast<float2 *>(slot) +
-                                          ((size_t)(slab * (D / 8) + 8 * ch + k) * 2) * 32 + lane;
-                            dst[0] = make_float2(as_f(o[4 * k]), as_f(o[4 * k + 1]));
-                            dst[32] = make_float2(as_f(o[4 * k + 2]), as_f(o[4 * k + 3]));
+                        for (int k = 0; k < 4; ++k) {              // 16 columns: this thread's four of row a, then of row a + 8
+                            dst[64 * k] = make_uint4(o[8 * k], o[8 * k + 1], o[8 * k + 4], o[8 * k + 5]);
+                            dst[64 * k + 32] = make_uint4(o[8 * k + 2], o[8 * k + 3], o[8 * k + 6], o[8 * k + 7]);
                         }
                     }
                     if ((lane & 3) == 0) {
-                        float2 *ml = reinterpret_cast<float2 *>(slot + (size_t)kQTileRows * D) + slab * 16 + (lane >> 2);
+                        float2 *ml = reinterpret_cast<float2 *>(slot + (size_t)kQTileRows * D) + wr.slab() * 16 + (lane >> 2);
                         ml[0] = make_float2(m_a, l_a);
                         ml[8] = make_float2(m_b, l_b);
                     }
                     __threadfence();
                     __syncwarp();
                     uint32_t arrived = 0;
-                    if (lane == 0) arrived = atomicAdd(p.counters + i0 * kSlabs + slab, 1u);
+                    if (lane == 0) arrived = atomicAdd(p.counters + i0 * kSlabs + wr.slab(), 1u);
                     arrived = __shfl_sync(0xffffffffu, arrived, 0);
-                    finish = arrived == (uint32_t)(n_parts - 1);
-                    if (finish) {
-                        if (lane == 0) p.counters[i0 * kSlabs + slab] = 0;    // ready for the next launch
-                        __threadfence();
-                    }
-                }
-                if (finish) {
-                    // the slot of part i, and this thread's two (max, sum) pairs in it
-                    auto part_slot = [&](int i) -> const float * {
-                        return p.partial + (size_t)(2 * i + (i == i0 ? 1 : 0)) * slot_floats;
-                    };
-                    auto part_ml = [&](const float *slot) -> const float2 * {
-                        return reinterpret_cast<const float2 *>(slot + (size_t)kQTileRows * D) + slab * 16 + (lane >> 2);
-                    };
-                    // Reference maximum and sum over all parts.  A split column is merged from the
-                    // slots alone, the own part included, in the order of the parts, so the result
-                    // does not depend on which part happened to arrive last.
-                    float mm_a = m_a, mm_b = m_b, ll_a = l_a, ll_b = l_b;
-                    if (!whole) {
-                        for (int i = i0; i < i0 + n_parts; ++i) {
-                            const float2 *ml = part_ml(part_slot(i));
-                            mm_a = fmaxf(mm_a, __ldcg(ml).x);
-                            mm_b = fmaxf(mm_b, __ldcg(ml + 8).x);
-                        }
-                        ll_a = ll_b = 0.f;
-                        for (int i = i0; i < i0 + n_parts; ++i) {
-                            const float2 *ml = part_ml(part_slot(i));
-                            const float2 pa = __ldcg(ml), pb = __ldcg(ml + 8);
-                            ll_a = fmaf(pa.y, ex2(pa.x - mm_a), ll_a);
-                            ll_b = fmaf(pb.y, ex2(pb.x - mm_b), ll_b);
-                        }
-                    }
-                    const float v_scale = item.v_scale ? __ldg(item.v_scale + s.head) : 1.f;   // 8-bit caches: value codes x scale
-                    const float inv_a = v_scale / ll_a, inv_b = v_scale / ll_b;
-#pragma unroll 1
-                    for (int ch = 0; ch < C::kOChunks; ++ch) {
-                        uint32_t o[32];
-                        if (whole) {
-                            tmem_ld_16x256b_x8(t_o + 64 * ch, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                o[4 * k] = as_u(as_f(o[4 * k]) * inv_a);
-                                o[4 * k + 1] = as_u(as_f(o[4 * k + 1]) * inv_a);
-                                o[4 * k + 2] = as_u(as_f(o[4 * k + 2]) * inv_b);
-                                o[4 * k + 3] = as_u(as_f(o[4 * k + 3]) * inv_b);
-                            }
+                    if (arrived == (uint32_t)(n_parts - 1)) {
+                        if (lane == 0) p.counters[i0 * kSlabs + wr.slab()] = 0;    // ready for the next launch
+                        if (kMergeLate) {
+                            to_merge |= 1u << which;
                         } else {
-#pragma unroll
-                            for (int k = 0; k < 32; ++k) o[k] = 0u;
-                            for (int i = i0; i < i0 + n_parts; ++i) {
-                                const float *slot = part_slot(i);
-                                const float2 *ml = part_ml(slot);
-                                const float wa = ex2(__ldcg(ml).x - mm_a) * inv_a, wb = ex2(__ldcg(ml + 8).x - mm_b) * inv_b;
-#pragma unroll
-                                for (int k = 0; k < 8; ++k) {
-                                    const float2 *src = reinterpret_cast<const float2 *>(slot) +
-                                                        ((size_t)(slab * (D / 8) + 8 * ch + k) * 2) * 32 + lane;
-                                    const float2 xa = __ldcg(src), xb = __ldcg(src + 32);
-                                    o[4 * k] = as_u(fmaf(xa.x, wa, as_f(o[4 * k])));
-                                    o[4 * k + 1] = as_u(fmaf(xa.y, wa, as_f(o[4 * k + 1])));
-                                    o[4 * k + 2] = as_u(fmaf(xb.x, wb, as_f(o[4 * k + 2])));
-                                    o[4 * k + 3] = as_u(fmaf(xb.y, wb, as_f(o[4 * k + 3])));
-                                }
-                            }
+                            __threadfence();
+                            merge_column<D>(p, s, own, wr, p_smem, p_at);
                         }
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const int col = 64 * ch + 8 * k + cq;
-                            if (live_a)
-                                *reinterpret_cast<uint32_t *>(dst_a + col) = cvt_bf16x2(as_f(o[4 * k]), as_f(o[4 * k + 1]));
-                            if (live_b)
-                                *reinterpret_cast<uint32_t *>(dst_b + col) = cvt_bf16x2(as_f(o[4 * k + 2]), as_f(o[4 * k + 3]));
-                        }
-                    }
-                    if (lse_a && (lane & 3) == 0) {
-                        if (live_a) lse_a[0] = (mm_a + log2f(ll_a)) * 0.6931471805599453f;
-                        if (live_b) lse_a[8] = (mm_b + log2f(ll_b)) * 0.6931471805599453f;
                     }
                 }
                 // the O columns may be overwritten by the next column's first PV
@@ -779,6 +867,14 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kOEmpty + w));
                 ++oc;
+            }
+            if (kMergeLate && to_merge) {
+                __threadfence();                                   // the other parts' slots, seen complete above
+                const int own = p.share_of_cta[cta];
+                for (WorkIter it(p, cta); it.next(s);) {
+                    if (w >= s.n_sub || (s.kt0 == 0 && s.kt1 == p.g[s.g].n_kt)) continue;
+                    if ((to_merge >> (s.kt0 == 0 ? 1 : 0)) & 1u) merge_column<D>(p, s, own, wr, p_smem, p_at);
+                }
             }
         }();
     }
