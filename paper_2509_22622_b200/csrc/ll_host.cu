@@ -831,18 +831,18 @@ int ll_qkv_proj_append(ll_cache *c, int layer, const ll_bf16 *x, int d_model, co
         ll::QkvParams p;
         memset(&p, 0, sizeof p);
         p.n_tokens = n_frames * c->P; p.d_model = d_model; p.heads = c->H; p.head_dim = c->D;
-        p.m_tiles = (p.n_tokens + 127) / 128;
+        p.m_tiles = (p.n_tokens + 255) / 256;
         {
-            // tile width: the one whose last round of tiles leaves the SMs less idle
-            const int hd = c->H * c->D, sms = c->sm_count > 0 ? c->sm_count : 148;
+            // tile width: the one whose last round of tiles leaves the SM pairs less idle (wider on a tie)
+            const int hd = c->H * c->D, pairs = std::max(1, (c->sm_count > 0 ? c->sm_count : 148) / 2);
             long long best = -1;
-            for (int tn : {256, 192}) {
+            for (int tn : {256, 192, 128}) {
                 if (hd % tn) continue;
-                const long long tiles = (long long)p.m_tiles * (3 * hd / tn), cost = (tiles + sms - 1) / sms * tn;
+                const long long tiles = (long long)p.m_tiles * (3 * hd / tn), cost = (tiles + pairs - 1) / pairs * tn;
                 if (best < 0 || cost < best) { best = cost; p.tile_n = tn; }
             }
             p.n_tiles = 3 * hd / p.tile_n;
-            p.ssq_slots = 2 * hd / p.tile_n;
+            p.ssq_slots = p.tile_n == 128 ? hd / 128 : 2 * hd / p.tile_n;   // at most one per 96 features
         }
         p.P = c->P; p.grid_w = grid_w; p.n_t = rp.n_t; p.n_h = rp.n_h;
         p.with_norm = with_norm ? 1 : 0; p.eps = eps;
@@ -861,7 +861,7 @@ int ll_qkv_proj_append(ll_cache *c, int layer, const ll_bf16 *x, int d_model, co
                        (uint64_t)p.n_tokens * d_model * 2, 128, 1);
         if (s != LL_OK) return s;
         s = encode_map(&wmap, w_qkv, (uint64_t)d_model, (uint64_t)3 * c->H * c->D, 1, (uint64_t)d_model * 2,
-                       (uint64_t)3 * c->H * c->D * d_model * 2, (uint32_t)p.tile_n, 1);
+                       (uint64_t)3 * c->H * c->D * d_model * 2, (uint32_t)p.tile_n / 2, 1);
         if (s != LL_OK) return s;
         cudaError_t e = ll::launch_qkv_gemm(p, xmap, wmap, c->sm_count > 0 ? c->sm_count : 148, (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e, "qkv projection kernel");
