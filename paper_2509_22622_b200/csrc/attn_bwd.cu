@@ -54,6 +54,8 @@ __device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_
 template <int D>
 __global__ void __launch_bounds__(256) bwd_delta_kernel(const __grid_constant__ BwdParams p)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= (long long)p.nq_total * p.heads) return;
@@ -252,10 +254,12 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kBars; ++i) mbar_init(bar(i), (i == kSFree || i == kDsFull) ? kComputeWarps : 1);
-        *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
         fence_mbar_init();
     }
     if (warp == kIssueWarp) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+    grid_dep_launch();
+    grid_dep_wait();
+    if (threadIdx.x == 0) *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -501,10 +505,12 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kBars; ++i) mbar_init(bar(i), (i == kSFree || i == kDsFull) ? kComputeWarps : 1);
-        *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
         fence_mbar_init();
     }
     if (warp == kIssueWarp) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+    grid_dep_launch();
+    grid_dep_wait();
+    if (threadIdx.x == 0) *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -689,18 +695,21 @@ cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, cudaSt
     if (e != cudaSuccess) return e;
     const long long warps = (long long)p.nq_total * p.heads;
     const unsigned dblocks = (unsigned)((warps * 32 + 255) / 256);
-    if (D == 128) bwd_delta_kernel<128><<<dblocks, 256, 0, stream>>>(p); else bwd_delta_kernel<64><<<dblocks, 256, 0, stream>>>(p);
+    e = D == 128 ? launch_dependent(true, bwd_delta_kernel<128>, dblocks, 256, 0, stream, p) : launch_dependent(true, bwd_delta_kernel<64>, dblocks, 256, 0, stream, p);
     count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
+    long long steps = 0;
+    for (int g = 0; g < p.n_groups; ++g) steps += (long long)p.heads * ((p.g[g].q_rows + kTile - 1) / kTile) * p.g[g].n_kt;
+    const bool early = steps <= kEarlySteps * 148;
     dim3 gq((unsigned)p.n_qtiles, (unsigned)p.heads), gk((unsigned)p.n_ktiles, (unsigned)p.heads);
-    if (D == 128) bwd_dq_kernel<128><<<gq, kBwdThreads, smem_dq, stream>>>(p, maps);
-    else          bwd_dq_kernel<64><<<gq, kBwdThreads, smem_dq, stream>>>(p, maps);
+    e = D == 128 ? launch_dependent(early, bwd_dq_kernel<128>, gq, kBwdThreads, smem_dq, stream, p, maps)
+                 : launch_dependent(early, bwd_dq_kernel<64>, gq, kBwdThreads, smem_dq, stream, p, maps);
     count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (D == 128) bwd_dkdv_kernel<128><<<gk, kDkdvThreads, smem_kv, stream>>>(p, maps);
-    else          bwd_dkdv_kernel<64><<<gk, kDkdvThreads, smem_kv, stream>>>(p, maps);
+    if (e != cudaSuccess) return e;
+    e = D == 128 ? launch_dependent(early, bwd_dkdv_kernel<128>, gk, kDkdvThreads, smem_kv, stream, p, maps)
+                 : launch_dependent(early, bwd_dkdv_kernel<64>, gk, kDkdvThreads, smem_kv, stream, p, maps);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace ll

@@ -371,6 +371,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
     const int cta = blockIdx.x;
 
     // ---- setup ------------------------------------------------------------------
+    grid_dep_launch();
     if (threadIdx.x == 0) {
         for (int i = 0; i < kNumBars; ++i) {
             uint32_t count = 1;
@@ -379,14 +380,15 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
             if (i == kQEmpty || i >= kKvEmpty) count = 2;                      // both MMA warps release Q and every K/V stage
             mbar_init(bar(i), count);
         }
-        // an earlier CTA already gave up on a wait: this one does not start (flag value 2)
-        *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
         fence_mbar_init();
     }
     if (warp == kTmaWarp) {
         tmem_alloc(smem_u32(tmem_slot), C::kTmemCols);
         tmem_relinquish();
     }
+    grid_dep_wait();
+    // an earlier CTA already gave up on a wait: this one does not start (flag value 2)
+    if (threadIdx.x == 0) *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -944,10 +946,13 @@ cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps 
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < kMaxDevices) prepared[dev][which].store(1, std::memory_order_release);
     }
-    if (which) attn_sm100_kernel<128><<<grid, kThreads, Cfg<128>::kSmemBytes, stream>>>(p, maps);
-    else       attn_sm100_kernel<64><<<grid, kThreads, Cfg<64>::kSmemBytes, stream>>>(p, maps);
+    long long steps = 0;
+    for (int g = 0; g < p.n_groups; ++g) steps += (long long)p.heads * p.g[g].tiles * p.g[g].n_kt;
+    const bool early = steps <= kEarlySteps * p.n_ctas;
+    e = which ? launch_dependent(early, attn_sm100_kernel<128>, grid, kThreads, Cfg<128>::kSmemBytes, stream, p, maps)
+              : launch_dependent(early, attn_sm100_kernel<64>, grid, kThreads, Cfg<64>::kSmemBytes, stream, p, maps);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace ll

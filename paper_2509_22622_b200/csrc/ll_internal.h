@@ -5,7 +5,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <string.h>
+
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "llattn.h"
@@ -187,7 +190,36 @@ struct BwdParams {
 struct BwdMaps { CUtensorMap q, d_out, k, v; };
 cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, cudaStream_t stream);
 
+// Launch on `stream` so that the kernel may start before the one in front of it has ended
+// (grid_dep_wait in ptx.cuh): the launch latency and the set-up of a kernel then run under its predecessor's
+// last blocks.  With `early` false it starts as usual, when its predecessor has ended.  That is for the
+// tensor-core kernels with long work: their blocks fill whole SMs, and when these come free one by one instead of
+// all at once the blocks of a head no longer start together, which costs more cycles (recache of the benchmark
+// layer 1.60 -> 1.63 M, backward of the 21-frame clip 14.85 -> 14.97 M) than the gap in front of them.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_dependent(bool early, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                    Args &&...args)
+{
+    cudaLaunchAttribute attr;
+    memset(&attr, 0, sizeof attr);
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();       // the caller reports it: it does not stay behind for others to find
+    return e;
+}
+
 // kernel launchers (each returns the cudaError of the launch)
+// Key steps per SM up to which a tensor-core attention launch starts early: 32 steps take about 50 us, a gap 1 us.
+constexpr long long kEarlySteps = 32;
 cudaError_t launch_rope_tables(float2 *t_tab, int64_t t_base, int n_t_frames, int n_t,
                                float2 *h_tab, int grid_h, float2 *w_tab, int grid_w, int n_hw,
                                float theta, bool do_t, bool do_hw, cudaStream_t stream);

@@ -21,6 +21,16 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
     return t;
 }
 
+// ---- programmatic dependent launch -------------------------------------------
+
+// Every kernel of the library is launched with launch_dependent (ll_internal.h): it may start while
+// the kernel before it in the stream is still running.  It calls grid_dep_launch() first thing, which lets the
+// kernel behind it do the same once all its blocks have started, and grid_dep_wait() before its
+// first access to global memory: that returns when the kernels before it have completed and their writes are
+// visible.  What can be done without memory (barriers, tensor memory, index arithmetic) comes before the wait.
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- mbarrier ---------------------------------------------------------------
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)

@@ -253,9 +253,9 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
     const uint32_t rank = cluster_rank();              // 0: the leader, whose barriers and issuer serve the pair
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
+    grid_dep_launch();
     if (threadIdx.x == 0) {
         for (int i = 0; i < G::kBars; ++i) mbar_init(bar(i), (i >= kAccEmpty) ? 2u * G::kEpiWarps : 1u);   // both CTAs' epilogue warps free a buffer
-        *abort_flag = (rank == 0 && *reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
         fence_mbar_init();
     }
     if (warp == 0) {
@@ -263,7 +263,10 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
+    grid_dep_wait();
+    if (threadIdx.x == 0) *abort_flag = (rank == 0 && *reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
     tc_fence_before_sync();
+    __syncwarp();
     cluster_sync();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
@@ -375,6 +378,8 @@ qkv_finish_kernel(const __grid_constant__ QkvParams p)
 {
     constexpr int kHeld = 6;
     const int token = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    grid_dep_launch();
+    grid_dep_wait();
     if (token >= p.n_tokens) return;
     const int HD = p.heads * p.head_dim, vecs = HD / 8, per_head = p.head_dim / 8;
     const int frame = token / p.P, cell = token - frame * p.P;
@@ -429,8 +434,7 @@ cudaError_t launch_qkv_gemm(const QkvParams &p, const CUtensorMap &xmap, const C
     if (p.head_dim == DD && p.tile_n == TT) {                                                                                  \
         e = cudaFuncSetAttribute(qkv_gemm_kernel<DD, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<TT>::kSmem);   \
         if (e != cudaSuccess) return e;                                                                                        \
-        qkv_gemm_kernel<DD, TT><<<grid, GemmCfg<TT>::kThreads, GemmCfg<TT>::kSmem, stream>>>(p, xmap, wmap);                            \
-        e = cudaGetLastError();                                                                                                \
+        e = launch_dependent(true, qkv_gemm_kernel<DD, TT>, grid, GemmCfg<TT>::kThreads, GemmCfg<TT>::kSmem, stream, p, xmap, wmap); \
     }
     LL_GEMM_CASE(128, 256)
     LL_GEMM_CASE(128, 192)
@@ -441,9 +445,9 @@ cudaError_t launch_qkv_gemm(const QkvParams &p, const CUtensorMap &xmap, const C
 #undef LL_GEMM_CASE
     count_launch();
     if (e != cudaSuccess || !p.with_norm) return e;
-    qkv_finish_kernel<<<(unsigned)((p.n_tokens + 7) / 8), 256, 0, stream>>>(p);
+    e = launch_dependent(true, qkv_finish_kernel, (unsigned)((p.n_tokens + 7) / 8), 256, 0, stream, p);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace ll

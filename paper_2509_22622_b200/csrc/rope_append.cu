@@ -10,6 +10,7 @@
 #include <cuda_bf16.h>
 
 #include "ll_internal.h"
+#include "ptx.cuh"
 #include "rope_math.cuh"
 
 namespace ll {
@@ -26,6 +27,8 @@ __global__ void rope_table_kernel(float2 *t_tab, long long t_base, int n_t_frame
                                   float2 *h_tab, int grid_h, float2 *w_tab, int grid_w, int n_hw,
                                   double theta, int do_t, int do_hw)
 {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int n_tt = do_t ? n_t_frames * n_t : 0;
     const int n_hh = do_hw ? grid_h * n_hw : 0;
     const int n_ww = do_hw ? grid_w * n_hw : 0;
@@ -62,6 +65,8 @@ __global__ void __launch_bounds__(kThreads)
 rope_append_kernel(const __grid_constant__ RopeAppendParams p)
 {
     constexpr int kVecs = D / 8;                       // 16-byte vectors per head row
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int head_groups = (p.heads + kHeadsPerThread - 1) / kHeadsPerThread;
     const long long gid = (long long)blockIdx.x * kThreads + threadIdx.x;
     const int vec = (int)(gid % kVecs);
@@ -131,6 +136,8 @@ __global__ void __launch_bounds__(kThreads)
 rope_append_e4m3_kernel(const __grid_constant__ RopeAppendParams p)
 {
     constexpr int kVecs = D / 8;
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int head_groups = (p.heads + kHeadsPerThread - 1) / kHeadsPerThread;
     const long long gid = (long long)blockIdx.x * kThreads + threadIdx.x;
     const int vec = (int)(gid % kVecs);
@@ -187,6 +194,8 @@ __global__ void __launch_bounds__(kThreads)
 stage_e4m3_kernel(const __grid_constant__ StageParams p)
 {
     constexpr int kVecs = D / 16;                      // 16-code vectors per row
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     long long gid = (long long)blockIdx.x * kThreads + threadIdx.x;
     const int vec = (int)(gid % kVecs);
     gid /= kVecs;
@@ -269,6 +278,8 @@ norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float 
     constexpr int kVecs = D / 8;                       // 16-byte vectors per head row
     static_assert(32 % kVecs == 0, "a lane must meet the same rotation pairs in all its vectors");
     constexpr int kHeld = kIters > 0 ? kIters : 1;
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int lane = threadIdx.x & 31;
     const long long token = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     if (token >= p.n_tokens) return;
@@ -351,14 +362,14 @@ norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float 
 }
 
 template <int D>
-void launch_norm_variant(const RopeAppendParams &p, const float *gain_q, const float *gain_k, float eps,
+cudaError_t launch_norm_variant(const RopeAppendParams &p, const float *gain_q, const float *gain_k, float eps,
                          unsigned blocks, cudaStream_t stream)
 {
     const int iters = (p.heads * (D / 8) + 31) / 32;
-    if (iters <= 2)      norm_rope_append_kernel<D, 2><<<blocks, kThreads, 0, stream>>>(p, gain_q, gain_k, eps);
-    else if (iters <= 4) norm_rope_append_kernel<D, 4><<<blocks, kThreads, 0, stream>>>(p, gain_q, gain_k, eps);
-    else if (iters <= 6) norm_rope_append_kernel<D, 6><<<blocks, kThreads, 0, stream>>>(p, gain_q, gain_k, eps);
-    else                 norm_rope_append_kernel<D, 0><<<blocks, kThreads, 0, stream>>>(p, gain_q, gain_k, eps);
+    if (iters <= 2) return launch_dependent(true, norm_rope_append_kernel<D, 2>, blocks, kThreads, 0, stream, p, gain_q, gain_k, eps);
+    if (iters <= 4) return launch_dependent(true, norm_rope_append_kernel<D, 4>, blocks, kThreads, 0, stream, p, gain_q, gain_k, eps);
+    if (iters <= 6) return launch_dependent(true, norm_rope_append_kernel<D, 6>, blocks, kThreads, 0, stream, p, gain_q, gain_k, eps);
+    return launch_dependent(true, norm_rope_append_kernel<D, 0>, blocks, kThreads, 0, stream, p, gain_q, gain_k, eps);
 }
 
 }  // namespace
@@ -368,10 +379,10 @@ cudaError_t launch_norm_rope_append(const RopeAppendParams &p, int head_dim, con
 {
     const unsigned blocks = (unsigned)((p.n_tokens + kThreads / 32 - 1) / (kThreads / 32));
     if (blocks == 0) return cudaSuccess;
-    if (head_dim == 128) launch_norm_variant<128>(p, gain_q, gain_k, eps, blocks, stream);
-    else                 launch_norm_variant<64>(p, gain_q, gain_k, eps, blocks, stream);
+    const cudaError_t e = head_dim == 128 ? launch_norm_variant<128>(p, gain_q, gain_k, eps, blocks, stream)
+                                          : launch_norm_variant<64>(p, gain_q, gain_k, eps, blocks, stream);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_rope_tables(float2 *t_tab, int64_t t_base, int n_t_frames, int n_t, float2 *h_tab,
@@ -381,10 +392,10 @@ cudaError_t launch_rope_tables(float2 *t_tab, int64_t t_base, int n_t_frames, in
     int total = (do_t ? n_t_frames * n_t : 0) + (do_hw ? (grid_h + grid_w) * n_hw : 0);
     if (total == 0) return cudaSuccess;
     int blocks = (total + 127) / 128;
-    rope_table_kernel<<<blocks, 128, 0, stream>>>(t_tab, (long long)t_base, n_t_frames, n_t, h_tab, grid_h,
-                                                  w_tab, grid_w, n_hw, (double)theta, do_t, do_hw);
+    const cudaError_t e = launch_dependent(true, rope_table_kernel, blocks, 128, 0, stream, t_tab, (long long)t_base, n_t_frames, n_t, h_tab,
+                                           grid_h, w_tab, grid_w, n_hw, (double)theta, (int)do_t, (int)do_hw);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_rope_append_e4m3(const RopeAppendParams &p, int head_dim, cudaStream_t stream)
@@ -393,10 +404,10 @@ cudaError_t launch_rope_append_e4m3(const RopeAppendParams &p, int head_dim, cud
     const long long threads = (long long)p.n_tokens * head_groups * (head_dim / 8);
     const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
     if (blocks == 0) return cudaSuccess;
-    if (head_dim == 128) rope_append_e4m3_kernel<128><<<blocks, kThreads, 0, stream>>>(p);
-    else                 rope_append_e4m3_kernel<64><<<blocks, kThreads, 0, stream>>>(p);
+    const cudaError_t e = head_dim == 128 ? launch_dependent(true, rope_append_e4m3_kernel<128>, blocks, kThreads, 0, stream, p)
+                                          : launch_dependent(true, rope_append_e4m3_kernel<64>, blocks, kThreads, 0, stream, p);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_stage_e4m3(const StageParams &p, int head_dim, cudaStream_t stream)
@@ -406,10 +417,10 @@ cudaError_t launch_stage_e4m3(const StageParams &p, int head_dim, cudaStream_t s
     const long long threads = rows * (head_dim / 16);
     const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
     if (blocks == 0) return cudaSuccess;
-    if (head_dim == 128) stage_e4m3_kernel<128><<<blocks, kThreads, 0, stream>>>(p);
-    else                 stage_e4m3_kernel<64><<<blocks, kThreads, 0, stream>>>(p);
+    const cudaError_t e = head_dim == 128 ? launch_dependent(true, stage_e4m3_kernel<128>, blocks, kThreads, 0, stream, p)
+                                          : launch_dependent(true, stage_e4m3_kernel<64>, blocks, kThreads, 0, stream, p);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_rope_append(const RopeAppendParams &p, int head_dim, cudaStream_t stream)
@@ -418,10 +429,10 @@ cudaError_t launch_rope_append(const RopeAppendParams &p, int head_dim, cudaStre
     const long long threads = (long long)p.n_tokens * head_groups * (head_dim / 8);
     const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
     if (blocks == 0) return cudaSuccess;
-    if (head_dim == 128) rope_append_kernel<128><<<blocks, kThreads, 0, stream>>>(p);
-    else                 rope_append_kernel<64><<<blocks, kThreads, 0, stream>>>(p);
+    const cudaError_t e = head_dim == 128 ? launch_dependent(true, rope_append_kernel<128>, blocks, kThreads, 0, stream, p)
+                                          : launch_dependent(true, rope_append_kernel<64>, blocks, kThreads, 0, stream, p);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace ll
