@@ -279,6 +279,54 @@ struct AttnCall {
     const float *q_scale;                         // per-row factor on the queries, or null
 };
 
+// Fewer columns than CTAs, all equally long: every column in the same number of equal parts, one part per
+// CTA, when that is the cheapest way.  In steps, a part costs its own length; splitting at all costs the trip of
+// the parts through the scratch slots (kSplitSteps) and the merge, which loads four parts at a time
+// (kMergeSteps each).  Against levelled shares it saves a CTA's second column segment
+// (kSegmentSteps: its first loads and its drain) and a part per column.  Over 40 drawn launches of
+// up to 100 GF the split by these costs takes 0.926 of the time of levelled shares (geometric mean; 95 x 662, 40
+// heads of 128: 19.5 -> 12.8 us); with (kSplitSteps, kMergeSteps) of (1, 0.75) or (2.5, 1.5) shapes of 10 to 20
+// steps are split that are faster whole.  The benchmark layer's preview grid (17 x 29): 76 -> 71 us.
+bool even_split(ll::AttnParams *p, int sms, long long all_cols)
+{
+    constexpr double kSplitSteps = 2.5, kMergeSteps = 2.5, kSegmentSteps = 2;
+    if (all_cols >= sms || all_cols <= 0) return false;
+    const long long n_kt = p->g[0].n_kt;
+    for (int g = 1; g < p->n_groups; ++g)
+        if (p->g[g].n_kt != n_kt) return false;
+    auto merge = [&](long long parts) { return parts > 1 ? kSplitSteps + kMergeSteps * ((parts + 3) / 4) : 0.; };
+    long long best = 1;
+    double cost = (double)n_kt;
+    for (long long k = 2; k <= std::min<long long>(sms / all_cols, n_kt); ++k) {
+        const double c = (double)((n_kt + k - 1) / k) + merge(k);
+        if (c < cost) { cost = c; best = k; }
+    }
+    const double share = (double)((all_cols * n_kt + sms - 1) / sms);
+    if (cost > share + kSegmentSteps + merge((long long)((double)n_kt / share) + 2)) return false;
+    p->n_ctas = (int)(all_cols * best);
+    p->n_shares = 0;
+    p->share_begin[0] = 0;
+    for (int i = 0; i < p->n_ctas; ++i) p->share_of_cta[i] = -1;
+    const bool whole = best == 1;
+    p->n_waves = whole ? 1 : 0;
+    long long steps = 0;
+    for (int g = 0; g < p->n_groups; ++g) {
+        ll::AttnGroup &G = p->g[g];
+        const long long cols = (long long)p->heads * G.tiles;
+        G.wave_cols = whole ? (int)cols : 0;
+        G.step_begin = steps;
+        if (!whole) steps += cols * n_kt;
+    }
+    p->total_steps = steps;
+    if (whole) return true;
+    for (long long col = 0; col < all_cols; ++col)
+        for (long long i = 1; i <= best; ++i) {
+            p->share_of_cta[p->n_shares] = (short)p->n_shares;
+            p->share_begin[++p->n_shares] = (int)(col * n_kt + i * n_kt / best);
+        }
+    return true;
+}
+
 // Divide the columns of all groups between the CTAs (one persistent CTA per SM).  The
 // columns are numbered through, group after group.  While a CTA's worth of them is
 // left they go out whole, one per CTA and wave (CTAs on the same head then walk the keys
@@ -291,11 +339,14 @@ void plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_ste
     p->n_ctas = waves ? sms : (int)std::min<long long>(sms, all_steps);
     p->n_waves = waves ? (int)(all_cols / sms) : 0;
     p->all_cols = (int)all_cols;
+    if (even_split(p, sms, all_cols)) return;
     {
         // Short columns: splitting the leftover columns saves at most their length minus an even
-        // share, and costs every part a trip through the scratch slots (about kMergeSteps steps'
-        // worth).  When that does not pay, the leftover goes out whole as one more, partial wave.
-        constexpr long long kMergeSteps = 3;
+        // share, and costs every part a trip through the scratch slots and most CTAs a second
+        // segment (about kMergeSteps steps' worth: 6163 x 826 queries and keys, 6 heads of 128, 39.1 us
+        // split at 3, 32.9 us whole at 6; 9 made a launch of six streams 9 % slower).  When that does not
+        // pay, the leftover goes out whole as one more, partial wave.
+        constexpr long long kMergeSteps = 6;
         const long long first_left = (long long)p->n_waves * sms;
         long long left_steps = 0, left_longest = 0;
         for (int g = 0; g < p->n_groups; ++g) {

@@ -225,3 +225,26 @@ def test_closed_form_histogram_of_eight_streams_in_one_launch():
         guard()
         assert_histogram(item[4], want)
         cache.close()
+
+
+@pytest.mark.parametrize("heads,dim,n_q,n_k", [(2, 128, 300, 1500),       # 4 columns of 12 steps, four or more parts each
+                                               (40, 128, 95, 662),        # 40 columns of 6 steps: whole
+                                               (1, 64, 129, 128 * 40),    # 1 column of 40 steps, many parts (batches of the merge)
+                                               (12, 128, 1479, 47 * 128 - 100),   # two equal parts per column, one odd
+                                               (5, 64, 2000, 700)])
+def test_columns_in_equal_parts(heads, dim, n_q, n_k):
+    """Fewer columns than SMs: every column in the same number of parts (or whole), against plain torch in 64 bits."""
+    gen = torch.Generator(device="cuda").manual_seed(n_q)
+    q, k, v = (torch.randn(n, heads, dim, device="cuda", generator=gen).to(torch.bfloat16) for n in (n_q, n_k, n_k))
+    cache = B.Cache(1, heads, dim, 16, 1, 1, 1)
+    out, guard = guarded((n_q, heads, dim), fill=float("nan"))
+    lse = torch.full((heads, n_q), float("nan"), device="cuda")
+    for _ in range(2):                               # the second launch finds the first one's scratch and counters
+        cache.cross_attn(q, k, v, out, lse)
+    cache.check_device()
+    guard()
+    s = torch.einsum("qhd,khd->hqk", q.double(), k.double()) * dim ** -0.5
+    want = torch.einsum("hqk,khd->qhd", s.softmax(-1), v.double()).cpu().numpy()
+    check_attn(f64(out), want)
+    assert (lse.double() - s.logsumexp(-1)).abs().max().item() <= 1e-4
+    cache.close()
