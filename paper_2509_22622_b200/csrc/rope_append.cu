@@ -121,14 +121,31 @@ rope_append_kernel(const __grid_constant__ RopeAppendParams p)
 
 // ---- the same into an 8-bit cache ---------------------------------------------------------
 //
-// K (rotated, fp32) and V are divided by their head's scale (IEEE division) and rounded to
+// K (rotated, fp32) and V are divided by their head's scale (the correctly rounded quotient) and rounded to
 // E4M3, round to nearest even, saturating; a thread's eight elements make one 8-byte store, 16
 // consecutive threads cover a 128-byte cache row.  Q is rotated to bf16 as in the bf16 kernel.
-__device__ __forceinline__ uint2 quantise_vec(const float (&x)[8], float scale)
+//   The quotient comes from the correctly rounded reciprocal r of the scale by Markstein's correction
+// (P. Markstein, IBM J. Res. Dev. 34, 1990): q = x r, then q + (x - q s) r with fused operations is x / s
+// correctly rounded, as long as nothing leaves the exponent range.  Scales in [2^-60, 2^60] keep it
+// inside for every quotient that is not rounded to zero or saturated anyway; other scales divide.  With the
+// division for every element and each head's loads behind the stores of the one before: 20.9 us, now 16.9 us for 4680
+// tokens of 12 heads of 128 (72 MB, 11 us at the copy rate).
+__device__ __forceinline__ uint2 quantise_vec(const float (&x)[8], float scale, float recip)
 {
     uint32_t c[4];
+    if (scale >= 0x1p-60f && scale <= 0x1p60f) {
+        float q[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) c[u] = cvt_e4m3x2(__fdiv_rn(x[2 * u], scale), __fdiv_rn(x[2 * u + 1], scale));
+        for (int u = 0; u < 8; ++u) {
+            const float q0 = x[u] * recip, q1 = fmaf(fmaf(-q0, scale, x[u]), recip, q0);
+            q[u] = fabsf(q0) < 1024.f && q0 != 0.f ? q1 : q0;   // else saturated, infinite, NaN, or a zero with its sign
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = cvt_e4m3x2(q[2 * u], q[2 * u + 1]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = cvt_e4m3x2(__fdiv_rn(x[2 * u], scale), __fdiv_rn(x[2 * u + 1], scale));
+    }
     return make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
 }
 
@@ -138,7 +155,6 @@ rope_append_e4m3_kernel(const __grid_constant__ RopeAppendParams p)
 {
     constexpr int kVecs = D / 8;
     ptx::grid_dep_launch();
-    ptx::grid_dep_wait();
     const int head_groups = (p.heads + kHeadsPerThread - 1) / kHeadsPerThread;
     const long long gid = (long long)blockIdx.x * kThreads + threadIdx.x;
     const int vec = (int)(gid % kVecs);
@@ -150,9 +166,25 @@ rope_append_e4m3_kernel(const __grid_constant__ RopeAppendParams p)
     const int frame = (int)(token / p.P);
     const int cell = (int)(token % p.P);
     const int y = cell / p.grid_w, x = cell % p.grid_w;
+    const int h0 = hg * kHeadsPerThread;
+    const size_t in_base = ((size_t)token * p.heads + h0) * D + (size_t)vec * 8;
+    ptx::grid_dep_wait();
     if ((unsigned)p.slot[frame] >= (unsigned)p.n_slots) {         // never with the host's slot rule: refuse, report
         record_status(p.status, kStatusBadRow, (uint32_t)p.slot[frame], (uint32_t)frame);
         return;
+    }
+    // everything a thread reads goes out at once
+    uint4 kq[kHeadsPerThread], kk[kHeadsPerThread], kv[kHeadsPerThread];
+    float ks[kHeadsPerThread], vs[kHeadsPerThread];
+#pragma unroll
+    for (int u = 0; u < kHeadsPerThread; ++u) {
+        if (h0 + u < p.heads) {
+            kk[u] = ld16(p.k + in_base + (size_t)u * D);
+            kv[u] = ld16(p.v + in_base + (size_t)u * D);
+            if (p.q_out) kq[u] = ld16(p.q + in_base + (size_t)u * D);
+            ks[u] = __ldg(p.k_scale + h0 + u);
+            vs[u] = __ldg(p.v_scale + h0 + u);
+        }
     }
     float2 cs[4];
 #pragma unroll
@@ -164,16 +196,12 @@ rope_append_e4m3_kernel(const __grid_constant__ RopeAppendParams p)
         else                        src = p.w_tab + (size_t)x * p.n_h + (j - p.n_t - p.n_h);
         cs[u] = __ldg(src);
     }
-    const int h0 = hg * kHeadsPerThread;
-    const size_t in_base = ((size_t)token * p.heads + h0) * D + (size_t)vec * 8;
     const size_t cache_row = (size_t)p.slot[frame] * p.P + cell;
     uint8_t *kc = static_cast<uint8_t *>(p.kcache), *vc = static_cast<uint8_t *>(p.vcache);
 #pragma unroll
     for (int u = 0; u < kHeadsPerThread; ++u) {
         if (h0 + u >= p.heads) break;
-        const uint4 k = ld16(p.k + in_base + (size_t)u * D);
-        const uint4 v = ld16(p.v + in_base + (size_t)u * D);
-        const uint32_t kw[4] = {k.x, k.y, k.z, k.w}, vw[4] = {v.x, v.y, v.z, v.w};
+        const uint32_t kw[4] = {kk[u].x, kk[u].y, kk[u].z, kk[u].w}, vw[4] = {kv[u].x, kv[u].y, kv[u].z, kv[u].w};
         float kr[8], vr[8];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -182,9 +210,9 @@ rope_append_e4m3_kernel(const __grid_constant__ RopeAppendParams p)
             vr[2 * t + 1] = __uint_as_float(vw[t] & 0xffff0000u);
         }
         const size_t dst = (((size_t)(h0 + u)) * p.rows_per_head + cache_row) * D + (size_t)vec * 8;
-        *reinterpret_cast<uint2 *>(kc + dst) = quantise_vec(kr, __ldg(p.k_scale + h0 + u));
-        *reinterpret_cast<uint2 *>(vc + dst) = quantise_vec(vr, __ldg(p.v_scale + h0 + u));
-        if (p.q_out) st16(p.q_out + in_base + (size_t)u * D, rotate_vec(ld16(p.q + in_base + (size_t)u * D), cs));
+        *reinterpret_cast<uint2 *>(kc + dst) = quantise_vec(kr, ks[u], __frcp_rn(ks[u]));
+        *reinterpret_cast<uint2 *>(vc + dst) = quantise_vec(vr, vs[u], __frcp_rn(vs[u]));
+        if (p.q_out) st16(p.q_out + in_base + (size_t)u * D, rotate_vec(kq[u], cs));
     }
 }
 
