@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const __grid_constant__ 
     for (int r = 0; r < kRows; ++r) {
         const bool live = row0 + r < p.nq_total;
         const size_t off = ((size_t)(row0 + r) * p.heads + head) * D + 8 * lane;
-        a[r] = live ? __ldg(reinterpret_cast<const uint4 *>(p.out + off)) : make_uint4(0u, 0u, 0u, 0u);
-        b[r] = live ? __ldg(reinterpret_cast<const uint4 *>(p.d_out + off)) : make_uint4(0u, 0u, 0u, 0u);
+        a[r] = live ? *reinterpret_cast<const uint4 *>(p.out + off) : make_uint4(0u, 0u, 0u, 0u);
+        b[r] = live ? *reinterpret_cast<const uint4 *>(p.d_out + off) : make_uint4(0u, 0u, 0u, 0u);
     }
     float mine = 0.f;
 #pragma unroll
@@ -110,7 +110,7 @@ __device__ __forceinline__ void store_grad_row(uint32_t taddr, float mul, ll_bf1
             float a = as_f(r[2 * i]) * mul, b = as_f(r[2 * i + 1]) * mul;
             if (kRotateBack) {
                 const int j = 16 * ch + i;
-                const float2 cs = j < kNt ? __ldg(t_row + j) : j < kNt + kNh ? __ldg(h_row + (j - kNt)) : __ldg(w_row + (j - kNt - kNh));
+                const float2 cs = j < kNt ? t_row[j] : j < kNt + kNh ? h_row[j - kNt] : w_row[j - kNt - kNh];
                 const float a2 = fmaf(a, cs.x, b * cs.y), b2 = fmaf(b, cs.x, -(a * cs.y));
                 a = a2;
                 b = b2;
@@ -296,7 +296,7 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
             uint32_t w[32];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const uint4 u = live ? __ldg(src + 8 * c + i) : make_uint4(0u, 0u, 0u, 0u);
+                const uint4 u = live ? src[8 * c + i] : make_uint4(0u, 0u, 0u, 0u);
                 w[4 * i] = u.x; w[4 * i + 1] = u.y; w[4 * i + 2] = u.z; w[4 * i + 3] = u.w;
             }
             tmem_st_32x32b_x32(dst + 32 * c, w);

@@ -300,7 +300,7 @@ __device__ __forceinline__ void merge_column(const AttnParams &p, const Segment 
             l_b = fmaf(pb[u].y, ex2(pb[u].x - m_b), l_b);
         }
     }
-    const float v_scale = item.v_scale ? __ldg(item.v_scale + s.head) : 1.f;   // 8-bit caches: value codes x scale
+    const float v_scale = item.v_scale ? item.v_scale[s.head] : 1.f;   // 8-bit caches: value codes x scale
     const float inv_a = v_scale / l_a, inv_b = v_scale / l_b;
 #pragma unroll 1
     for (int ch = 0; ch < D / 64; ++ch) {
@@ -589,14 +589,14 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 }
                 // log2(e)/sqrt(D), times the head's key scale when the cache holds 8-bit codes
                 const float *k_scale = p.item[G.item].k_scale;
-                const float c = k_scale ? p.scale_log2 * __ldg(k_scale + s.head) : p.scale_log2;
+                const float c = k_scale ? p.scale_log2 * k_scale[s.head] : p.scale_log2;
                 // ... and times the query row's own factor when the caller brings one (a q/k norm whose
                 // per-token factor was left out of the stored q)
                 float c_a = c, c_b = c;
                 if (const float *q_scale = p.item[G.item].q_scale) {
                     const int r = 128 * w + wr.row_a();
-                    if (r < s.rows_valid) c_a *= __ldg(q_scale + s.q0 + r);
-                    if (r + 8 < s.rows_valid) c_b *= __ldg(q_scale + s.q0 + r + 8);
+                    if (r < s.rows_valid) c_a *= q_scale[s.q0 + r];
+                    if (r + 8 < s.rows_valid) c_b *= q_scale[s.q0 + r + 8];
                 }
                 float m_a = -INFINITY, m_b = -INFINITY;
                 uint64_t acc_a = 0ull, acc_b = 0ull;       // two partial sums per row
@@ -806,7 +806,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 const AttnItem &item = p.item[G.item];
                 if (s.kt0 == 0 && s.kt1 == G.n_kt) {
                     // a whole column: normalise and store
-                    const float v_scale = item.v_scale ? __ldg(item.v_scale + s.head) : 1.f;   // 8-bit caches: value codes x scale
+                    const float v_scale = item.v_scale ? item.v_scale[s.head] : 1.f;   // 8-bit caches: value codes x scale
                     const float inv_a = v_scale / l_a, inv_b = v_scale / l_b;
 #pragma unroll 1
                     for (int ch = 0; ch < C::kOChunks; ++ch) {

@@ -23,11 +23,15 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 
 // ---- programmatic dependent launch -------------------------------------------
 
-// Every kernel of the library is launched with launch_dependent (ll_internal.h): it may start while
-// the kernel before it in the stream is still running.  It calls grid_dep_launch() first thing, which lets the
-// kernel behind it do the same once all its blocks have started, and grid_dep_wait() before its
-// first access to global memory: that returns when the kernels before it have completed and their writes are
-// visible.  What can be done without memory (barriers, tensor memory, index arithmetic) comes before the wait.
+// A kernel launched with launch_dependent (ll_internal.h) may start while the kernel before it in the stream
+// is still running.  It calls grid_dep_launch() early, which lets the kernel behind it do the same once all its
+// blocks have started, and grid_dep_wait() before its first access to global memory: that returns when the
+// kernels before it have completed and their writes are visible.  What can be done without memory (barriers,
+// tensor memory, index arithmetic) comes before the wait.  rope_q_static_kernel, attn_simt_kernel and
+// wait_probe_kernel have neither call and are launched the ordinary way.
+//   What such a kernel reads behind the wait may have been written during its own lifetime, so it is read with
+// ordinary loads: ld.global.nc (__ldg, or what the compiler makes of a const __restrict__ pointer) is for
+// memory that nobody writes while the kernel lives, and the wait promises nothing for it.
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -142,7 +142,7 @@ struct EpiRow {
     }
     // (cos, sin) of rotation pair j of a head row
     template <int kNt, int kNh>
-    __device__ float2 turn(int j) const { return __ldg(j < kNt ? t_row + j : j < kNt + kNh ? h_row + (j - kNt) : w_row + (j - kNt - kNh)); }
+    __device__ float2 turn(int j) const { return *(j < kNt ? t_row + j : j < kNt + kNh ? h_row + (j - kNt) : w_row + (j - kNt - kNh)); }
 };
 
 // A warp's 16 rows x COLS features of the accumulator tile, 32 features at a time: bias, sum of squares,
@@ -180,8 +180,8 @@ __device__ __forceinline__ float2 epilogue_rows(const QkvParams &p, uint32_t tad
         float2 bias[4], gg[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            bias[k] = p.bias ? __ldg(reinterpret_cast<const float2 *>(p.bias + n0 + 32 * ch + 8 * k + cq)) : make_float2(0.f, 0.f);
-            gg[k] = which < 2 && p.with_norm ? __ldg(reinterpret_cast<const float2 *>(gain + cw + 8 * k + cq)) : make_float2(1.f, 1.f);
+            bias[k] = p.bias ? *reinterpret_cast<const float2 *>(p.bias + n0 + 32 * ch + 8 * k + cq) : make_float2(0.f, 0.f);
+            gg[k] = which < 2 && p.with_norm ? *reinterpret_cast<const float2 *>(gain + cw + 8 * k + cq) : make_float2(1.f, 1.f);
         }
         tmem_wait_ld();
         float2 va[4], vb[4];

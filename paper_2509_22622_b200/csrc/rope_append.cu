@@ -92,7 +92,7 @@ rope_append_kernel(const __grid_constant__ RopeAppendParams p)
         if (j < p.n_t)             src = p.t_tab + (size_t)frame * p.n_t + j;
         else if (j < p.n_t + p.n_h) src = p.h_tab + (size_t)y * p.n_h + (j - p.n_t);
         else                        src = p.w_tab + (size_t)x * p.n_h + (j - p.n_t - p.n_h);
-        cs[u] = __ldg(src);
+        cs[u] = *src;
     }
 
     const int h0 = hg * kHeadsPerThread;
@@ -182,8 +182,8 @@ rope_append_e4m3_kernel(const __grid_constant__ RopeAppendParams p)
             kk[u] = ld16(p.k + in_base + (size_t)u * D);
             kv[u] = ld16(p.v + in_base + (size_t)u * D);
             if (p.q_out) kq[u] = ld16(p.q + in_base + (size_t)u * D);
-            ks[u] = __ldg(p.k_scale + h0 + u);
-            vs[u] = __ldg(p.v_scale + h0 + u);
+            ks[u] = p.k_scale[h0 + u];
+            vs[u] = p.v_scale[h0 + u];
         }
     }
     float2 cs[4];
@@ -194,7 +194,7 @@ rope_append_e4m3_kernel(const __grid_constant__ RopeAppendParams p)
         if (j < p.n_t)             src = p.t_tab + (size_t)frame * p.n_t + j;
         else if (j < p.n_t + p.n_h) src = p.h_tab + (size_t)y * p.n_h + (j - p.n_t);
         else                        src = p.w_tab + (size_t)x * p.n_h + (j - p.n_t - p.n_h);
-        cs[u] = __ldg(src);
+        cs[u] = *src;
     }
     const size_t cache_row = (size_t)p.slot[frame] * p.P + cell;
     uint8_t *kc = static_cast<uint8_t *>(p.kcache), *vc = static_cast<uint8_t *>(p.vcache);
@@ -304,8 +304,8 @@ __device__ __forceinline__ uint4 norm_rotate_vec(uint4 x, const float *gain, con
 // passes (one read of q, k, v from memory); kIters == 0: any row length, second pass re-reads.
 template <int D, int kIters>
 __global__ void __launch_bounds__(kNormThreads)
-norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float *__restrict__ gain_q,
-                        const float *__restrict__ gain_k, float eps)
+norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float *gain_q,
+                        const float *gain_k, float eps)
 {
     constexpr int kVecs = D / 8;                       // 16-byte vectors per head row
     static_assert(32 % kVecs == 0, "a lane must meet the same rotation pairs in all its vectors");
@@ -348,7 +348,7 @@ norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float 
         if (j < p.n_t)             src = p.t_tab + (size_t)frame * p.n_t + j;
         else if (j < p.n_t + p.n_h) src = p.h_tab + (size_t)y * p.n_h + (j - p.n_t);
         else                        src = p.w_tab + (size_t)x * p.n_h + (j - p.n_t - p.n_h);
-        cs[u] = __ldg(src);
+        cs[u] = *src;
     }
     const size_t cache_row = (size_t)p.slot[frame] * p.P + cell;
     auto cache_at = [&](int v) -> size_t { return ((size_t)(v / kVecs) * p.rows_per_head + cache_row) * D + (size_t)vec * 8; };
