@@ -711,7 +711,7 @@ cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, cudaSt
     // D / 8 threads per four rows of a head
     const long long threads = (long long)((p.nq_total + 3) / 4) * p.heads * (D / 8);
     const unsigned dblocks = (unsigned)((threads + 255) / 256);
-    e = D == 128 ? launch_dependent(true, bwd_delta_kernel<128>, dblocks, 256, 0, stream, p) : launch_dependent(true, bwd_delta_kernel<64>, dblocks, 256, 0, stream, p);
+    e = D == 128 ? launch_spread<&bwd_delta_kernel<128>>(dblocks, 256, stream, p) : launch_spread<&bwd_delta_kernel<64>>(dblocks, 256, stream, p);
     count_launch();
     if (e != cudaSuccess) return e;
     long long steps = 0;

@@ -605,6 +605,18 @@ int attn_entry(ll_cache *c, int layer, const ll_bf16 *q_roped, int64_t q_frame_s
 namespace ll {
 void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 void set_last_error(const char *msg) { g_err = msg; }
+
+cudaError_t query_residency(const void *kernel, int threads, Residency *r)
+{
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r->smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r->per_sm, kernel, threads, 0);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, r->smem / 2);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
 }  // namespace ll
 
 extern "C" {

@@ -7,6 +7,7 @@
 
 #include <string.h>
 
+#include <atomic>
 #include <string>
 #include <utility>
 #include <vector>
@@ -215,6 +216,52 @@ inline cudaError_t launch_dependent(bool early, void (*kernel)(Params...), dim3 
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
     if (e != cudaSuccess) (void)cudaGetLastError();       // the caller reports it: it does not stay behind for others to find
     return e;
+}
+
+// How many blocks of a kernel an SM holds, and what that follows from.
+struct Residency {
+    int sms, per_sm, smem;            // SMs; blocks per SM without dynamic shared memory; shared memory of an SM, bytes
+};
+cudaError_t query_residency(const void *kernel, int threads, Residency *r);
+
+// How a small kernel on a grid of `blocks` starts early.
+struct Spread { bool early; size_t smem; };
+inline Spread spread_of(long long blocks, const Residency &r)
+{
+    const long long need = (blocks + r.sms - 1) / r.sms;
+    if (need >= r.per_sm || (need > 4 && 4 * need >= 3 * r.per_sm)) return {true, 0};   // fills the chip, or nearly
+    if (need > 4) return {false, 0};
+    return {true, (size_t)(r.smem / (need + 1))};         // with what the system adds to each, need + 1 blocks do not fit
+}
+
+// launch_dependent for the kernels of small blocks.  Blocks of an early kernel go to the SMs in the order in which
+// these come free, as many as fit on each, and stay there until the wait is over: a grid that does not fill the chip then
+// sits on the few SMs that were free first.  So it is given as much (unused) shared memory as lets no more blocks
+// onto an SM than an even share.  That is for up to four blocks an SM; more lose more by it than they gain
+// (shared memory comes out of the L1 cache: norm append, 40 heads of 128, 4680 tokens, 8 of 9 blocks an SM, 65.6 us early,
+// 67.6 ordinary, 75.1 spread) and start the ordinary way unless they fill three quarters of the chip.
+//   Eight streams of 512 tokens, 12 heads of 128: 131 us a step with stacked blocks, 121 with ordinary starts, 107
+// spread; norm append of 40 heads, 918 tokens: 20.5 / 18.6 / 18.5 us, with its attention 151 / 128 / 128; projection with norm,
+// 40 heads, 512 tokens: 87 / 78 / 77.
+template <auto kKernel, typename... Args>
+inline cudaError_t launch_spread(unsigned blocks, unsigned threads, cudaStream_t stream, Args &&...args)
+{
+    constexpr int kMaxDevices = 64;
+    static std::atomic<const Residency *> known[kMaxDevices];      // asked for once per kernel and device
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    Residency fresh;
+    const Residency *r = dev < kMaxDevices ? known[dev].load(std::memory_order_acquire) : nullptr;
+    if (!r) {
+        if ((e = query_residency((const void *)kKernel, (int)threads, &fresh)) != cudaSuccess) return e;
+        r = &fresh;
+        const Residency *none = nullptr;
+        Residency *kept = dev < kMaxDevices ? new Residency(fresh) : nullptr;
+        if (kept && !known[dev].compare_exchange_strong(none, kept, std::memory_order_acq_rel)) delete kept;
+    }
+    const Spread s = spread_of(blocks, *r);
+    return launch_dependent(s.early, kKernel, blocks, threads, s.smem, stream, std::forward<Args>(args)...);
 }
 
 // kernel launchers (each returns the cudaError of the launch)

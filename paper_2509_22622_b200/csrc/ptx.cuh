@@ -23,7 +23,7 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 
 // ---- programmatic dependent launch -------------------------------------------
 
-// A kernel launched with launch_dependent (ll_internal.h) may start while the kernel before it in the stream
+// A kernel launched with launch_dependent or launch_spread (ll_internal.h) may start while the kernel before it in the stream
 // is still running.  It calls grid_dep_launch() early, which lets the kernel behind it do the same once all its
 // blocks have started, and grid_dep_wait() before its first access to global memory: that returns when the
 // kernels before it have completed and their writes are visible.  What can be done without memory (barriers,

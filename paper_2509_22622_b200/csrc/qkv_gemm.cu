@@ -445,7 +445,7 @@ cudaError_t launch_qkv_gemm(const QkvParams &p, const CUtensorMap &xmap, const C
 #undef LL_GEMM_CASE
     count_launch();
     if (e != cudaSuccess || !p.with_norm) return e;
-    e = launch_dependent(true, qkv_finish_kernel, (unsigned)((p.n_tokens + 7) / 8), 256, 0, stream, p);
+    e = launch_spread<&qkv_finish_kernel>((unsigned)((p.n_tokens + 7) / 8), 256, stream, p);
     count_launch();
     return e;
 }

@@ -415,10 +415,10 @@ cudaError_t launch_norm_variant(const RopeAppendParams &p, const float *gain_q, 
                          unsigned blocks, cudaStream_t stream)
 {
     const int iters = (p.heads * (D / 8) + 31) / 32;
-    if (iters <= 2) return launch_dependent(true, norm_rope_append_kernel<D, 2>, blocks, kNormThreads, 0, stream, p, gain_q, gain_k, eps);
-    if (iters <= 4) return launch_dependent(true, norm_rope_append_kernel<D, 4>, blocks, kNormThreads, 0, stream, p, gain_q, gain_k, eps);
-    if (iters <= 6) return launch_dependent(true, norm_rope_append_kernel<D, 6>, blocks, kNormThreads, 0, stream, p, gain_q, gain_k, eps);
-    return launch_dependent(true, norm_rope_append_kernel<D, 0>, blocks, kNormThreads, 0, stream, p, gain_q, gain_k, eps);
+    if (iters <= 2) return launch_spread<&norm_rope_append_kernel<D, 2>>(blocks, kNormThreads, stream, p, gain_q, gain_k, eps);
+    if (iters <= 4) return launch_spread<&norm_rope_append_kernel<D, 4>>(blocks, kNormThreads, stream, p, gain_q, gain_k, eps);
+    if (iters <= 6) return launch_spread<&norm_rope_append_kernel<D, 6>>(blocks, kNormThreads, stream, p, gain_q, gain_k, eps);
+    return launch_spread<&norm_rope_append_kernel<D, 0>>(blocks, kNormThreads, stream, p, gain_q, gain_k, eps);
 }
 
 }  // namespace
@@ -453,8 +453,8 @@ cudaError_t launch_rope_append_e4m3(const RopeAppendParams &p, int head_dim, cud
     const long long threads = (long long)p.n_tokens * head_groups * (head_dim / 8);
     const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
     if (blocks == 0) return cudaSuccess;
-    const cudaError_t e = head_dim == 128 ? launch_dependent(true, rope_append_e4m3_kernel<128>, blocks, kThreads, 0, stream, p)
-                                          : launch_dependent(true, rope_append_e4m3_kernel<64>, blocks, kThreads, 0, stream, p);
+    const cudaError_t e = head_dim == 128 ? launch_spread<&rope_append_e4m3_kernel<128>>(blocks, kThreads, stream, p)
+                                          : launch_spread<&rope_append_e4m3_kernel<64>>(blocks, kThreads, stream, p);
     count_launch();
     return e;
 }
@@ -466,8 +466,8 @@ cudaError_t launch_stage_e4m3(const StageParams &p, int head_dim, cudaStream_t s
     const long long threads = rows * (head_dim / 16);
     const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
     if (blocks == 0) return cudaSuccess;
-    const cudaError_t e = head_dim == 128 ? launch_dependent(true, stage_e4m3_kernel<128>, blocks, kThreads, 0, stream, p)
-                                          : launch_dependent(true, stage_e4m3_kernel<64>, blocks, kThreads, 0, stream, p);
+    const cudaError_t e = head_dim == 128 ? launch_spread<&stage_e4m3_kernel<128>>(blocks, kThreads, stream, p)
+                                          : launch_spread<&stage_e4m3_kernel<64>>(blocks, kThreads, stream, p);
     count_launch();
     return e;
 }
@@ -478,8 +478,8 @@ cudaError_t launch_rope_append(const RopeAppendParams &p, int head_dim, cudaStre
     const long long threads = (long long)p.n_tokens * head_groups * (head_dim / 8);
     const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
     if (blocks == 0) return cudaSuccess;
-    const cudaError_t e = head_dim == 128 ? launch_dependent(true, rope_append_kernel<128>, blocks, kThreads, 0, stream, p)
-                                          : launch_dependent(true, rope_append_kernel<64>, blocks, kThreads, 0, stream, p);
+    const cudaError_t e = head_dim == 128 ? launch_spread<&rope_append_kernel<128>>(blocks, kThreads, stream, p)
+                                          : launch_spread<&rope_append_kernel<64>>(blocks, kThreads, stream, p);
     count_launch();
     return e;
 }

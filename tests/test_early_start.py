@@ -34,7 +34,7 @@ def kernels(text):
 
 
 ALL = {name: (f, body) for f in FILES for name, body in kernels(source(f)).items()}
-EARLY = sorted({k for f in FILES for call in re.findall(r"launch_dependent\([^;]*;", source(f)) for k in re.findall(r"\w+_kernel\b", call)})
+EARLY = sorted({k for f in FILES for call in re.findall(r"launch_(?:dependent|spread)\b[^;]*;", source(f)) for k in re.findall(r"\w+_kernel\b", call)})
 
 
 def test_the_early_kernels_are_found():
