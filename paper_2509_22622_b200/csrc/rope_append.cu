@@ -264,11 +264,11 @@ stage_e4m3_kernel(const __grid_constant__ StageParams p)
 // (1536 elements at head_dim 128) stay in registers between the passes; longer ones are
 // read again (from L1/L2).  The row stride in vectors (32) is a multiple of the vectors per head (8 or
 // 16), so a lane meets the same four rotation pairs in every vector it owns; their (cos, sin) are fetched
-// with the row and take the row's factor with them.
-//   Bound by memory, with the warp's two dependent phases on top: v leaves before the row's factor is known,
-// blocks of four warps (instead of eight) free their registers sooner, and the rotation pairs take the factor, so
-// an element costs one multiply less.  4680 tokens of 1536: 22.8 -> 21.7 us a pass (86 MB, 13.2 us at the copy
-// rate).
+// with the row.
+//   Bound by memory, with the warp's two dependent phases on top: v leaves before the row's factor is known and
+// blocks of four warps (instead of eight) free their registers sooner.  4680 tokens of 1536: 22.8 -> 21.8 us a pass
+// (86 MB, 13.2 us at the copy rate); with the factor in the rotation pairs, one multiply less per element, it is
+// 21.7 us.
 __device__ __forceinline__ uint64_t widen(uint32_t packed)
 {
     return ptx::pack2(__uint_as_float(packed << 16), __uint_as_float(packed & 0xffff0000u));
@@ -285,19 +285,20 @@ __device__ __forceinline__ uint64_t add_squares(uint4 x, uint64_t acc)
     return acc;
 }
 
-// One packed pair times its gains, turned by cs (which carries the row's factor), in fp32, one rounding.
-__device__ __forceinline__ uint32_t norm_rotate_pair(uint32_t packed, float gx, float gy, float2 cs)
+// One packed pair times the row's factor (both halves of r), then its gains, turned by cs, in fp32, one rounding.  In
+// this order: the factor brings the elements to the order of 1, element times gain alone may leave the range.
+__device__ __forceinline__ uint32_t norm_rotate_pair(uint32_t packed, uint64_t r, float gx, float gy, float2 cs)
 {
     float a, b;
-    ptx::unpack2(ptx::mul2(widen(packed), ptx::pack2(gx, gy)), a, b);
+    ptx::unpack2(ptx::mul2(ptx::mul2(widen(packed), r), ptx::pack2(gx, gy)), a, b);
     return ptx::cvt_bf16x2(fmaf(a, cs.x, -(b * cs.y)), fmaf(a, cs.y, b * cs.x));
 }
 
-__device__ __forceinline__ uint4 norm_rotate_vec(uint4 x, const float *gain, const float2 (&cs)[4])
+__device__ __forceinline__ uint4 norm_rotate_vec(uint4 x, uint64_t r, const float *gain, const float2 (&cs)[4])
 {
     const float4 g0 = *reinterpret_cast<const float4 *>(gain), g1 = *reinterpret_cast<const float4 *>(gain + 4);
-    return make_uint4(norm_rotate_pair(x.x, g0.x, g0.y, cs[0]), norm_rotate_pair(x.y, g0.z, g0.w, cs[1]),
-                      norm_rotate_pair(x.z, g1.x, g1.y, cs[2]), norm_rotate_pair(x.w, g1.z, g1.w, cs[3]));
+    return make_uint4(norm_rotate_pair(x.x, r, g0.x, g0.y, cs[0]), norm_rotate_pair(x.y, r, g0.z, g0.w, cs[1]),
+                      norm_rotate_pair(x.z, r, g1.x, g1.y, cs[2]), norm_rotate_pair(x.w, r, g1.z, g1.w, cs[3]));
 }
 
 // kIters > 0: the row's vectors fit kIters per lane and stay in registers between the two
@@ -386,15 +387,10 @@ norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float 
     }
     const float inv_n = 1.f / (float)(row_vecs * 8);
     const float rq = 1.f / sqrtf(fmaf(sq, inv_n, eps)), rk = 1.f / sqrtf(fmaf(sk, inv_n, eps));
-    float2 cq[4], ck[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        cq[u] = make_float2(cs[u].x * rq, cs[u].y * rq);
-        ck[u] = make_float2(cs[u].x * rk, cs[u].y * rk);
-    }
+    const uint64_t rq2 = ptx::pack2(rq, rq), rk2 = ptx::pack2(rk, rk);
     auto emit = [&](int v, uint4 xq, uint4 xk) {
-        st16(static_cast<ll_bf16 *>(p.kcache) + cache_at(v), norm_rotate_vec(xk, gain_k + (size_t)v * 8, ck));
-        if (with_q) st16(p.q_out + in_base + (size_t)v * 8, norm_rotate_vec(xq, gain_q + (size_t)v * 8, cq));
+        st16(static_cast<ll_bf16 *>(p.kcache) + cache_at(v), norm_rotate_vec(xk, rk2, gain_k + (size_t)v * 8, cs));
+        if (with_q) st16(p.q_out + in_base + (size_t)v * 8, norm_rotate_vec(xq, rq2, gain_q + (size_t)v * 8, cs));
     };
     if (kIters > 0) {
 #pragma unroll
