@@ -194,28 +194,44 @@ cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, cudaSt
 // Launch on `stream` so that the kernel may start before the one in front of it has ended
 // (grid_dep_wait in ptx.cuh): the launch latency and the set-up of a kernel then run under its predecessor's
 // last blocks.  With `early` false it starts as usual, when its predecessor has ended.  That is for the
-// tensor-core kernels with long work: their blocks fill whole SMs, and when these come free one by one instead of
+// attention kernels with long work: their blocks fill whole SMs, and when these come free one by one instead of
 // all at once the blocks of a head no longer start together, which costs more cycles (recache of the benchmark
 // layer 1.60 -> 1.63 M, backward of the 21-frame clip 14.85 -> 14.97 M) than the gap in front of them.
+// The projection has no such order to lose and always starts early (40 heads of 128, 4680 tokens, 757 us; 759 with an
+// ordinary start).  `carveout`: percentage of an SM's shared memory and L1 cache that the kernel wants as shared
+// memory, -1 the driver's choice.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_dependent(bool early, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_dependent(bool early, int carveout, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                     Args &&...args)
 {
-    cudaLaunchAttribute attr;
-    memset(&attr, 0, sizeof attr);
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    memset(attr, 0, sizeof attr);
+    unsigned n = 0;
+    if (early) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (carveout >= 0) {
+        attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[n++].val.sharedMemCarveout = (unsigned)carveout;
+    }
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = early ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
     if (e != cudaSuccess) (void)cudaGetLastError();       // the caller reports it: it does not stay behind for others to find
     return e;
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_dependent(bool early, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args)
+{
+    return launch_dependent(early, -1, kernel, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 
 // How many blocks of a kernel an SM holds, and what that follows from.
@@ -224,14 +240,15 @@ struct Residency {
 };
 cudaError_t query_residency(const void *kernel, int threads, Residency *r);
 
-// How a small kernel on a grid of `blocks` starts early.
-struct Spread { bool early; size_t smem; };
+// How a small kernel on a grid of `blocks` starts: early or not, with how much (unused) shared memory.
+struct Spread { bool early; int smem, carveout; };
 inline Spread spread_of(long long blocks, const Residency &r)
 {
-    const long long need = (blocks + r.sms - 1) / r.sms;
-    if (need >= r.per_sm || (need > 4 && 4 * need >= 3 * r.per_sm)) return {true, 0};   // fills the chip, or nearly
-    if (need > 4) return {false, 0};
-    return {true, (size_t)(r.smem / (need + 1))};         // with what the system adds to each, need + 1 blocks do not fit
+    const int need = (int)((blocks + r.sms - 1) / r.sms);
+    if (need >= r.per_sm || (need > 4 && 4 * need >= 3 * r.per_sm)) return {true, 0, 0};   // fills the chip, or nearly
+    if (need > 4) return {false, 0, 0};
+    const int smem = r.smem / (need + 1), block = smem + 1152;     // with what the system adds (1 KB, rounding) need + 1 do not fit
+    return {true, smem, (int)((100ll * need * block + r.smem - 1) / r.smem)};
 }
 
 // launch_dependent for the kernels of small blocks.  Blocks of an early kernel go to the SMs in the order in which
@@ -243,6 +260,9 @@ inline Spread spread_of(long long blocks, const Residency &r)
 //   Eight streams of 512 tokens, 12 heads of 128: 131 us a step with stacked blocks, 121 with ordinary starts, 107
 // spread; norm append of 40 heads, 918 tokens: 20.5 / 18.6 / 18.5 us, with its attention 151 / 128 / 128; projection with norm,
 // 40 heads, 512 tokens: 87 / 78 / 77.
+//   The split between shared memory and L1 cache is asked for with the launch: an early block otherwise runs in the split that
+// its predecessor left, and behind attention (all shared memory) that is an L1 cache too small for the loads in flight.
+// Recache of 12 heads of 128, 9 frames of 638 tokens: 195.7 us, 187.3 with ordinary starts, 186.7 early with the split (191.2 before the early start).
 template <auto kKernel, typename... Args>
 inline cudaError_t launch_spread(unsigned blocks, unsigned threads, cudaStream_t stream, Args &&...args)
 {
@@ -261,7 +281,7 @@ inline cudaError_t launch_spread(unsigned blocks, unsigned threads, cudaStream_t
         if (kept && !known[dev].compare_exchange_strong(none, kept, std::memory_order_acq_rel)) delete kept;
     }
     const Spread s = spread_of(blocks, *r);
-    return launch_dependent(s.early, kKernel, blocks, threads, s.smem, stream, std::forward<Args>(args)...);
+    return launch_dependent(s.early, s.carveout, kKernel, blocks, threads, (size_t)s.smem, stream, std::forward<Args>(args)...);
 }
 
 // kernel launchers (each returns the cudaError of the launch)
