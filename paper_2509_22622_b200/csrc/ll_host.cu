@@ -340,60 +340,69 @@ void plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_ste
     p->n_waves = waves ? (int)(all_cols / sms) : 0;
     p->all_cols = (int)all_cols;
     if (even_split(p, sms, all_cols)) return;
-    {
-        // Short columns: splitting the leftover columns saves at most their length minus an even
-        // share, and costs every part a trip through the scratch slots and most CTAs a second
-        // segment (about kMergeSteps steps' worth: 6163 x 826 queries and keys, 6 heads of 128, 39.1 us
-        // split at 3, 32.9 us whole at 6; 9 made a launch of six streams 9 % slower).  When that does not
-        // pay, the leftover goes out whole as one more, partial wave.
-        constexpr long long kMergeSteps = 6;
-        const long long first_left = (long long)p->n_waves * sms;
-        long long left_steps = 0, left_longest = 0;
+    // What goes out whole and what is left of it, and the steps each CTA gets as whole columns
+    long long load[ll::kMaxCtas], steps = 0;
+    auto deal = [&]() {
+        const long long whole_cols = std::min<long long>((long long)p->n_waves * p->n_ctas, all_cols);
+        std::fill(load, load + ll::kMaxCtas, 0);
+        steps = 0;
         for (int g = 0; g < p->n_groups; ++g) {
-            const ll::AttnGroup &G = p->g[g];
+            ll::AttnGroup &G = p->g[g];
             const long long cols = (long long)p->heads * G.tiles;
-            const long long left = std::min(cols, std::max<long long>(0, G.col_begin + cols - first_left));
-            left_steps += left * G.n_kt;
-            if (left > 0) left_longest = std::max<long long>(left_longest, G.n_kt);
+            G.wave_cols = (int)std::min(cols, std::max<long long>(0, whole_cols - G.col_begin));
+            G.step_begin = steps;
+            steps += (cols - G.wave_cols) * G.n_kt;
+            // of the columns [0, x) CTA i takes those congruent to i: (x + n - 1 - i) / n of them
+            const long long lo = G.col_begin, hi = G.col_begin + G.wave_cols, n = p->n_ctas;
+            for (int i = 0; i < p->n_ctas; ++i)
+                load[i] += ((hi + n - 1 - i) / n - (lo + n - 1 - i) / n) * G.n_kt;
         }
-        if (left_steps > 0 && left_longest <= (left_steps + sms - 1) / sms + kMergeSteps) {
-            p->n_waves += 1;
-            p->n_ctas = (int)std::min<long long>(sms, all_cols);
-        }
-    }
-    const long long whole_cols = std::min<long long>((long long)p->n_waves * p->n_ctas, all_cols);
-    long long steps = 0;
-    for (int g = 0; g < p->n_groups; ++g) {
-        ll::AttnGroup &G = p->g[g];
-        const long long cols = (long long)p->heads * G.tiles;
-        G.wave_cols = (int)std::min(cols, std::max<long long>(0, whole_cols - G.col_begin));
-        G.step_begin = steps;
-        steps += (cols - G.wave_cols) * G.n_kt;
-    }
-    p->total_steps = steps;
-    // steps each CTA gets as whole columns
-    long long load[ll::kMaxCtas] = {};
-    for (int g = 0; g < p->n_groups && p->n_ctas > 0; ++g) {
-        // of the columns [0, x) CTA i takes those congruent to i: (x + n - 1 - i) / n of them
-        const ll::AttnGroup &G = p->g[g];
-        const long long lo = G.col_begin, hi = G.col_begin + G.wave_cols, n = p->n_ctas;
-        for (int i = 0; i < p->n_ctas; ++i)
-            load[i] += ((hi + n - 1 - i) / n - (lo + n - 1 - i) / n) * G.n_kt;
-    }
+    };
     // the highest level T that the shared steps can fill: sum over CTAs of max(0, T - load) <= steps
     auto fill = [&](long long T) {
         long long need = 0;
         for (int i = 0; i < p->n_ctas; ++i) need += std::max<long long>(0, T - load[i]);
         return need;
     };
-    long long lo = 0, hi = 0;
-    for (int i = 0; i < p->n_ctas; ++i) hi = std::max(hi, load[i]);
-    hi += steps + 1;                                     // fill(hi) > steps
-    while (hi - lo > 1) {
-        const long long mid = lo + (hi - lo) / 2;
-        if (fill(mid) <= steps) lo = mid; else hi = mid;
+    auto level = [&]() {
+        long long lo = 0, hi = *std::max_element(load, load + ll::kMaxCtas) + steps + 1;   // fill(hi) > steps
+        while (hi - lo > 1) {
+            const long long mid = lo + (hi - lo) / 2;
+            if (fill(mid) <= steps) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
+    deal();
+    if (steps > 0) {
+        // Short columns: splitting the leftover columns saves at most their length minus an even
+        // share, and costs every part a trip through the scratch slots and most CTAs a second
+        // segment (about kMergeSteps steps' worth: 6163 x 826 queries and keys, 6 heads of 128, 39.1 us
+        // split at 3, 32.9 us whole at 6).  When that does not pay, the leftover goes out whole as one more,
+        // partial wave - unless that wave would stand behind CTAs that the waves before gave more than the others:
+        // whole it ends with the longest of them, split with the longest of the waves before or, kSplitSteps above
+        // the level of the shares, with a CTA that merges.  (Streams of 19 and 7 steps, 40 heads of 798 queries: 163 us
+        // whole behind two columns of 19, 140 split.  Over the 37 of 60 drawn launches with unequal loads that the first
+        // condition lets through, 14 to 16 steps choose within 0.5 % of the faster way, 8 within 1.8 %.)
+        constexpr long long kMergeSteps = 6, kSplitSteps = 15;
+        const long long first_left = (long long)p->n_waves * p->n_ctas;
+        long long left_longest = 0, whole_top = 0;
+        for (int g = 0; g < p->n_groups; ++g) {
+            const ll::AttnGroup &G = p->g[g];
+            const long long end = G.col_begin + (long long)p->heads * G.tiles;
+            for (long long col = std::max<long long>(G.col_begin, first_left); col < end; ++col) {
+                left_longest = std::max<long long>(left_longest, G.n_kt);
+                whole_top = std::max(whole_top, load[col - first_left] + G.n_kt);
+            }
+        }
+        if (left_longest <= (steps + sms - 1) / sms + kMergeSteps &&
+            whole_top <= std::max(*std::max_element(load, load + ll::kMaxCtas), level() + kSplitSteps)) {
+            p->n_waves += 1;
+            p->n_ctas = (int)std::min<long long>(sms, all_cols);
+            deal();
+        }
     }
-    const long long T = lo;
+    p->total_steps = steps;
+    const long long T = level();
     long long extra = steps - fill(T);                   // fewer than the CTAs at or below T: one more step each
     int k = 0;
     p->share_begin[0] = 0;

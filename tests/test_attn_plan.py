@@ -203,3 +203,37 @@ def test_short_columns_are_not_split():
     check_plan(plan)
     B.ll_cache_destroy(h)
     B.ll_cache_destroy(small)
+
+
+@pytest.mark.parametrize("heads,P,C,S,W,chunks,parts", [
+    (1, 256, 1, 0, 16, 16, 8),           # one column of 32 steps
+    (12, 493, 3, 3, 9, 6, 2),            # 72 columns of 47 steps, two parts each on 144 CTAs
+    (4, 256, 1, 0, 6, 6, 4),             # 4 columns of 12 steps: the merge loads four parts at a time
+    (40, 95, 1, 0, 7, 7, 1),             # 40 columns of 6 steps: whole
+])
+def test_equal_columns_in_equal_parts(heads, P, C, S, W, chunks, parts):
+    """Fewer columns than SMs, all equally long: each in the same number of parts, one per CTA."""
+    h = make_cache(heads, P, C, S, W, chunks)
+    plan = B.ll_debug_attn_plan(h, sm_count=148)
+    cols, n_kt = plan.heads * plan.tiles[0], plan.n_kt[0]
+    assert plan.n_ctas == cols * parts
+    if parts == 1:
+        assert (plan.n_waves, plan.n_shares, plan.wave_cols[0]) == (1, 0, cols)
+    else:
+        assert plan.n_waves == 0 and plan.n_shares == cols * parts
+        assert list(plan.share_begin[:plan.n_shares + 1]) == [c * n_kt + i * n_kt // parts for c in range(cols) for i in range(parts)] + [cols * n_kt]
+    check_plan(plan)
+    B.ll_cache_destroy(h)
+
+
+def test_a_last_wave_does_not_stand_behind_longer_columns():
+    """Streams of 19 and 7 steps, 160 columns each: two waves, and the CTAs that took two of the long columns would end seven steps
+    after everybody else if the 24 columns left over went out whole behind them."""
+    handles = [make_cache(40, 399, 2, 0, 6, n) for n in (15, 1)]
+    plan = B.ll_debug_attn_plan_batched([(h, 0) for h in handles], sm_count=148)
+    assert [plan.n_kt[g] for g in range(2)] == [19, 7] and plan.all_cols == 320
+    assert plan.n_waves == 2 and plan.shared_steps == 24 * 7 and plan.n_shares > 0
+    assert all(plan.share_of_cta[i] < 0 for i in range(12))          # those with two long columns take no share
+    check_plan(plan)
+    for h in handles:
+        B.ll_cache_destroy(h)
