@@ -70,6 +70,11 @@ typedef struct ll_attn_plan {
 int ll_debug_attn_plan(ll_cache *cache, int layer, int recache, int sm_count, ll_attn_plan *out);
 int ll_debug_attn_plan_batched(const ll_attn_item *items, int n_items, int sm_count, ll_attn_plan *out);
 
+/* The division of ll_qkv_proj_append's GEMM for n_tokens tokens and q, k, v rows of `width` features on a GPU of
+ * sm_count SMs: features per tile (256, 192 or 128; a tile has 256 tokens and a pair of SMs) and how many tiles the
+ * busiest pair works through.  Host-only. */
+int ll_debug_qkv_tiles(int n_tokens, int width, int sm_count, int *tile_n, int *tiles_per_pair);
+
 /* Byte offsets, inside the bound storage, of the regions of the aux block that
  * the attention kernel and the bounded waits write: the status words and the
  * arrival counters of the split-column merge (Sec. 3.3's attention needs

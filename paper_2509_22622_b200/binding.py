@@ -136,6 +136,7 @@ SIGNATURES = {
     "ll_debug_wait_timeout": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p]),
     "ll_debug_attn_plan": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.POINTER(ll_attn_plan)]),
     "ll_debug_attn_plan_batched": (C.c_int, [C.POINTER(ll_attn_item), C.c_int, C.c_int, C.POINTER(ll_attn_plan)]),
+    "ll_debug_qkv_tiles": (C.c_int, [C.c_int] * 3 + [C.POINTER(C.c_int)] * 2),
     "ll_debug_aux_layout": (C.c_int, [C.c_void_p] + [C.POINTER(C.c_size_t)] * 4),
     "ll_debug_guard_layout": (C.c_int, [C.c_void_p] + [C.POINTER(C.c_size_t)] * 3),
     "ll_launch_count": (C.c_int64, []),
@@ -364,6 +365,13 @@ def ll_debug_attn_plan_batched(handles_and_layers, sm_count=0) -> ll_attn_plan:
     plan = ll_attn_plan()
     _check(lib().ll_debug_attn_plan_batched(arr, len(handles_and_layers), sm_count, C.byref(plan)))
     return plan
+
+
+def ll_debug_qkv_tiles(n_tokens, width, sm_count=0):
+    """(features per tile, tiles of the busiest pair of SMs) of the projection."""
+    v = [C.c_int() for _ in range(2)]
+    _check(lib().ll_debug_qkv_tiles(n_tokens, width, sm_count, *[C.byref(x) for x in v]))
+    return tuple(x.value for x in v)
 
 
 def ll_debug_aux_layout(h):

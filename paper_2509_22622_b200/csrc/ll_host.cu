@@ -279,6 +279,27 @@ struct AttnCall {
     const float *q_scale;                         // per-row factor on the queries, or null
 };
 
+// Tiles of the projection that the busiest of the SM pairs works through.
+long long qkv_rounds(int n_tokens, int width, int sm_count, int tile_n)
+{
+    const long long pairs = std::max(1, (sm_count > 0 ? sm_count : 148) / 2);
+    return ((n_tokens + 255) / 256 * (3ll * width / tile_n) + pairs - 1) / pairs;
+}
+
+// Features per tile of the projection: the width whose last round of tiles leaves the SM pairs less idle (wider on a
+// tie), of those that divide a q, k or v row; 0 if none does.
+int qkv_tile_width(int n_tokens, int width, int sm_count)
+{
+    int best = 0;
+    long long best_cost = 0;
+    for (int tn : {256, 192, 128}) {
+        if (width % tn) continue;
+        const long long cost = qkv_rounds(n_tokens, width, sm_count, tn) * tn;
+        if (!best || cost < best_cost) { best = tn; best_cost = cost; }
+    }
+    return best;
+}
+
 // Fewer columns than CTAs, all equally long: every column in the same number of equal parts, one part per
 // CTA, when that is the cheapest way.  In steps, a part costs its own length; splitting at all costs the trip of
 // the parts through the scratch slots (kSplitSteps) and the merge, which loads four parts at a time
@@ -904,18 +925,9 @@ int ll_qkv_proj_append(ll_cache *c, int layer, const ll_bf16 *x, int d_model, co
         memset(&p, 0, sizeof p);
         p.n_tokens = n_frames * c->P; p.d_model = d_model; p.heads = c->H; p.head_dim = c->D;
         p.m_tiles = (p.n_tokens + 255) / 256;
-        {
-            // tile width: the one whose last round of tiles leaves the SM pairs less idle (wider on a tie)
-            const int hd = c->H * c->D, pairs = std::max(1, (c->sm_count > 0 ? c->sm_count : 148) / 2);
-            long long best = -1;
-            for (int tn : {256, 192, 128}) {
-                if (hd % tn) continue;
-                const long long tiles = (long long)p.m_tiles * (3 * hd / tn), cost = (tiles + pairs - 1) / pairs * tn;
-                if (best < 0 || cost < best) { best = cost; p.tile_n = tn; }
-            }
-            p.n_tiles = 3 * hd / p.tile_n;
-            p.ssq_slots = p.tile_n == 128 ? hd / 128 : 2 * hd / p.tile_n;   // at most one per 96 features
-        }
+        p.tile_n = qkv_tile_width(p.n_tokens, c->H * c->D, c->sm_count);
+        p.n_tiles = 3 * c->H * c->D / p.tile_n;
+        p.ssq_slots = p.tile_n == 128 ? c->H * c->D / 128 : 2 * c->H * c->D / p.tile_n;   // at most one per 96 features
         p.P = c->P; p.grid_w = grid_w; p.n_t = rp.n_t; p.n_h = rp.n_h;
         p.with_norm = with_norm ? 1 : 0; p.eps = eps;
         p.bias = bias; p.gain_q = gain_q; p.gain_k = gain_k;
@@ -1306,6 +1318,16 @@ int ll_debug_wait_timeout(ll_cache *c, int limit_ms, ll_stream stream)
     cudaError_t e = ll::launch_wait_probe(reinterpret_cast<uint32_t *>(c->storage + c->off_status),
                                           (uint64_t)limit_ms * 1000000ull, (cudaStream_t)stream);
     return e == cudaSuccess ? LL_OK : cuda_fail(e, "wait probe kernel");
+}
+
+int ll_debug_qkv_tiles(int n_tokens, int width, int sm_count, int *tile_n, int *tiles_per_pair)
+{
+    if (n_tokens <= 0 || width <= 0 || !tile_n || !tiles_per_pair) return fail(LL_ERR_INVALID_ARG, "bad argument to ll_debug_qkv_tiles");
+    const int tn = qkv_tile_width(n_tokens, width, sm_count);
+    if (!tn) return fail(LL_ERR_UNSUPPORTED_SHAPE, "no tile width divides %d", width);
+    *tile_n = tn;
+    *tiles_per_pair = (int)qkv_rounds(n_tokens, width, sm_count, tn);
+    return LL_OK;
 }
 
 int ll_debug_aux_layout(const ll_cache *c, size_t *status_offset, size_t *status_bytes, size_t *counters_offset,

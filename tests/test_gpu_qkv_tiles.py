@@ -1,8 +1,9 @@
 """GPU parity of the fused projection at the edges of its tiles.
 
 A pair of CTAs works on 256 tokens x 256, 192 or 128 features.  The shapes here sit at the edges:
-one token, a last tile of one row, one CTA of the pair without rows, every tile width, more tiles than pairs
-(accumulator buffers reused), K blocks with a tail, heads of 64 and 128.  Reference: plain torch in 64 bits."""
+one token, a last tile of one row, one CTA of the pair without rows, every tile width at both head sizes, more tiles than
+pairs (accumulator buffers reused), K blocks with a tail, rows of one and of several sweeps of the norm's second kernel.  What
+a shape is there for - tile width, tiles of the busiest pair - is asked of the library.  Reference: plain torch in 64 bits."""
 import pytest
 import torch
 
@@ -10,14 +11,21 @@ from paper_2509_22622_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
 
-# heads, head_dim, grid_h, grid_w, d_model
+# heads, head_dim, grid_h, grid_w, d_model; tile width, tiles of the busiest pair
 SHAPES = [
-    (2, 128, 1, 1, 64),         # one token, one K block; width 256
-    (4, 64, 1, 129, 72),        # the second CTA holds one row; K tail of 8
-    (3, 64, 1, 255, 1544),      # width 192, last row missing
-    (3, 128, 1, 257, 128),      # width 384: the width on which the last round is fuller; a tile of one row
-    (2, 128, 79, 80, 136),      # 75 tiles of 256 would need a second round: tiles of 128
-    (12, 128, 10, 52, 384),     # several tiles per pair
+    (2, 128, 1, 1, 64, 128, 1),         # one token, one K block
+    (4, 64, 1, 129, 72, 128, 1),        # the second CTA holds one row; K tail of 8
+    (3, 64, 1, 255, 1544, 192, 1),      # last row missing
+    (3, 128, 1, 257, 128, 128, 1),      # a tile of one row
+    (2, 128, 79, 80, 136, 128, 3),      # 25 tiles of 256 tokens
+    (12, 128, 10, 52, 384, 192, 1),
+    (24, 64, 30, 156, 136, 256, 5),     # the widest tiles at head_dim 64, both accumulator buffers used again
+    (12, 128, 30, 156, 72, 256, 5),
+    (9, 64, 1, 4100, 72, 192, 3),       # both accumulator buffers used again at width 192
+    (3, 128, 100, 124, 64, 192, 4),
+    (12, 64, 79, 80, 64, 128, 7),
+    (40, 128, 1, 130, 200, 256, 1),     # 5120 features: four sweeps of the norm's second kernel
+    (64, 128, 1, 40, 64, 128, 3),       # 8192, the most that is accepted
 ]
 
 
@@ -27,9 +35,10 @@ def turn(x, cos, sin):
 
 
 @pytest.mark.parametrize("with_norm", [False, True], ids=["plain", "norm"])
-@pytest.mark.parametrize("heads,dim,gh,gw,d_model", SHAPES)
-def test_tile_edges(heads, dim, gh, gw, d_model, with_norm):
+@pytest.mark.parametrize("heads,dim,gh,gw,d_model,tile_n,per_pair", SHAPES)
+def test_tile_edges(heads, dim, gh, gw, d_model, tile_n, per_pair, with_norm):
     n, width = gh * gw, heads * dim
+    assert B.ll_debug_qkv_tiles(n, width, 148) == (tile_n, per_pair)
     gen = torch.Generator(device="cuda").manual_seed(n + d_model)
     x = torch.randn(n, d_model, device="cuda", generator=gen).to(torch.bfloat16)
     w = (torch.randn(3 * width, d_model, device="cuda", generator=gen) * d_model ** -0.5).to(torch.bfloat16)

@@ -1,12 +1,13 @@
 """GPU parity where the softmax references have to move.
 
 The attention kernel computes a 64-key piece against the reference maxima of the
-keys before it and moves a reference only when a score rises more than 32 octaves
-above it.  Random activations seldom do that, so the scores here are made to:
-one feature of the keys climbs by a chosen number of octaves at chosen keys (in the
-first and in the second piece of a step, at the first key of a step, at the last),
-and the queries follow it with different signs and strengths, so that within one
-warp some rows move and others do not."""
+keys before it and moves the references of a warp's rows when the sum of the 16
+weights that a thread holds of a row reaches 128: a single score seven octaves above
+its reference, or sixteen of them three octaves above.  Random activations seldom do
+that, so the scores here are made to: one feature of the keys climbs by a chosen
+number of octaves at chosen keys (in the first and in the second piece of a step, at
+the first key of a step, at the last), and the queries follow it with different
+signs and strengths, so that within one warp some rows move and others do not."""
 import numpy as np
 import pytest
 import torch
@@ -18,17 +19,11 @@ from gpu_util import f64
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("head_dim", [64, 128])
-@pytest.mark.parametrize("octaves", [5.0, 8.0, 33.0, 120.0, 300.0])
-@pytest.mark.parametrize("n_q,n_k", [(40, 400), (300, 129)])
-def test_scores_that_climb(head_dim, octaves, n_q, n_k):
-    heads = 3
-    gen = torch.Generator().manual_seed(int(octaves) * 1000 + n_k + head_dim)
+def check_climb(head_dim, climb, n_q, seed, scale=1.0):
+    heads, n_k = 3, len(climb)
+    gen = torch.Generator().manual_seed(seed)
     q, k, v = (torch.randn(n, heads, head_dim, generator=gen) for n in (n_q, n_k, n_k))
-    climb = torch.zeros(n_k)
-    for at in (3, 64, 70, 128, 191, 255, 256, 383, 399):
-        if at < n_k:
-            climb[at:] += octaves
+    q *= scale
     # feature 0 adds strength * climb octaves to a score: strengths 1, 0.5, 0, -1 row by row
     strength = torch.tensor([1.0, 0.5, 0.0, -1.0]).repeat(n_q // 4 + 1)[:n_q]
     q[:, :, 0] = strength[:, None] * 8.0
@@ -52,3 +47,29 @@ def test_scores_that_climb(head_dim, octaves, n_q, n_k):
     # scores are fp32 sums: 2^-20 of the largest, and the weights' own error (7.5e-5 of a weight at head_dim 64)
     assert np.abs(lse.cpu().numpy() - want_lse).max() <= 2e-4 + 2.0 ** -20 * s.abs().max().item()
     cache.close()
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("octaves", [5.0, 8.0, 33.0, 120.0, 300.0])
+@pytest.mark.parametrize("n_q,n_k", [(40, 400), (300, 129)])
+def test_scores_that_climb(head_dim, octaves, n_q, n_k):
+    climb = torch.zeros(n_k)
+    for at in (3, 64, 70, 128, 191, 255, 256, 383, 399):
+        if at < n_k:
+            climb[at:] += octaves
+    check_climb(head_dim, climb, n_q, int(octaves) * 1000 + n_k + head_dim)
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("octaves,single", [(6.5, True), (7.5, True), (2.75, False), (3.25, False)])
+def test_scores_on_both_sides_of_the_limit(head_dim, octaves, single):
+    """One key a piece up by just under and just over seven octaves; all keys of a piece up by just under and just over three,
+    so that no weight but their sum comes near the limit.  The other features only blur this: they are small here."""
+    climb = torch.zeros(520)
+    if single:
+        climb[torch.tensor([70, 133, 200, 260, 390, 519])] = octaves
+    else:
+        climb[64:128] = octaves
+        climb[256:320] = octaves
+        climb[448:] = octaves
+    check_climb(head_dim, climb, 40, int(4 * octaves) + head_dim, scale=0.05)
