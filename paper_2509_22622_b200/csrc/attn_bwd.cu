@@ -694,7 +694,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
 
 }  // namespace
 
-cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, cudaStream_t stream)
+cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, int sm_count, cudaStream_t stream)
 {
     const int D = p.head_dim;
     const size_t tile = (size_t)128 * D * 2, ptile = 2 * 128 * 128;
@@ -716,7 +716,7 @@ cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, cudaSt
     if (e != cudaSuccess) return e;
     long long steps = 0;
     for (int g = 0; g < p.n_groups; ++g) steps += (long long)p.heads * ((p.g[g].q_rows + kTile - 1) / kTile) * p.g[g].n_kt;
-    const bool early = steps <= kEarlySteps * 148;
+    const bool early = steps <= kEarlySteps * sm_count;
     dim3 gq((unsigned)p.n_qtiles, (unsigned)p.heads), gk((unsigned)p.n_ktiles, (unsigned)p.heads);
     e = D == 128 ? launch_dependent(early, bwd_dq_kernel<128>, gq, kBwdThreads, smem_dq, stream, p, maps)
                  : launch_dependent(early, bwd_dq_kernel<64>, gq, kBwdThreads, smem_dq, stream, p, maps);

@@ -74,7 +74,8 @@ constexpr float kSafeSum = 128.f;
 // Register reallocation draws on what the CTA was launched with: 640 threads x 96
 // registers = (16 softmax warps x kSoftmaxRegs + 4 producer-group warps x kProducerRegs) x 32.  A
 // request beyond that total would block forever.  At head_dim 64 the softmax warps hold a whole
-// score tile (64 registers), which spills at 104.
+// score tile (64 registers) and take what the producers can spare (24 bytes of spill
+// stores and 124 of loads remain).
 constexpr int kLaunchRegs = 96;
 template <int D> constexpr int kSoftmaxRegs = D == 64 ? 112 : 104;
 template <int D> constexpr int kProducerRegs = D == 64 ? 32 : 64;
@@ -87,7 +88,7 @@ static_assert(kRegsFit<64> && kRegsFit<128>, "setmaxnreg targets exceed the CTA'
 // 0.4047 ms with one group in four, 0.4218 ms with two; 0.4664 / 0.4715 / 0.4915 ms in a long
 // loop at the power cap).  head_dim 64 has twice the exponentials per flop and is bound by
 // them: one group in four (0.681 ms against 0.726 ms with none, 0.684 / 0.683 ms with one in
-// eight / three in eight, 24 heads on the same grid).
+// eight / three in eight, 24 heads on the same grid; measured when the loop still took half a score tile at a time).
 template <int D> constexpr uint32_t kPolyMask = D == 64 ? 0x8888u : 0x0000u;
 
 template <int D>

@@ -302,20 +302,22 @@ int qkv_tile_width(int n_tokens, int width, int sm_count)
 
 // Fewer columns than CTAs, all equally long: every column in the same number of equal parts, one part per
 // CTA, when that is the cheapest way.  In steps, a part costs its own length; splitting at all costs the trip of
-// the parts through the scratch slots (kSplitSteps) and the merge, which loads four parts at a time
-// (kMergeSteps each).  Against levelled shares it saves a CTA's second column segment
+// the parts through the scratch slots (kTripSteps) and the merge, by four parts (kBatchSteps each).  Against levelled shares it saves a CTA's second column segment
 // (kSegmentSteps: its first loads and its drain) and a part per column.  Over 40 drawn launches of
 // up to 100 GF the split by these costs takes 0.926 of the time of levelled shares (geometric mean; 95 x 662, 40
-// heads of 128: 19.5 -> 12.8 us); with (kSplitSteps, kMergeSteps) of (1, 0.75) or (2.5, 1.5) shapes of 10 to 20
-// steps are split that are faster whole.  The benchmark layer's preview grid (17 x 29): 76 -> 71 us.
+// heads of 128: 19.5 -> 12.8 us); with (kTripSteps, kBatchSteps) of (1, 0.75) or (2.5, 1.5) shapes of 10 to 20
+// steps are split that are faster whole.  The benchmark layer's preview grid (17 x 29): 76 -> 70 us.
+//   Every part takes its weights against references of its own, and the largest weight of a row and part is exactly 1
+// in bf16: with fewer parts fewer weights are exact.  Against 64 bits the relative error of few short columns is 2.25e-3 to
+// 2.36e-3 where levelled shares of a step or two gave 2.17e-3 to 2.28e-3; that of long columns is up to 2.37e-3 either way.
 bool even_split(ll::AttnParams *p, int sms, long long all_cols)
 {
-    constexpr double kSplitSteps = 2.5, kMergeSteps = 2.5, kSegmentSteps = 2;
+    constexpr double kTripSteps = 2.5, kBatchSteps = 2.5, kSegmentSteps = 2;
     if (all_cols >= sms || all_cols <= 0) return false;
     const long long n_kt = p->g[0].n_kt;
     for (int g = 1; g < p->n_groups; ++g)
         if (p->g[g].n_kt != n_kt) return false;
-    auto merge = [&](long long parts) { return parts > 1 ? kSplitSteps + kMergeSteps * ((parts + 3) / 4) : 0.; };
+    auto merge = [&](long long parts) { return parts > 1 ? kTripSteps + kBatchSteps * ((parts + 3) / 4) : 0.; };
     long long best = 1;
     double cost = (double)n_kt;
     for (long long k = 2; k <= std::min<long long>(sms / all_cols, n_kt); ++k) {
@@ -1227,7 +1229,7 @@ int ll_clip_attn_backward(ll_cache *c, int layer, const ll_bf16 *q_roped, const 
     if (s != LL_OK) return s;
     maps.k = c->kmap[layer];
     maps.v = c->vmap[layer];
-    cudaError_t e = ll::launch_attn_backward(p, maps, (cudaStream_t)stream);
+    cudaError_t e = ll::launch_attn_backward(p, maps, c->sm_count > 0 ? c->sm_count : 148, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "clip backward kernels");
     return LL_OK;
 }

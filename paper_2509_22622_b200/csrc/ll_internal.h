@@ -189,7 +189,7 @@ struct BwdParams {
     AttnGroup g[kMaxGroups];
 };
 struct BwdMaps { CUtensorMap q, d_out, k, v; };
-cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, cudaStream_t stream);
+cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, int sm_count, cudaStream_t stream);
 
 // Launch on `stream` so that the kernel may start before the one in front of it has ended
 // (grid_dep_wait in ptx.cuh): the launch latency and the set-up of a kernel then run under its predecessor's
