@@ -364,27 +364,23 @@ void plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_ste
     p->all_cols = (int)all_cols;
     if (even_split(p, sms, all_cols)) return;
     // What goes out whole and what is left of it, and the steps each CTA gets as whole columns
-    long long load[ll::kMaxCtas], steps = 0;
-    auto deal = [&]() {
-        const long long whole_cols = std::min<long long>((long long)p->n_waves * p->n_ctas, all_cols);
-        std::fill(load, load + ll::kMaxCtas, 0);
-        steps = 0;
-        for (int g = 0; g < p->n_groups; ++g) {
-            ll::AttnGroup &G = p->g[g];
-            const long long cols = (long long)p->heads * G.tiles;
-            G.wave_cols = (int)std::min(cols, std::max<long long>(0, whole_cols - G.col_begin));
-            G.step_begin = steps;
-            steps += (cols - G.wave_cols) * G.n_kt;
-            // of the columns [0, x) CTA i takes those congruent to i: (x + n - 1 - i) / n of them
-            const long long lo = G.col_begin, hi = G.col_begin + G.wave_cols, n = p->n_ctas;
-            for (int i = 0; i < p->n_ctas; ++i)
-                load[i] += ((hi + n - 1 - i) / n - (lo + n - 1 - i) / n) * G.n_kt;
-        }
-    };
+    long long load[ll::kMaxCtas] = {}, steps = 0;
+    const int n = p->n_ctas;
+    const long long whole_cols = std::min<long long>((long long)p->n_waves * n, all_cols);
+    for (int g = 0; g < p->n_groups && n > 0; ++g) {
+        ll::AttnGroup &G = p->g[g];
+        const long long cols = (long long)p->heads * G.tiles;
+        G.wave_cols = (int)std::min(cols, std::max<long long>(0, whole_cols - G.col_begin));
+        G.step_begin = steps;
+        steps += (cols - G.wave_cols) * G.n_kt;
+        // of the columns [0, x) CTA i takes those congruent to i: x / n, and one more below x % n
+        const int lo = (int)G.col_begin, hi = lo + G.wave_cols, lo_q = lo / n, lo_r = lo % n, hi_q = hi / n, hi_r = hi % n;
+        for (int i = 0; i < n; ++i) load[i] += (long long)(hi_q + (i < hi_r) - lo_q - (i < lo_r)) * G.n_kt;
+    }
     // the highest level T that the shared steps can fill: sum over CTAs of max(0, T - load) <= steps
     auto fill = [&](long long T) {
         long long need = 0;
-        for (int i = 0; i < p->n_ctas; ++i) need += std::max<long long>(0, T - load[i]);
+        for (int i = 0; i < n; ++i) need += std::max<long long>(0, T - load[i]);
         return need;
     };
     auto level = [&]() {
@@ -395,7 +391,6 @@ void plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_ste
         }
         return lo;
     };
-    deal();
     if (steps > 0) {
         // Short columns: splitting the leftover columns saves at most their length minus an even
         // share, and costs every part a trip through the scratch slots and most CTAs a second
@@ -407,7 +402,7 @@ void plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_ste
         // whole behind two columns of 19, 140 split.  Over the 37 of 60 drawn launches with unequal loads that the first
         // condition lets through, 14 to 16 steps choose within 0.5 % of the faster way, 8 within 1.8 %.)
         constexpr long long kMergeSteps = 6, kSplitSteps = 15;
-        const long long first_left = (long long)p->n_waves * p->n_ctas;
+        const long long first_left = (long long)p->n_waves * n;
         long long left_longest = 0, whole_top = 0;
         for (int g = 0; g < p->n_groups; ++g) {
             const ll::AttnGroup &G = p->g[g];
@@ -421,7 +416,13 @@ void plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_ste
             whole_top <= std::max(*std::max_element(load, load + ll::kMaxCtas), level() + kSplitSteps)) {
             p->n_waves += 1;
             p->n_ctas = (int)std::min<long long>(sms, all_cols);
-            deal();
+            for (int g = 0; g < p->n_groups; ++g) {
+                p->g[g].wave_cols = p->heads * p->g[g].tiles;
+                p->g[g].step_begin = 0;
+            }
+            for (int i = 0; i < p->n_ctas; ++i) p->share_of_cta[i] = -1;
+            p->total_steps = 0;
+            return;                                      // n_shares 0, share_begin[0] 0: the parameters start out zero
         }
     }
     p->total_steps = steps;
