@@ -17,11 +17,14 @@
 // release its tensor memory at once, so the next step's S is formed while they are in the
 // exponentials; dP is read only for the last multiply.
 //   What they compute goes back to tensor memory as the A operand of the products that follow: dS over dP, and in
-// the dk/dv kernel P over S.  Through shared memory those tiles cost a store and a read of 32 KB each beside
-// operands of 64 KB per 512 clk of products.
-//   21-frame clip of the benchmark layer (32760 rows, 12 heads of 128): 9.20 -> 8.56 ms in a loop at the power limit, 8.46 ->
-// 7.85 ms in bursts; the dq kernel alone 4.44 -> 4.07 ms, the dk/dv kernel 3.80 -> 3.49.  Serving the two 64-key halves of the dq kernel's steps as chains
-// of their own, half a step apart, was slower (64-wide products: 4.66 ms for the kernel, 9.22 ms in the loop).
+// the dk/dv kernel P over S (at head_dim 64 beside them, where columns are left).  Through shared memory those tiles
+// cost a store and a read of 32 KB each beside operands of 64 KB per 512 clk of products.
+//   Products run in the order of their issue only if they share accumulator and shape.  One that overwrites columns
+// which an earlier one reads as its A operand is therefore issued behind that one's commit; stores from registers are
+// behind a later product's commit anyway, which covers all products before it.
+//   21-frame clip of the benchmark layer (32760 rows, 12 heads of 128): 9.25 -> 8.80 ms in a loop at the power limit (8.65 without
+// the waits between products).  Serving the two 64-key halves of the dq kernel's steps as chains of their own, half a step
+// apart, was slower (64-wide products: 4.66 ms for the kernel where it took 4.07 without those waits).
 #include <cuda_bf16.h>
 
 #include "bounded_wait.cuh"
@@ -218,9 +221,9 @@ __device__ __forceinline__ void scores_to_weights(uint32_t (&s)[64], float c, fl
 // half).  Per 128-key step j the tensor pipe runs S(j+1) | dQ(j) | dP(j+1) ...: the compute warps
 // take S(j) into registers and release it at once, so S(j+1) is formed while they are in the
 // exponentials; dP(j) is only needed for the last multiply, dS = P (dP - delta), which goes back
-// over it as bf16 (products of one thread run in order, so dP(j+1) may overwrite dS(j) behind dQ(j) without a
-// wait).  K and V tiles sit in three stages; K is needed until the step's dQ product, V only until its dP.
-//   tensor memory columns: S 0..127, dP 128..255 (dS of key half h at 128 + 64 h..), dQ 256..256+D-1, Q 384.., dO 448..
+// over it as bf16, so that dP(j+1) waits for dQ(j), or at head_dim 64 into columns of its own.  K and V tiles sit in
+// three stages; K is needed until the step's dQ product, V only until its dP.
+//   tensor memory columns: S 0..127, dP 128..255, dQ 256..256+D-1, Q 384.., dO 448..; dS of key half h at 128 + 64 h.. or 416 + 64 h..
 template <int D>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMaps maps)
@@ -260,7 +263,9 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
     WaitCtx ctx{abort_flag, p.status, warp};
     auto wait = [&](int bar_id, uint32_t parity, int iter) -> bool { return wait_bar(bar(bar_id), parity & 1u, ctx, bar_id, iter); };
     const bool skip = *abort_flag != 0;
-    const uint32_t t_s = tmem, t_dp = tmem + 128, t_dq = tmem + 256, t_q = tmem + 384, t_do = tmem + 448;
+    constexpr bool kOverDp = D == 128;                           // dS takes the place of dP
+    const uint32_t t_s = tmem, t_dp = tmem + 128, t_dq = tmem + 256, t_q = tmem + 384, t_do = tmem + 448,
+                   t_ds = kOverDp ? t_dp : tmem + 416;
 
     // the tile's Q rows (warps 0-3) and dO rows (warps 4-7) into tensor memory; rows past the
     // group's end become zeros
@@ -328,8 +333,9 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
             auto issue_dp = [&](int j) -> bool {                 // dP(j) = dO V(j)^T
                 const int st = j % kStages;
                 if (!wait(kVFull + st, j / kStages, j)) return false;
-                tc_fence_after_sync();
                 const uint32_t b_lo = v_lo + ((uint32_t)(st * C::kTileBytes) >> 4);
+                if (kOverDp && j > 0 && !wait(kKEmpty + (j - 1) % kStages, (j - 1) / kStages, j)) return false;      // dQ(j-1) has read dS(j-1)
+                tc_fence_after_sync();
                 if (elected) {
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk)
@@ -353,13 +359,13 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
                     if (!wait(kSFree, j, j)) return;             // S(j) is in the compute warps' registers
                     if (!issue_s(j + 1)) return;
                 }
-                if (!wait(kDsFull, j, j)) return;                // dS(j) is in shared memory, dP(j) has been read
+                if (!wait(kDsFull, j, j)) return;                // dS(j) is in tensor memory, dP(j) has been read
                 tc_fence_after_sync();
                 const uint32_t k_mn = lo_mnmajor(k_s + st * C::kTileBytes);
                 if (elected) {
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
-                        mma_ts(t_dq, t_dp + (kk >= 4 ? 64 : 0) + 8 * (kk & 3), smem_desc_join(k_mn + slice_mnmajor(kk), hi), idesc_dq,
+                        mma_ts(t_dq, t_ds + (kk >= 4 ? 64 : 0) + 8 * (kk & 3), smem_desc_join(k_mn + slice_mnmajor(kk), hi), idesc_dq,
                                (j > 0 || kk > 0) ? 1u : 0u);
                 }
                 __syncwarp();
@@ -396,7 +402,7 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
             tc_fence_after_sync();
             const uint64_t nd2 = pack2(-delta, -delta);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {                        // dS = p (dP - delta), bf16, over dP
+            for (int h = 0; h < 2; ++h) {                        // dS = p (dP - delta), bf16
                 uint32_t dp[32], dw[16];
                 tmem_ld_32x32b_x32(t_dp + lane_off + 64 * half + 32 * h, dp);
                 tmem_wait_ld();
@@ -407,7 +413,7 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
                                  add2(pack2(as_f(dp[2 * i]), as_f(dp[2 * i + 1])), nd2)), d0, d1);
                     dw[i] = cvt_bf16x2(d0, d1);
                 }
-                tmem_st_32x32b_x16(t_dp + lane_off + 64 * half + 16 * h, dw);
+                tmem_st_32x32b_x16(t_ds + lane_off + 64 * half + 16 * h, dw);
             }
             tmem_wait_st();
             tc_fence_before_sync();
@@ -487,13 +493,14 @@ struct QTiles {
 // K and V of the tile stay in shared memory; per step j one query tile's Q and dO stream in (two slots each, loaded
 // by a warp of their own).  Scores are formed with the keys as rows, S^T = K Q^T and dP^T = V dO^T, so that
 // P^T and dS^T are the A operands of dV += P^T dO and dK += dS^T Q in the rows they are computed in: they go back to
-// tensor memory as bf16, over S and dP (all 512 columns are taken), and never through shared memory.
-//   The tensor pipe runs, per step,  dV(j) | S(j+1) | dK(j) | dP(j+1);  products of one thread run in order, so S(j+1)
-// may overwrite P(j) without a wait, and dP(j+1) dS(j).  P(j) is handed over in two pieces, so that half of dV(j) runs
-// under the second piece's exponentials, and dS(j) is formed under the rest of dV(j) and S(j+1).
+// tensor memory as bf16 and never through shared memory.  At head_dim 128 all 512 columns are taken and they go over S and
+// dP, so that S(j+1) waits for dV(j), and dP(j+1) for dK(j); at 64 they have columns of their own.
+//   The tensor pipe runs, per step,  dV(j) | S(j+1) | dK(j) | dP(j+1).  P(j) is handed over in two pieces, so that half of
+// dV(j) runs under the second piece's exponentials, and dS(j) is formed under the rest of dV(j) and S(j+1).
 // The row statistics are per column here: the load warp lays them out in shared memory (negated, in pairs for
 // the packed arithmetic).
-//   tensor memory columns: S 0..127 (P: 16-query slices 0-3 at 0.., 4-7 at 64..), dP 128..255 (dS likewise), dK, dV.
+//   tensor memory columns: S 0..127, dP 128..255, dK and dV 256..256+2D-1; P (16-query slices 0-3 at 0.., 4-7 at 64.. of it) at 0
+// or 384, dS (likewise) at 128 or 416.
 template <int D>
 __global__ void __launch_bounds__(kDkdvThreads, 1)
 bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMaps maps)
@@ -532,7 +539,9 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
     WaitCtx ctx{abort_flag, p.status, warp};
     auto wait = [&](int bar_id, uint32_t parity, int iter) -> bool { return wait_bar(bar(bar_id), parity & 1u, ctx, bar_id, iter); };
     const bool skip = *abort_flag != 0;
-    const uint32_t t_s = tmem, t_dp = tmem + 128, t_dk = tmem + 256, t_dv = tmem + 256 + D;
+    constexpr bool kOver = D == 128;                             // P and dS take the places of S and dP
+    const uint32_t t_s = tmem, t_dp = tmem + 128, t_dk = tmem + 256, t_dv = tmem + 256 + D,
+                   t_p = kOver ? t_s : tmem + 384, t_ds = kOver ? t_dp : tmem + 416;
 
     if (skip) {
     } else if (warp == kLoadWarp) {
@@ -595,6 +604,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
             auto issue_s = [&](int j) -> bool {                  // S^T(j) = K Q(j)^T
                 const int sl = j & 1;
                 if (!wait(kQFull + sl, j >> 1, j)) return false;
+                if (kOver && j > 0 && !wait(kDoEmpty + (sl ^ 1), (j - 1) >> 1, j)) return false;     // dV(j-1) has read P(j-1)
                 tc_fence_after_sync();
                 if (elected) mma_slices<0, D / 16, false, false>(t_s, k_k, lo_kmajor(q_s + sl * C::kTileBytes), idesc_s, 0u);
                 __syncwarp();
@@ -604,6 +614,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
             auto issue_dp = [&](int j) -> bool {                 // dP^T(j) = V dO(j)^T
                 const int sl = j & 1;
                 if (!wait(kDoFull + sl, j >> 1, j)) return false;
+                if (kOver && j > 0 && !wait(kQEmpty + (sl ^ 1), (j - 1) >> 1, j)) return false;      // dK(j-1) has read dS(j-1)
                 tc_fence_after_sync();
                 if (elected) mma_slices<0, D / 16, false, false>(t_dp, v_k, lo_kmajor(do_s + sl * C::kTileBytes), idesc_s, 0u);
                 __syncwarp();
@@ -625,10 +636,10 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                     if (!wait(h ? kPFull : kPHalf, j, j)) return;
                     tc_fence_after_sync();
                     if (elected) {
-                        slice(t_dv, t_s, do_mn, 2 * h, (j > 0 || h > 0) ? 1u : 0u);
-                        slice(t_dv, t_s, do_mn, 2 * h + 1, 1u);
-                        slice(t_dv, t_s, do_mn, 2 * h + 4, 1u);
-                        slice(t_dv, t_s, do_mn, 2 * h + 5, 1u);
+                        slice(t_dv, t_p, do_mn, 2 * h, (j > 0 || h > 0) ? 1u : 0u);
+                        slice(t_dv, t_p, do_mn, 2 * h + 1, 1u);
+                        slice(t_dv, t_p, do_mn, 2 * h + 4, 1u);
+                        slice(t_dv, t_p, do_mn, 2 * h + 5, 1u);
                     }
                     __syncwarp();
                 }
@@ -638,7 +649,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                 tc_fence_after_sync();
                 if (elected) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) slice(t_dk, t_dp, q_mn, kk, (j > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < 8; ++kk) slice(t_dk, t_ds, q_mn, kk, (j > 0 || kk > 0) ? 1u : 0u);
                 }
                 __syncwarp();
                 commit(kQEmpty + sl);
@@ -653,7 +664,8 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
         };
         const int row = threadIdx.x & 127, half = threadIdx.x >> 7;      // key row of the tile = TMEM lane; 64-query half
         const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-        const uint32_t t_sh = t_s + lane_off + 64 * half, t_dph = t_dp + lane_off + 64 * half;
+        const uint32_t t_sh = t_s + lane_off + 64 * half, t_dph = t_dp + lane_off + 64 * half,
+                       t_ph = t_p + lane_off + 64 * half, t_dsh = t_ds + lane_off + 64 * half;
         const uint64_t c2 = pack2(p.scale_log2, p.scale_log2);
         uint32_t step = 0;
         for (int g = 0; g < p.n_groups; ++g) {
@@ -692,7 +704,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                     }
 #pragma unroll
                     for (int k = 0; k < 16; ++k) pw[k] = cvt_bf16x2(as_f(w[32 * h + 2 * k]), as_f(w[32 * h + 2 * k + 1]));
-                    tmem_st_32x32b_x16(t_sh + 16 * h, pw);
+                    tmem_st_32x32b_x16(t_ph + 16 * h, pw);
                     tmem_wait_st();
                     tc_fence_before_sync();
                     __syncwarp();
@@ -715,7 +727,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                         unpack2(mul2(pack2(as_f(v[2]), as_f(v[3])), add2(pack2(as_f(x[2]), as_f(x[3])), pack2(n.z, n.w))), d0, d1);
                         dw[2 * k + 1] = cvt_bf16x2(d0, d1);
                     }
-                    tmem_st_32x32b_x16(t_dph + 16 * h, dw);
+                    tmem_st_32x32b_x16(t_dsh + 16 * h, dw);
                 }
                 tmem_wait_st();
                 tc_fence_before_sync();
