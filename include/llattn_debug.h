@@ -82,6 +82,10 @@ int ll_debug_attn_tiles(ll_cache *cache, int layer, int sm_count, int *tile_ctas
  * busiest pair works through.  Host-only. */
 int ll_debug_qkv_tiles(int n_tokens, int width, int sm_count, int *tile_n, int *tiles_per_pair);
 
+/* Whether ll_norm_rope_append_kv of n_tokens tokens streams its rows through shared memory (1) or not (0) on a GPU of
+ * sm_count SMs (148 when 0); with_q = 0: k and v alone.  Host-only. */
+int ll_debug_norm_rows(int heads, int head_dim, int n_tokens, int with_q, int sm_count, int *streamed);
+
 /* Byte offsets, inside the bound storage, of the regions of the aux block that
  * the attention kernel and the bounded waits write: the status words and the
  * arrival counters of the split-column merge (Sec. 3.3's attention needs

@@ -137,6 +137,7 @@ SIGNATURES = {
     "ll_debug_attn_plan": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.POINTER(ll_attn_plan)]),
     "ll_debug_attn_plan_batched": (C.c_int, [C.POINTER(ll_attn_item), C.c_int, C.c_int, C.POINTER(ll_attn_plan)]),
     "ll_debug_attn_tiles": (C.c_int, [C.c_void_p, C.c_int, C.c_int] + [C.POINTER(C.c_int)] * 3),
+    "ll_debug_norm_rows": (C.c_int, [C.c_int] * 5 + [C.POINTER(C.c_int)]),
     "ll_debug_qkv_tiles": (C.c_int, [C.c_int] * 3 + [C.POINTER(C.c_int)] * 2),
     "ll_debug_aux_layout": (C.c_int, [C.c_void_p] + [C.POINTER(C.c_size_t)] * 4),
     "ll_debug_guard_layout": (C.c_int, [C.c_void_p] + [C.POINTER(C.c_size_t)] * 3),
@@ -373,6 +374,13 @@ def ll_debug_attn_tiles(h, layer=0, sm_count=0):
     v = [C.c_int() for _ in range(3)]
     _check(lib().ll_debug_attn_tiles(h, layer, sm_count, *[C.byref(x) for x in v]))
     return tuple(x.value for x in v)
+
+
+def ll_debug_norm_rows(heads, head_dim, n_tokens, with_q=True, sm_count=0) -> bool:
+    """Whether the append with the norm streams its rows through shared memory."""
+    v = C.c_int()
+    _check(lib().ll_debug_norm_rows(heads, head_dim, n_tokens, int(with_q), sm_count, C.byref(v)))
+    return bool(v.value)
 
 
 def ll_debug_qkv_tiles(n_tokens, width, sm_count=0):

@@ -1403,6 +1403,13 @@ int ll_debug_qkv_tiles(int n_tokens, int width, int sm_count, int *tile_n, int *
     return LL_OK;
 }
 
+int ll_debug_norm_rows(int heads, int head_dim, int n_tokens, int with_q, int sm_count, int *streamed)
+{
+    if (heads <= 0 || (head_dim != 64 && head_dim != 128) || n_tokens <= 0 || !streamed) return fail(LL_ERR_INVALID_ARG, "bad argument to ll_debug_norm_rows");
+    *streamed = ll::norm_append_streams(heads, head_dim, n_tokens, with_q != 0, sm_count);
+    return LL_OK;
+}
+
 int ll_debug_aux_layout(const ll_cache *c, size_t *status_offset, size_t *status_bytes, size_t *counters_offset,
                         size_t *counters_bytes)
 {

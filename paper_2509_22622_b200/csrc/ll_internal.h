@@ -307,6 +307,7 @@ struct StageParams {
     int start[kMaxStageRuns], len[kMaxStageRuns];
 };
 cudaError_t launch_stage_e4m3(const StageParams &p, int head_dim, cudaStream_t stream);
+bool norm_append_streams(int heads, int head_dim, int n_tokens, bool with_q, int sm_count);
 cudaError_t launch_norm_rope_append(const RopeAppendParams &p, int head_dim, const float *gain_q, const float *gain_k,
                                     float eps, int sm_count, cudaStream_t stream);
 cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps &maps, cudaStream_t stream);
