@@ -47,10 +47,14 @@ int ll_debug_wait_timeout(ll_cache *cache, int limit_ms, ll_stream stream);
  * When the columns are short (merging the parts of a split column would cost
  * more than splitting saves) nothing is shared: the last wave is partial,
  * columns numbered all_cols and up do not exist, and n_shares is 0.
- * Equally long columns may go out by 128-row tiles instead when that is faster: ll_debug_attn_tiles
- * says so, and the division into columns above is then not used.
+ * Equally long columns may go out by 128-row tiles instead when that is faster.  The division into columns
+ * above is then not used, and tile_ctas, otherwise 0, is the number of CTAs: the row_tiles[g] tiles of a group's heads are
+ * numbered one after the other, group after group, and CTA i takes tiles_each consecutive ones, one more when
+ * i < tiles_extra, two of one head at a time.
  * ll_debug_attn_plan_batched: the same for ll_sink_window_attn_batched of the
- * newest chunk of every item (only cache and layer of an item are read). */
+ * newest chunk of every item (only cache and layer of an item are read).
+ * ll_debug_attn_plan_clip: for ll_clip_append_attn (and its backward), of the newest n_frames frames.
+ * ll_debug_attn_plan_cross: for ll_cross_attn. */
 #define LL_MAX_GROUPS 24
 #define LL_MAX_CTAS 160
 typedef struct ll_attn_plan {
@@ -68,13 +72,17 @@ typedef struct ll_attn_plan {
     int64_t step_begin[LL_MAX_GROUPS];
     int32_t share_begin[LL_MAX_CTAS + 1];
     int32_t share_of_cta[LL_MAX_CTAS];
+    int32_t tile_ctas;
+    int32_t tiles_each;
+    int32_t tiles_extra;
+    int32_t row_tiles[LL_MAX_GROUPS];
 } ll_attn_plan;
 int ll_debug_attn_plan(ll_cache *cache, int layer, int recache, int sm_count, ll_attn_plan *out);
 int ll_debug_attn_plan_batched(const ll_attn_item *items, int n_items, int sm_count, ll_attn_plan *out);
+int ll_debug_attn_plan_clip(ll_cache *cache, int layer, int n_frames, int attn_window_frames, int sm_count, ll_attn_plan *out);
+int ll_debug_attn_plan_cross(ll_cache *cache, int64_t n_q, int64_t n_k, int sm_count, ll_attn_plan *out);
 
-/* The same call's division by 128-row tiles (tiles of a group's heads one after the other, group after group): CTA i of
- * tile_ctas takes tiles_each consecutive tiles, one more when i < tiles_extra, two of one head at a time.  tile_ctas = 0:
- * it goes out by ll_debug_attn_plan. */
+/* The tile_ctas, tiles_each and tiles_extra of ll_debug_attn_plan with recache = 0. */
 int ll_debug_attn_tiles(ll_cache *cache, int layer, int sm_count, int *tile_ctas, int *tiles_each, int *tiles_extra);
 
 /* The division of ll_qkv_proj_append's GEMM for n_tokens tokens and q, k, v rows of `width` features on a GPU of

@@ -62,6 +62,10 @@ class ll_attn_plan(C.Structure):
         ("step_begin", C.c_int64 * LL_MAX_GROUPS),
         ("share_begin", C.c_int32 * (LL_MAX_CTAS + 1)),
         ("share_of_cta", C.c_int32 * LL_MAX_CTAS),
+        ("tile_ctas", C.c_int32),
+        ("tiles_each", C.c_int32),
+        ("tiles_extra", C.c_int32),
+        ("row_tiles", C.c_int32 * LL_MAX_GROUPS),
     ]
 
 
@@ -136,6 +140,8 @@ SIGNATURES = {
     "ll_debug_wait_timeout": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p]),
     "ll_debug_attn_plan": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.POINTER(ll_attn_plan)]),
     "ll_debug_attn_plan_batched": (C.c_int, [C.POINTER(ll_attn_item), C.c_int, C.c_int, C.POINTER(ll_attn_plan)]),
+    "ll_debug_attn_plan_clip": (C.c_int, [C.c_void_p] + [C.c_int] * 4 + [C.POINTER(ll_attn_plan)]),
+    "ll_debug_attn_plan_cross": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_int, C.POINTER(ll_attn_plan)]),
     "ll_debug_attn_tiles": (C.c_int, [C.c_void_p, C.c_int, C.c_int] + [C.POINTER(C.c_int)] * 3),
     "ll_debug_norm_rows": (C.c_int, [C.c_int] * 5 + [C.POINTER(C.c_int)]),
     "ll_debug_qkv_tiles": (C.c_int, [C.c_int] * 3 + [C.POINTER(C.c_int)] * 2),
@@ -366,6 +372,18 @@ def ll_debug_attn_plan_batched(handles_and_layers, sm_count=0) -> ll_attn_plan:
         arr[i].layer = layer
     plan = ll_attn_plan()
     _check(lib().ll_debug_attn_plan_batched(arr, len(handles_and_layers), sm_count, C.byref(plan)))
+    return plan
+
+
+def ll_debug_attn_plan_clip(h, n_frames, attn_window_frames, layer=0, sm_count=0) -> ll_attn_plan:
+    plan = ll_attn_plan()
+    _check(lib().ll_debug_attn_plan_clip(h, layer, n_frames, attn_window_frames, sm_count, C.byref(plan)))
+    return plan
+
+
+def ll_debug_attn_plan_cross(h, n_q, n_k, sm_count=0) -> ll_attn_plan:
+    plan = ll_attn_plan()
+    _check(lib().ll_debug_attn_plan_cross(h, n_q, n_k, sm_count, C.byref(plan)))
     return plan
 
 

@@ -279,6 +279,17 @@ struct AttnCall {
     const float *q_scale;                         // per-row factor on the queries, or null
 };
 
+// The chunks of a clip, each with its own window.
+AttnCall clip_call(ll_cache *c, int layer, const ll_bf16 *q, ll_bf16 *out, float *lse, int64_t frame_start, int n_groups, int attn_window_frames)
+{
+    AttnCall call{c, layer, q, out, lse, n_groups, {}, 0, {}};
+    for (int g = 0; g < n_groups; ++g) {
+        call.group_frame_start[g] = frame_start + (int64_t)g * c->C;
+        call.group_lo_floor[g] = call.group_frame_start[g] + c->C - attn_window_frames;
+    }
+    return call;
+}
+
 // Tiles of the projection that the busiest of the SM pairs works through.
 long long qkv_rounds(int n_tokens, int width, int sm_count, int tile_n)
 {
@@ -1164,11 +1175,7 @@ int ll_clip_append_attn(ll_cache *c, int layer, const ll_bf16 *q, const ll_bf16 
     }
     st.end += n_frames;
     st.n_appends += n_groups;
-    AttnCall call{c, layer, q_out, out, lse_out, n_groups, {}, 0, {}};
-    for (int g = 0; g < n_groups; ++g) {
-        call.group_frame_start[g] = frame_start + (int64_t)g * c->C;
-        call.group_lo_floor[g] = call.group_frame_start[g] + c->C - attn_window_frames;
-    }
+    const AttnCall call = clip_call(c, layer, q_out, out, lse_out, frame_start, n_groups, attn_window_frames);
     ll::AttnParams ap;
     int s = build_attn_params(&call, 1, &ap);
     if (s == LL_OK && !c->dry_run) {
@@ -1230,11 +1237,7 @@ int ll_clip_attn_backward(ll_cache *c, int layer, const ll_bf16 *q_roped, const 
     int s = need_storage(c);
     if (s != LL_OK) return s;
     // the forward's query groups and key runs
-    AttnCall call{c, layer, q_roped, nullptr, nullptr, n_groups, {}, 0, {}};
-    for (int g = 0; g < n_groups; ++g) {
-        call.group_frame_start[g] = frame_start + (int64_t)g * c->C;
-        call.group_lo_floor[g] = call.group_frame_start[g] + c->C - attn_window_frames;
-    }
+    const AttnCall call = clip_call(c, layer, q_roped, nullptr, nullptr, frame_start, n_groups, attn_window_frames);
     ll::AttnParams ap;
     s = build_attn_params(&call, 1, &ap);
     if (s != LL_OK) return s;
@@ -1284,8 +1287,17 @@ int ll_clip_attn_backward(ll_cache *c, int layer, const ll_bf16 *q_roped, const 
 }
 
 namespace {
-void copy_plan(const ll::AttnParams &p, ll_attn_plan *out)
+// The division of a launch, on sm_count SMs if that is positive.
+int debug_plan(const AttnCall *calls, int n_calls, int sm_count, ll_attn_plan *out)
 {
+    static_assert(LL_MAX_GROUPS == ll::kMaxGroups && LL_MAX_CTAS == ll::kMaxCtas, "header and kernel disagree on a limit");
+    ll_cache *c0 = calls[0].c;
+    const int saved = c0->sm_count;
+    if (sm_count > 0) c0->sm_count = sm_count;
+    ll::AttnParams p;
+    const int s = build_attn_params(calls, n_calls, &p);
+    c0->sm_count = saved;
+    if (s != LL_OK) return s;
     memset(out, 0, sizeof *out);
     out->n_ctas = p.n_ctas;
     out->n_groups = p.n_groups;
@@ -1302,7 +1314,12 @@ void copy_plan(const ll::AttnParams &p, ll_attn_plan *out)
         out->col_begin[g] = p.g[g].col_begin;
         out->wave_cols[g] = p.g[g].wave_cols;
         out->step_begin[g] = p.g[g].step_begin;
+        out->row_tiles[g] = (p.g[g].q_rows + 127) / 128;
     }
+    out->tile_ctas = p.tile_ctas;
+    out->tiles_each = p.tiles_each;
+    out->tiles_extra = p.tiles_extra;
+    return LL_OK;
 }
 }  // namespace
 
@@ -1318,20 +1335,12 @@ int ll_debug_attn_plan_batched(const ll_attn_item *items, int n_items, int sm_co
         if (st.end < it.cache->C) return fail(LL_ERR_BAD_POSITION, "no chunk has been appended yet");
         calls[i] = AttnCall{it.cache, it.layer, nullptr, nullptr, nullptr, 1, {st.end - it.cache->C}, 0};
     }
-    ll_cache *c0 = items[0].cache;
-    const int saved = c0->sm_count;
-    if (sm_count > 0) c0->sm_count = sm_count;
-    ll::AttnParams p;
-    const int s = build_attn_params(calls, n_items, &p);
-    c0->sm_count = saved;
-    if (s != LL_OK) return s;
-    copy_plan(p, out);
-    return LL_OK;
+    return debug_plan(calls, n_items, sm_count, out);
 }
 
 namespace {
-// The launch parameters of ll_sink_window_attn of the newest chunk, or of ll_recache of the resident window.
-int debug_params(ll_cache *c, int layer, int recache, int sm_count, ll::AttnParams *p)
+// ll_sink_window_attn of the newest chunk, or ll_recache of the resident window.
+int debug_call_plan(ll_cache *c, int layer, int recache, int sm_count, ll_attn_plan *out)
 {
     const ll::LayerState &st = c->layers[layer];
     int n_groups = 1;
@@ -1346,39 +1355,46 @@ int debug_params(ll_cache *c, int layer, int recache, int sm_count, ll::AttnPara
         if (st.end < c->C) return fail(LL_ERR_BAD_POSITION, "no chunk has been appended yet");
         gstart[0] = st.end - c->C;
     }
-    memset(p, 0, sizeof *p);
+    memset(out, 0, sizeof *out);
     if (n_groups == 0) return LL_OK;
-    const int saved = c->sm_count;
-    if (sm_count > 0) c->sm_count = sm_count;
     AttnCall call{c, layer, nullptr, nullptr, nullptr, n_groups, {}, lo_floor};
     for (int g = 0; g < n_groups; ++g) call.group_frame_start[g] = gstart[g];
-    const int s = build_attn_params(&call, 1, p);
-    c->sm_count = saved;
-    return s;
+    return debug_plan(&call, 1, sm_count, out);
 }
 }  // namespace
 
 int ll_debug_attn_plan(ll_cache *c, int layer, int recache, int sm_count, ll_attn_plan *out)
 {
     if (!layer_ok(c, layer) || !out) return fail(LL_ERR_INVALID_ARG, "bad argument to ll_debug_attn_plan");
-    static_assert(LL_MAX_GROUPS == ll::kMaxGroups && LL_MAX_CTAS == ll::kMaxCtas, "header and kernel disagree on a limit");
-    ll::AttnParams p;
-    const int s = debug_params(c, layer, recache, sm_count, &p);
-    if (s != LL_OK) return s;
-    memset(out, 0, sizeof *out);
-    if (p.n_groups > 0) copy_plan(p, out);
-    return LL_OK;
+    return debug_call_plan(c, layer, recache, sm_count, out);
+}
+
+int ll_debug_attn_plan_clip(ll_cache *c, int layer, int n_frames, int attn_window_frames, int sm_count, ll_attn_plan *out)
+{
+    if (!layer_ok(c, layer) || !out || n_frames <= 0 || n_frames % c->C || n_frames / c->C > ll::kMaxGroups || attn_window_frames < c->C ||
+        attn_window_frames % c->C || n_frames > c->layers[layer].end || (int64_t)attn_window_frames + n_frames - c->C > c->W)
+        return fail(LL_ERR_INVALID_ARG, "bad argument to ll_debug_attn_plan_clip");
+    const AttnCall call = clip_call(c, layer, nullptr, nullptr, nullptr, c->layers[layer].end - n_frames, n_frames / c->C, attn_window_frames);
+    return debug_plan(&call, 1, sm_count, out);
+}
+
+int ll_debug_attn_plan_cross(ll_cache *c, int64_t n_q, int64_t n_k, int sm_count, ll_attn_plan *out)
+{
+    if (!c || !out || n_q <= 0 || n_k <= 0 || n_q > (1ll << 30) || n_k > (1ll << 30))
+        return fail(LL_ERR_INVALID_ARG, "bad argument to ll_debug_attn_plan_cross");
+    const AttnCall call{c, 0, nullptr, nullptr, nullptr, 1, {}, 0, {}, n_q, n_k, nullptr, nullptr};
+    return debug_plan(&call, 1, sm_count, out);
 }
 
 int ll_debug_attn_tiles(ll_cache *c, int layer, int sm_count, int *tile_ctas, int *tiles_each, int *tiles_extra)
 {
     if (!layer_ok(c, layer) || !tile_ctas || !tiles_each || !tiles_extra) return fail(LL_ERR_INVALID_ARG, "bad argument to ll_debug_attn_tiles");
-    ll::AttnParams p;
-    const int s = debug_params(c, layer, 0, sm_count, &p);
+    ll_attn_plan plan;
+    const int s = debug_call_plan(c, layer, 0, sm_count, &plan);
     if (s != LL_OK) return s;
-    *tile_ctas = p.tile_ctas;
-    *tiles_each = p.tiles_each;
-    *tiles_extra = p.tiles_extra;
+    *tile_ctas = plan.tile_ctas;
+    *tiles_each = plan.tiles_each;
+    *tiles_extra = plan.tiles_extra;
     return LL_OK;
 }
 

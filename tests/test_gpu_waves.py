@@ -39,7 +39,7 @@ def oracle_for(oracle_mod, wl):
 
 def plan_is_waves_plus_shares(cache, recache=False):
     plan = B.ll_debug_attn_plan(cache.h, 0, recache, 148)
-    return plan.n_waves >= 1 and plan.n_shares > 0
+    return plan.tile_ctas == 0 and plan.n_waves >= 1 and plan.n_shares > 0
 
 
 @pytest.mark.parametrize("wl", [WIDE64, WIDE128], ids=lambda w: w.name)
@@ -50,7 +50,7 @@ def test_decode_in_whole_column_mode_every_row(oracle_mod, wl):
     nq = C * P
     saw_mode = 0
     worst = (0.0, 0.0)
-    for chunk in range(wl.n_chunks):
+    for chunk in range(wl.n_chunks + 2):                 # the first ones are short enough to go out otherwise
         q, k, v = synth.chunk_qkv(wl, chunk)
         dq, dk, dv = dev(q), dev(k), dev(v)
         q_out, q_guard = guarded(dq.shape)
@@ -124,7 +124,7 @@ def test_several_streams_in_whole_column_mode_every_row(oracle_mod):
         wants.append((want, guard))
         orc.close()
     plan = B.ll_debug_attn_plan_batched([(c.h, 0) for c in caches], 148)
-    assert plan.n_waves >= 3 and plan.n_shares > 0
+    assert plan.tile_ctas == 0 and plan.n_waves >= 3 and plan.n_shares > 0
     B.Cache.sink_window_attn_batched(items)
     for cache, item, (want, guard) in zip(caches, items, wants):
         cache.check_device()
@@ -227,16 +227,21 @@ def test_closed_form_histogram_of_eight_streams_in_one_launch():
         cache.close()
 
 
-@pytest.mark.parametrize("heads,dim,n_q,n_k", [(2, 128, 300, 1500),       # 4 columns of 12 steps, four or more parts each
-                                               (40, 128, 95, 662),        # 40 columns of 6 steps: whole
-                                               (1, 64, 129, 128 * 40),    # 1 column of 40 steps, many parts (batches of the merge)
-                                               (12, 128, 1479, 47 * 128 - 100),   # two equal parts per column, one odd
-                                               (5, 64, 2000, 700)])
-def test_columns_in_equal_parts(heads, dim, n_q, n_k):
+@pytest.mark.parametrize("heads,dim,n_q,n_k,plan", [
+    (2, 128, 300, 1500, (16, 16, 0)),                # 4 columns of 12 steps, four parts each
+    (40, 128, 95, 662, (40, 0, 0)),                  # 40 columns of 6 steps: whole
+    (1, 64, 129, 128 * 40, (8, 8, 0)),               # 1 column of 40 steps, many parts (batches of the merge)
+    (12, 128, 1479, 47 * 128 - 100, (144, 144, 0)),  # two equal parts per column, one odd
+    (40, 64, 95, 662, (40, 0, 0)),
+    (5, 64, 2000, 700, (40, 0, 80)),                 # 40 columns of 6 steps that go out by 128-row tiles instead
+])
+def test_columns_in_equal_parts(heads, dim, n_q, n_k, plan):
     """Fewer columns than SMs: every column in the same number of parts (or whole), against plain torch in 64 bits."""
     gen = torch.Generator(device="cuda").manual_seed(n_q)
     q, k, v = (torch.randn(n, heads, dim, device="cuda", generator=gen).to(torch.bfloat16) for n in (n_q, n_k, n_k))
     cache = B.Cache(1, heads, dim, 16, 1, 1, 1)
+    way = B.ll_debug_attn_plan_cross(cache.h, n_q, n_k, 148)
+    assert (way.n_ctas, way.n_shares, way.tile_ctas) == plan
     out, guard = guarded((n_q, heads, dim), fill=float("nan"))
     lse = torch.full((heads, n_q), float("nan"), device="cuda")
     for _ in range(2):                               # the second launch finds the first one's scratch and counters
