@@ -9,6 +9,8 @@
 // rows are fully coalesced.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "bounded_wait.cuh"
 #include "ll_internal.h"
 #include "ptx.cuh"
@@ -575,11 +577,11 @@ cudaError_t launch_norm_variant(const RopeAppendParams &p, const float *gain_q, 
 // begins a round and lose where they begin one of their own while it is still in its first; the longer the row, the more
 // a round of theirs gains.  us, streamed against not, buffers not in L2, 148 SMs, q too unless noted:
 //   5 heads of 128:   888 tokens 5.9 / 6.1, 2000 9.2 / 7.2, 4680 12.6 / 12.0, 7104 16.4 / 15.9
-//   8 heads:          888 tokens 6.7 / 7.0, 2000 10.5 / 8.9, 2516 11.0 / 10.6, 2960 11.2 / 12.3, 4680 14.7 / 16.1, 7104 19.9 / 21.8
+//   8 heads:         1184 tokens 7.1 / 7.3, 1776 8.5 / 8.2, 2000 10.5 / 8.9, 2516 11.0 / 10.6, 2960 11.2 / 12.3, 4680 14.7 / 16.1, 7104 19.9 / 21.8
 //   12 heads:        1479 tokens 9.4 / 9.9, 2368 13.2 / 11.8, 2516 13.3 / 16.1, 4680 18.8 / 21.0, 7104 27.5 / 28.5, 14400 52.0 / 48.9
 //   14 heads:         444 tokens 7.4 / 11.2, 2960 17.0 / 17.4, 4736 25.0 / 23.4
 //   16 heads:        1184 tokens 10.1 / 13.9, 4680 24.8 / 26.8, 14400 64.1 / 70.9; k and v alone 2960 14.5 / 15.1, 4736 18.9 / 18.7
-//   24 heads:        1184 tokens 15.2 / 18.9, 2368 27.1 / 25.4, 4736 42.8 / 41.7; k and v alone 1776 16.2 / 16.7, 2368 20.2 / 18.4
+//   24 heads:        1184 tokens 15.2 / 18.9, 2368 27.1 / 25.4, 4736 42.8 / 41.7; k and v alone 1924 16.3 / 17.3, 2368 20.2 / 18.4
 //   32 heads:        1184 tokens 18.6 / 24.1, 2368 31.3 / 35.4; k and v alone 1776 19.0 / 20.7, 2368 24.2 / 23.7
 //   k and v alone up to 8 heads: nothing to gain (8 heads, 888 tokens 5.7 / 5.6, 2368 8.8 / 7.3, 4736 11.8 / 11.9).
 // Heads of 64 go by the length of their rows as well (24 of 64 as 12 of 128, within 2 %).  Rows of up to 4 heads are too short (2 heads,
@@ -589,10 +591,10 @@ bool norm_append_streams(int heads, int head_dim, int n_tokens, bool with_q, int
     const int iters = (heads * (head_dim / 8) + 31) / 32;         // 16-byte vectors of a row per lane of a warp
     const int sms = sm_count > 0 ? sm_count : 148, each = (int)(((long long)n_tokens + sms - 1) / sms);
     if (iters <= 2 || iters > 16) return false;
-    if (iters <= 4) return with_q && (each <= 6 || (iters == 4 && each > 18 && each <= 48));
+    if (iters <= 4) return with_q && (each <= (iters == 3 ? 6 : 10) || (iters == 4 && each > 18 && each <= 48));
     if (iters <= 6) return each <= norm_stream_warps(heads, head_dim) || (each > 16 && each <= 48);
     if (iters <= 8) return each <= 24 || (iters == 8 && with_q);
-    return each <= (with_q ? 16 : 12);
+    return each <= (with_q ? 16 : std::min(16, 3 * norm_stream_warps(heads, head_dim)));
 }
 
 cudaError_t launch_norm_rope_append(const RopeAppendParams &p, int head_dim, const float *gain_q, const float *gain_k,

@@ -9,7 +9,7 @@ from paper_2509_22622_b200 import binding as B
     (4, 128, True, (), (1, 6, 12, 48)),
     (5, 128, True, (1, 6), (7, 13, 14, 16, 24, 32, 48)),
     (9, 64, True, (1, 6), (7, 14, 48)),
-    (8, 128, True, (1, 6, 19, 20, 32, 48), (7, 12, 14, 18, 49)),
+    (8, 128, True, (1, 10, 19, 20, 32, 48), (11, 12, 14, 18, 49)),
     (8, 128, False, (), (1, 6, 16, 20, 48)),
     (10, 128, True, (1, 12, 17, 48), (13, 16, 49)),
     (12, 128, True, (1, 11, 17, 32, 48), (12, 14, 16, 49, 98)),
@@ -18,7 +18,9 @@ from paper_2509_22622_b200 import binding as B
     (16, 128, True, (1, 24, 25, 98), ()),
     (16, 128, False, (1, 24), (25, 32)),
     (17, 128, True, (1, 16), (17, 32)),
-    (24, 128, False, (1, 12), (13, 16, 32)),
+    (17, 128, False, (1, 16), (17,)),
+    (24, 128, False, (1, 15), (16, 32)),
+    (32, 128, False, (1, 12), (13, 16)),
     (32, 128, True, (1, 16), (17,)),
     (33, 128, True, (), (1, 16, 48)),
 ])
