@@ -313,24 +313,44 @@ __host__ __device__ inline int norm_smem_bytes(int heads, int head_dim, int warp
     return norm_gain_bytes(heads, head_dim) + warps * (2 * norm_buffer_bytes(heads, head_dim) + 16) + 16;
 }
 
+// What a warp has of that.
+template <int D>
+struct NormStream {
+    float *gains;                                      // q, then k
+    uint8_t *own;                                      // its two buffers
+    volatile int *abort_flag;
+    uint32_t bars;                                     // and their barriers
+    __device__ NormStream(int heads, uint8_t *smem)
+    {
+        const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5, buffers = 2 * norm_buffer_bytes(heads, D);
+        gains = reinterpret_cast<float *>(smem);
+        own = smem + norm_gain_bytes(heads, D) + (size_t)warp * buffers;
+        bars = ptx::smem_u32(smem + norm_gain_bytes(heads, D) + (size_t)warps * buffers) + 16u * warp;
+        abort_flag = reinterpret_cast<volatile int *>(smem + norm_smem_bytes(heads, D, warps) - 16);
+    }
+    // no memory but shared: before the wait for the kernel in front
+    __device__ void init_barriers() const
+    {
+        if ((threadIdx.x & 31) < 2) ptx::mbar_init(bars + 8u * (threadIdx.x & 31), 1);
+        if (threadIdx.x == 0) *abort_flag = 0;
+        ptx::fence_mbar_init();
+    }
+};
+
 // The rows through shared memory: one persistent block per SM, two buffers per warp.
 template <int D>
-__device__ __forceinline__ void norm_rows_streamed(const RopeAppendParams &p, const float *gain_q, const float *gain_k, float eps)
+__device__ __forceinline__ void norm_rows_streamed(const RopeAppendParams &p, const float *gain_q, const float *gain_k, float eps,
+                                                   const NormStream<D> &stream)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
     constexpr int kVecs = D / 8, kBatch = 6;           // 16-byte vectors per head row; vectors per lane whose loads go out together
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int row_vecs = p.heads * kVecs, row_bytes = row_vecs * 16;
     const bool with_q = p.q_out != nullptr;
     const int vec = lane % kVecs;                      // the lane's vector inside every head row it meets
-    float *gains = reinterpret_cast<float *>(smem);    // q, then k
-    uint8_t *own = smem + norm_gain_bytes(p.heads, D) + (size_t)warp * 2 * (3 * row_bytes);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + norm_smem_bytes(p.heads, D, warps) - 16);
-    const uint32_t bars = ptx::smem_u32(smem + norm_gain_bytes(p.heads, D) + (size_t)warps * 2 * (3 * row_bytes)) + 16u * warp;
-    if (lane < 2) ptx::mbar_init(bars + 8u * lane, 1);
-    if (threadIdx.x == 0) *abort_flag = 0;
-    ptx::fence_mbar_init();
-    WaitCtx ctx{abort_flag, p.status, warp};
+    float *gains = stream.gains;
+    uint8_t *own = stream.own;
+    const uint32_t bars = stream.bars;
+    WaitCtx ctx{stream.abort_flag, p.status, warp};
     // tokens go round the blocks first, so that every SM gets its share of the last round
     const int first = blockIdx.x + gridDim.x * warp, stride = gridDim.x * warps;
     auto fetch = [&](int token, int buf) {             // lane 0: q, k and v row of a token
@@ -442,20 +462,23 @@ norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float 
     static_assert(32 % kVecs == 0, "a lane must meet the same rotation pairs in all its vectors");
     constexpr int kHeld = kIters > 0 ? kIters : 1;
     ptx::grid_dep_launch();
-    ptx::grid_dep_wait();
-    if constexpr (kIters == kStreamed) {
-        norm_rows_streamed<D>(p, gain_q, gain_k, eps);
-        return;
-    }
+    extern __shared__ __align__(128) uint8_t smem[];
+    const NormStream<D> stream(p.heads, smem);
     const int lane = threadIdx.x & 31;
     const long long token = (long long)blockIdx.x * (kNormThreads / 32) + (threadIdx.x >> 5);
-    if (token >= p.n_tokens) return;
+    if constexpr (kIters == kStreamed) stream.init_barriers();
+    else if (token >= p.n_tokens) return;
     const int row_vecs = p.heads * kVecs;
     const int frame = (int)(token / p.P);
     const int cell = (int)(token % p.P);
     const int y = cell / p.grid_w, x = cell % p.grid_w;
     const size_t in_base = (size_t)token * row_vecs * 8;
     const bool with_q = p.q_out != nullptr;
+    ptx::grid_dep_wait();
+    if constexpr (kIters == kStreamed) {
+        norm_rows_streamed<D>(p, gain_q, gain_k, eps, stream);
+        return;
+    }
     if ((unsigned)p.slot[frame] >= (unsigned)p.n_slots) {         // never with the host's slot rule: refuse, report
         record_status(p.status, kStatusBadRow, (uint32_t)p.slot[frame], (uint32_t)frame);
         return;

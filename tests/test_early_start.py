@@ -59,3 +59,9 @@ def test_other_kernels_start_the_ordinary_way(name):
 def test_no_read_only_loads(name):
     text = source(name)
     assert "__ldg(" not in text and "global.nc" not in text and "__restrict__" not in text
+
+
+@pytest.mark.parametrize("name", ["attn_sm100_kernel", "qkv_gemm_kernel", "bwd_dq_kernel", "bwd_dkdv_kernel", "norm_rope_append_kernel"])
+def test_barriers_are_set_up_before_the_wait(name):
+    body = ALL[name][1]
+    assert re.search(r"\b(mbar_init|init_barriers)\(", body[:body.index("grid_dep_wait()")])
