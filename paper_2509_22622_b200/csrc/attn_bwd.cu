@@ -173,16 +173,14 @@ __device__ __forceinline__ uint32_t lo_mnmajor(uint32_t tile) { return smem_desc
 __host__ __device__ constexpr uint32_t slice_kmajor(int kk) { return (uint32_t)(((kk / 4) * (128 * 128) + (kk % 4) * 32) >> 4); }
 __host__ __device__ constexpr uint32_t slice_mnmajor(int kk) { return (uint32_t)((kk * 2048) >> 4); }
 
-// Slices kBegin .. kEnd - 1 of D (+)= A B; kAMn / kBMn say which operand is MN-major.  The first
-// slice accumulates iff `acc_first`.
-template <int kBegin, int kEnd, bool kAMn, bool kBMn>
-__device__ __forceinline__ void mma_slices(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t acc_first)
+// D = A B over kSlices slices, both operands K-major in shared memory.
+template <int kSlices>
+__device__ __forceinline__ void mma_kmajor(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc)
 {
     constexpr uint32_t hi = smem_desc_hi_sw128(1024);
 #pragma unroll
-    for (int kk = kBegin; kk < kEnd; ++kk)
-        mma_ss(d, smem_desc_join(a_lo + (kAMn ? slice_mnmajor(kk) : slice_kmajor(kk)), hi),
-               smem_desc_join(b_lo + (kBMn ? slice_mnmajor(kk) : slice_kmajor(kk)), hi), idesc, kk > kBegin ? 1u : acc_first);
+    for (int kk = 0; kk < kSlices; ++kk)
+        mma_ss(d, smem_desc_join(a_lo + slice_kmajor(kk), hi), smem_desc_join(b_lo + slice_kmajor(kk), hi), idesc, kk > 0);
 }
 
 __device__ __forceinline__ void key_mask(int nvalid, uint32_t (&valid)[4])
@@ -606,7 +604,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                 if (!wait(kQFull + sl, j >> 1, j)) return false;
                 if (kOver && j > 0 && !wait(kDoEmpty + (sl ^ 1), (j - 1) >> 1, j)) return false;     // dV(j-1) has read P(j-1)
                 tc_fence_after_sync();
-                if (elected) mma_slices<0, D / 16, false, false>(t_s, k_k, lo_kmajor(q_s + sl * C::kTileBytes), idesc_s, 0u);
+                if (elected) mma_kmajor<D / 16>(t_s, k_k, lo_kmajor(q_s + sl * C::kTileBytes), idesc_s);
                 __syncwarp();
                 commit(kSFull);
                 return true;
@@ -616,7 +614,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                 if (!wait(kDoFull + sl, j >> 1, j)) return false;
                 if (kOver && j > 0 && !wait(kQEmpty + (sl ^ 1), (j - 1) >> 1, j)) return false;      // dK(j-1) has read dS(j-1)
                 tc_fence_after_sync();
-                if (elected) mma_slices<0, D / 16, false, false>(t_dp, v_k, lo_kmajor(do_s + sl * C::kTileBytes), idesc_s, 0u);
+                if (elected) mma_kmajor<D / 16>(t_dp, v_k, lo_kmajor(do_s + sl * C::kTileBytes), idesc_s);
                 __syncwarp();
                 commit(kDpFull);
                 return true;
