@@ -11,11 +11,11 @@
 //
 // Two kernels instead of one with atomics: every gradient element is accumulated by one CTA in one
 // order, so the result is run-to-run deterministic, at the price of forming S and dP twice.  Both
-// kernels have one warp that loads (TMA) and issues the MMAs (all its lanes walk the loop so that
-// descriptors are warp-uniform; one elected lane issues) and eight compute warps (one thread per
-// tile row and 64-key half, the 32x32b TMEM shape).  The compute warps take S into registers and
-// release its tensor memory at once, so the next step's S is formed while they are in the
-// exponentials; dP is read only for the last multiply.
+// kernels have one warp that issues the MMAs (all its lanes walk the loop so that descriptors are warp-uniform;
+// one elected lane issues) and eight compute warps (one thread per tile row and 64-column half, the 32x32b TMEM
+// shape).  The dq kernel's issuer also loads (TMA); its compute warps take S into registers and release its tensor
+// memory at once, so the next step's S is formed while they are in the exponentials.  The dk/dv kernel has a
+// load warp of its own, and forms the next S once P has been read.  dP is read only for the last multiply.
 //   What they compute goes back to tensor memory as the A operand of the products that follow: dS over dP, and in
 // the dk/dv kernel P over S (at head_dim 64 beside them, where columns are left).  Through shared memory those tiles
 // cost a store and a read of 32 KB each beside operands of 64 KB per 512 clk of products.

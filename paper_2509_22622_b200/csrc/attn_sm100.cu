@@ -9,7 +9,9 @@
 // each K/V tile is fetched from HBM once and shared through L2.  The steps of the
 // columns left over are laid end to end and cut into one share per CTA, sized on
 // the host so that every SM ends up with the same number of steps whatever the
-// number and length of the columns (very short columns go out whole instead).
+// number and length of the columns (very short columns go out whole instead).  Equally long
+// columns may also go out by their 128-row tiles, every CTA as many as any other or one more, two of one head at a
+// time as a column and what is left over alone (AttnParams::tile_ctas); then nothing is split.
 // A column whose steps fall into several CTAs is finished by whichever of them
 // arrives last:
 // every part leaves its unnormalised O rows, reference maxima and sums in a
@@ -33,8 +35,8 @@
 //   P does not go back over S: a lane's S buffer is free as soon as its softmax
 //   warps hold the tile in registers, so the MMA warp issues QK of step j+1 while
 //   the softmax of step j is still running, and the softmax warps find the next S
-//   waiting.  The tensor pipe then sees, per lane and step, PV(first half), QK(next),
-//   PV(second half), whenever their inputs arrive.  A share of the exponentials can be
+//   waiting.  The tensor pipe then sees, per lane and step, QK of the next step and
+//   PV of this one, whenever their inputs arrive.  A share of the exponentials can be
 //   evaluated with a cubic on the FMA pipe instead of the special-function unit
 //   (kPolyMask: none at head_dim 128, a quarter at head_dim 64, as measured).
 //
@@ -106,8 +108,8 @@ struct Cfg {
     static constexpr int kColP = 384;                       // P_w at kColP + 64 w (kPInTmem; two keys per column)
     // A move of the references rescales the O rows behind the piece's P instead of in front of it: then the piece's registers
     // are free and all loads of a row go out together (eight streams with outliers, which move in every fourth piece:
-    // 3750 -> 3512 us; the benchmark layer's decode, which hardly moves, 478 -> 473 us).  In chunks of 64 columns with 104 registers
-    // the decode took 507 us; at head_dim 64, whose loop has no registers to spare, 742 instead of 702 us.
+    // 3750 -> 3512 us; the benchmark layer's decode, which hardly moves, 473 us, the same within what runs differ).  In chunks of 64
+    // columns with 104 registers the decode took 507 us; at head_dim 64, whose loop has no registers to spare, 742 instead of 702 us.
     static constexpr bool kRescaleLate = D == 128;
     static constexpr int kOChunks = D / 64;                 // 64-column pieces of an O row
 };

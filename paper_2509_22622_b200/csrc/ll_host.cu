@@ -463,12 +463,15 @@ double plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_s
 // more, two of a head at a time (a column) and what is left over alone.  A tile alone takes about 0.7 of a column's time, 0.76 at
 // head_dim 64 (its steps wait on one chain of products and weights instead of two), nothing is split and nothing merged.  By tiles when the
 // busiest CTA is then done earlier: 4680 queries over 512 keys, 12 heads of 128, are 228 columns, two on 80 of 148 SMs,
-// or 444 tiles, three on each (26.7 -> 24.1 us); 390 over 512, 12 heads, 24 columns or 48 tiles (14.9 -> 11.7 us); 1100 over
+// or 444 tiles, three on each (25.8 -> 22.2 us); 390 over 512, 12 heads, 24 columns or 48 tiles (14.9 -> 11.7 us); 1100 over
 // 1500, 8 heads, 40 columns in three parts or 72 tiles (29 -> 22 us); 1000 over 1000, 40 heads, 148 columns whole and 12 shared or
 // 320 tiles (43.3 -> 31.6 us); 4680 over 2000 / 3000 / 4096, 12 heads, 148 whole and 80 shared or 444 tiles (70.5 -> 60.8, 95.5
 // -> 87.9, 118.7 -> 114.0 us).  Past the line: 1479 over 5916, 12 heads, 72 columns in two parts 59.1 us, 144 tiles 61.2 us.
-// At head_dim 64, 12 heads: 4680 over 512 / 2000 / 3000 18.9 -> 16.9, 52.7 -> 45.5, 69.5 -> 66.5 us; past the line 4680 over 4096
-// 84.8 us in shares, 85.4 by tiles.
+// At head_dim 64, 12 heads: 4680 over 512 / 2000 18.9 -> 16.9, 52.7 -> 45.5 us; past the line 4680 over 3000 / 4096 69.5 / 84.8 us in
+// shares, 66.5 / 85.4 by tiles.
+//   kGain: by tiles must look 5 % cheaper, which is what the two estimates are good for.  Of 120 drawn launches whose estimates lie within
+// 0.8 and 1.1 of each other, the 48 below 0.95 take 0.64 to 1.01 of the time by tiles (0.87 in the geometric mean); from there on
+// it goes both ways: 0.81 to 1.09 up to 0.975, 0.70 to 1.11 near 1, 0.73 to 1.14 above 1.05.
 void plan_tiles(ll::AttnParams *p, int sms, double cost, int head_dim)
 {
     constexpr double kGain = 0.95;

@@ -64,7 +64,8 @@ struct LayerState {
 // same number of steps (whole columns of groups with different key counts
 // weigh differently).  When the columns are so short that merging the parts of a
 // split column would cost more than it saves, the last columns go out whole as
-// a partial wave instead and nothing is shared.
+// a partial wave instead and nothing is shared.  Equally long columns may go out by
+// 128-row tiles instead of all this (AttnParams::tile_ctas).
 struct AttnGroup {
     int item;                         // which (cache, layer, q, out) of the launch the group belongs to
     int q_begin;                      // first query row of the group in its item's q tensor

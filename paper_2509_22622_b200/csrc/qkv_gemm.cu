@@ -376,7 +376,9 @@ done:
 __global__ void __launch_bounds__(256)
 qkv_finish_kernel(const __grid_constant__ QkvParams p)
 {
-    constexpr int kHeld = 3;                           // (with 6 an SM holds 24 warps instead of 40: 1 us more for 4680 tokens of 1536)
+    // (3, 4 and 6 are the same within what runs differ, 1 to 3 %: the projection with norm of 4680 tokens, widths 1536 / 2048 / 3072 / 5120,
+    // 72.4 / 146.3 / 297.8 / 772.8 us with 3, 75.1 / 146.8 / 298.2 / 774.9 with 6)
+    constexpr int kHeld = 3;
     const int token = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     grid_dep_launch();
     grid_dep_wait();
