@@ -27,7 +27,7 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // is still running.  It calls grid_dep_launch() early, which lets the kernel behind it do the same once all its
 // blocks have started, and grid_dep_wait() before its first access to global memory: that returns when the
 // kernels before it have completed and their writes are visible.  What can be done without memory (barriers,
-// tensor memory, index arithmetic) comes before the wait.  rope_q_static_kernel, attn_simt_kernel and
+// tensor memory, index arithmetic where it pays) comes before the wait.  rope_q_static_kernel, attn_simt_kernel and
 // wait_probe_kernel have neither call and are launched the ordinary way.
 //   What such a kernel reads behind the wait may have been written during its own lifetime, so it is read with
 // ordinary loads: ld.global.nc (__ldg, or what the compiler makes of a const __restrict__ pointer) is for

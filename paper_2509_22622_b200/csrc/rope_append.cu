@@ -464,21 +464,23 @@ norm_rope_append_kernel(const __grid_constant__ RopeAppendParams p, const float 
     ptx::grid_dep_launch();
     extern __shared__ __align__(128) uint8_t smem[];
     const NormStream<D> stream(p.heads, smem);
+    if constexpr (kIters == kStreamed) stream.init_barriers();
+    // The index arithmetic stays behind the wait.  In front of it, append and attention of 1 head of 64, 1188 tokens, take 19.97 us
+    // instead of 19.80 in a stream, 23.46 instead of 23.60 in a replayed graph; 6 heads, 240 tokens, 10.33 / 10.28 and 13.28 / 13.38.
+    ptx::grid_dep_wait();
+    if constexpr (kIters == kStreamed) {
+        norm_rows_streamed<D>(p, gain_q, gain_k, eps, stream);
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const long long token = (long long)blockIdx.x * (kNormThreads / 32) + (threadIdx.x >> 5);
-    if constexpr (kIters == kStreamed) stream.init_barriers();
-    else if (token >= p.n_tokens) return;
+    if (token >= p.n_tokens) return;
     const int row_vecs = p.heads * kVecs;
     const int frame = (int)(token / p.P);
     const int cell = (int)(token % p.P);
     const int y = cell / p.grid_w, x = cell % p.grid_w;
     const size_t in_base = (size_t)token * row_vecs * 8;
     const bool with_q = p.q_out != nullptr;
-    ptx::grid_dep_wait();
-    if constexpr (kIters == kStreamed) {
-        norm_rows_streamed<D>(p, gain_q, gain_k, eps, stream);
-        return;
-    }
     if ((unsigned)p.slot[frame] >= (unsigned)p.n_slots) {         // never with the host's slot rule: refuse, report
         record_status(p.status, kStatusBadRow, (uint32_t)p.slot[frame], (uint32_t)frame);
         return;
