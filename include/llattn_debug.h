@@ -51,6 +51,8 @@ int ll_debug_wait_timeout(ll_cache *cache, int limit_ms, ll_stream stream);
  * above is then not used, and tile_ctas, otherwise 0, is the number of CTAs: the row_tiles[g] tiles of a group's heads are
  * numbered one after the other, group after group, and CTA i takes tiles_each consecutive ones, one more when
  * i < tiles_extra, two of one head at a time.
+ * cluster_parts, otherwise 0, is the number of equal parts that every column comes in when the CTAs holding them are a cluster
+ * and merge them together (n_shares = n_ctas then, and CTA i takes share i).
  * ll_debug_attn_plan_batched: the same for ll_sink_window_attn_batched of the
  * newest chunk of every item (only cache and layer of an item are read).
  * ll_debug_attn_plan_clip: for ll_clip_append_attn (and its backward), of the newest n_frames frames.
@@ -76,6 +78,7 @@ typedef struct ll_attn_plan {
     int32_t tiles_each;
     int32_t tiles_extra;
     int32_t row_tiles[LL_MAX_GROUPS];
+    int32_t cluster_parts;
 } ll_attn_plan;
 int ll_debug_attn_plan(ll_cache *cache, int layer, int recache, int sm_count, ll_attn_plan *out);
 int ll_debug_attn_plan_batched(const ll_attn_item *items, int n_items, int sm_count, ll_attn_plan *out);

@@ -66,6 +66,7 @@ class ll_attn_plan(C.Structure):
         ("tiles_each", C.c_int32),
         ("tiles_extra", C.c_int32),
         ("row_tiles", C.c_int32 * LL_MAX_GROUPS),
+        ("cluster_parts", C.c_int32),
     ]
 
 

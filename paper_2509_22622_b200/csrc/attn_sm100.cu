@@ -16,7 +16,9 @@
 // arrives last:
 // every part leaves its unnormalised O rows, reference maxima and sums in a
 // scratch slot, bumps the column's arrival counter, and the last one merges the
-// parts and writes the output.  Nothing waits on another CTA.
+// parts and writes the output.  Nothing waits on another CTA.  Columns in up to eight equal parts are held by the
+// CTAs of a cluster (AttnParams::cluster_parts), which run at the same time, wait for one another and merge a share of the
+// head's columns each (merge_in_cluster).
 //
 // Inside a CTA (640 threads):
 //   warp 16 (one lane)  TMA producer: the column's Q tiles, then K_j V_j K_j+1 ...
@@ -117,8 +119,13 @@ struct Cfg {
 // barrier indices inside the shared barrier array (+ lane or + stage)
 enum Bar {
     kQFull = 0, kQEmpty = 2, kSFull = 4, kSEmpty = 6, kPFull = 8, kPEmpty = 10, kOFull = 12, kOEmpty = 14,
-    kKvFull = 16, kKvEmpty = 24, kNumBars = 32
+    kKvFull = 16, kKvEmpty = 24, kNumBars = 32,
+    kPartFull = 32, kNumBarsParts = kPartFull + kSlabs      // kFormParts: the other parts' rows of a slab are in their slots
 };
+
+// Which launches an instance of the kernel serves.  At head_dim 128 one serves columns and tiles; at 64, whose loop has no registers
+// to spare, the code for tiles costs the others 0.7 % (698 -> 703 us, 24 heads of 64 on the benchmark grid).
+enum Form { kFormColumns, kFormTiles /* columns too */, kFormParts /* AttnParams::cluster_parts */ };
 
 // Walks the visible key tiles of a group: runs in order, 128 rows at a time.
 struct KeyIter {
@@ -152,16 +159,17 @@ struct Segment {
 
 // A CTA's work in order: its whole columns, wave by wave, then its share of the steps
 // that are left.  Every role of the CTA walks the same sequence.
-// kTiles: also by 128-row tiles (AttnParams::tile_ctas).
-template <bool kTiles>
+template <int kForm>
 struct WorkIter {
+    static constexpr bool kTiles = kForm == kFormTiles;
     const AttnParams &p;
     int cta, g, wave, share;
     int u, end;
     __device__ WorkIter(const AttnParams &prm, int cta_)
-        : p(prm), cta(cta_), g(0), wave(0), share(prm.share_of_cta[cta_]), u(0), end(0)
+        : p(prm), cta(cta_), g(0), wave(0), share(kForm == kFormParts ? cta_ : prm.share_of_cta[cta_]), u(0), end(0)
     {
-        if (kTiles && p.tile_ctas > 0) {
+        if (kForm == kFormParts) {
+        } else if (kTiles && p.tile_ctas > 0) {
             u = cta * p.tiles_each + min(cta, p.tiles_extra);
             end = u + p.tiles_each + (cta < p.tiles_extra ? 1 : 0);
         } else if (share >= 0) {
@@ -183,6 +191,15 @@ struct WorkIter {
     }
     __device__ bool next(Segment &s)
     {
+        if (kForm == kFormParts) {                       // share `cta`, from its definition: the n-th part of a column
+            if (wave++ > 0) return false;
+            const int n = p.cluster_parts, col = cta / n, i = cta - col * n;
+            while (col >= p.g[g].col_begin + p.heads * p.g[g].tiles) ++g;
+            const AttnGroup &G = p.g[g];
+            fill(s, g, col - G.col_begin, i * G.n_kt / n, (i + 1) * G.n_kt / n);
+            s.col_begin = 0;
+            return true;
+        }
         if (kTiles && p.tile_ctas > 0) {
             if (u >= end) return false;
             while (u >= p.g[g].tile_begin + p.heads * p.g[g].row_tiles) ++g;
@@ -426,9 +443,138 @@ __device__ __forceinline__ void merge_column(const AttnParams &p, const Segment 
     __syncwarp();                                      // the P rows are read before another column's are staged
 }
 
-// kTiles: whether it serves launches by 128-row tiles.  At head_dim 128 one kernel serves both; at 64, whose loop has no registers
-// to spare, the code for them costs the others 0.7 % (698 -> 703 us, 24 heads of 64 on the benchmark grid).
-template <int D, bool kTiles>
+// The parts of a column that the CTAs of a cluster hold, merged for the warp's 16 rows.  Every CTA leaves what the others merge of
+// its unnormalised rows in its scratch slot, tells the same warp of each of them, and merges an n-th of the columns itself: those
+// of the 8-column groups k with k n / (D / 8) == its rank.  All SMs of the cluster then read and write (n - 1) / n of a part, where the one
+// that arrives last reads back all parts: from the last product to the end 5 us for two parts of 256 rows where that takes 8
+// (12 heads of 128, 1479 queries over 5916 keys; 450 over 2250, 8 heads: 24.6 us a call in four parts, 17.5 in six).  Through the cluster's shared memory the same exchange is slower (64 KB
+// each way 4100 clk to send for two CTAs, 7800 for four; to L2 2900 and 3500), so only the barriers are there.
+//   kPeers and kUnroll: other parts that x has room for, and groups at a time, so that about eight to fourteen loads are in flight.
+template <int D, int kPeers, int kUnroll>
+__device__ __forceinline__ void merge_groups(const AttnParams &p, const WarpRows &wr, int cta, int rank, int n, int g0, int g1, uint32_t t_o,
+                                             float v_scale, uint32_t stage, float &m_a, float &m_b, float &l_a, float &l_b)
+{
+    constexpr int kGroups = D / 8;
+    constexpr size_t kSlotFloats = (size_t)kQTileRows * (D + 2);
+    const int lane = wr.lane, slab = wr.slab();
+    // of the j-th peer (part j below this CTA's rank, part j + 1 from there on)
+    auto slot = [&](int j) { return p.partial + (size_t)2 * (cta - rank + j + (j >= rank ? 1 : 0)) * kSlotFloats; };
+    float4 x[kPeers][kUnroll];                         // of each group this thread's two columns of row a, then of row a + 8
+    auto load_groups = [&](int k0) {
+#pragma unroll
+        for (int j = 0; j < kPeers; ++j) {
+            const float4 *src = reinterpret_cast<const float4 *>(slot(j)) + (size_t)(slab * kGroups + k0) * 32 + lane;
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u)
+                x[j][u] = (j < n - 1 && k0 + u < g1) ? __ldcg(src + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    float2 ra[kPeers], rb[kPeers];                     // (reference, sum), rows a and a + 8
+#pragma unroll
+    for (int j = 0; j < kPeers; ++j) {
+        const float2 *ml = reinterpret_cast<const float2 *>(slot(j) + (size_t)kQTileRows * D) + slab * 16 + (lane >> 2);
+        ra[j] = j < n - 1 ? __ldcg(ml) : make_float2(-INFINITY, 0.f);
+        rb[j] = j < n - 1 ? __ldcg(ml + 8) : make_float2(-INFINITY, 0.f);
+    }
+    constexpr bool kAhead = kPeers <= 3;               // the first groups are in flight with them (with more the registers do not suffice)
+    if (kAhead) load_groups(g0);
+    const float own_a = m_a, own_b = m_b;
+#pragma unroll
+    for (int j = 0; j < kPeers; ++j) {
+        m_a = fmaxf(m_a, ra[j].x);
+        m_b = fmaxf(m_b, rb[j].x);
+    }
+    float w_a = ex2(own_a - m_a), w_b = ex2(own_b - m_b);
+    l_a *= w_a;
+    l_b *= w_b;
+#pragma unroll
+    for (int j = 0; j < kPeers; ++j) {                 // from here on .x is the part's weight (0 behind the last)
+        ra[j].x = ex2(ra[j].x - m_a);
+        rb[j].x = ex2(rb[j].x - m_b);
+        l_a = fmaf(ra[j].y, ra[j].x, l_a);
+        l_b = fmaf(rb[j].y, rb[j].x, l_b);
+    }
+    const float inv_a = v_scale / l_a, inv_b = v_scale / l_b;
+    w_a *= inv_a;
+    w_b *= inv_b;
+#pragma unroll
+    for (int j = 0; j < kPeers; ++j) {
+        ra[j].x *= inv_a;
+        rb[j].x *= inv_b;
+    }
+#pragma unroll 1
+    for (int k0 = g0; k0 < g1; k0 += kUnroll) {
+        if (!kAhead || k0 > g0) load_groups(k0);
+        uint32_t own[4 * kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u)
+            tmem_ld_16x256b_x1(t_o + 8 * min(k0 + u, kGroups - 1), own[4 * u], own[4 * u + 1], own[4 * u + 2], own[4 * u + 3]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            float4 o = make_float4(as_f(own[4 * u]) * w_a, as_f(own[4 * u + 1]) * w_a, as_f(own[4 * u + 2]) * w_b, as_f(own[4 * u + 3]) * w_b);
+#pragma unroll
+            for (int j = 0; j < kPeers; ++j) {
+                o.x = fmaf(x[j][u].x, ra[j].x, o.x);
+                o.y = fmaf(x[j][u].y, ra[j].x, o.y);
+                o.z = fmaf(x[j][u].z, rb[j].x, o.z);
+                o.w = fmaf(x[j][u].w, rb[j].x, o.w);
+            }
+            const int k = k0 + u;
+            if (k < g1)
+                stmatrix_x2(stage + (k >> 3) * Cfg<D>::kAtomBytes + (((uint32_t)k ^ lane) & 7u) * 16, cvt_bf16x2(o.x, o.y), cvt_bf16x2(o.z, o.w));
+        }
+    }
+}
+
+template <int D, class Wait>
+__device__ __forceinline__ bool merge_in_cluster(const AttnParams &p, const Segment &s, const WarpRows &wr, int cta, uint32_t t_o, float m_own_a,
+                                                 float m_own_b, float l_own_a, float l_own_b, uint32_t p_smem, uint32_t part_bar, Wait wait)
+{
+    using C = Cfg<D>;
+    constexpr int kGroups = D / 8;
+    const int n = p.cluster_parts, rank = (int)cluster_rank(), lane = wr.lane, slab = wr.slab();
+    const int g0 = (rank * kGroups + n - 1) / n, g1 = ((rank + 1) * kGroups + n - 1) / n;
+    float *slot = p.partial + (size_t)2 * cta * kQTileRows * (D + 2);
+#pragma unroll 1
+    for (int ch = 0; ch < C::kOChunks; ++ch) {
+        uint32_t o[32];
+        tmem_ld_16x256b_x8(t_o + 64 * ch, o);
+        tmem_wait_ld();
+        uint4 *dst = reinterpret_cast<uint4 *>(slot) + (size_t)(slab * kGroups + 8 * ch) * 32 + lane;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (8 * ch + k < g0 || 8 * ch + k >= g1) dst[32 * k] = make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+    }
+    if ((lane & 3) == 0) {
+        float2 *ml = reinterpret_cast<float2 *>(slot + (size_t)kQTileRows * D) + slab * 16 + (lane >> 2);
+        ml[0] = make_float2(m_own_a, l_own_a);
+        ml[8] = make_float2(m_own_b, l_own_b);
+    }
+    fence_cluster();
+    __syncwarp();
+    if (lane < n && lane != rank) mbar_arrive_remote(part_bar, (uint32_t)lane);
+    if (!__all_sync(0xffffffffu, wait())) return false;
+    const AttnItem &item = p.item[p.g[s.g].item];
+    const float v_scale = item.v_scale ? item.v_scale[s.head] : 1.f;   // 8-bit caches: value codes x scale
+    // the merged rows wait in the lane's P tile (its last PV has completed; every warp uses its own 16 rows) for 16-byte stores
+    const uint32_t tile = p_smem + wr.w * C::kPBytes, stage = tile + (uint32_t)(wr.first() + (lane & 15)) * 128;
+    float m_a = m_own_a, m_b = m_own_b, l_a = l_own_a, l_b = l_own_b;
+    if (n == 2) merge_groups<D, 1, 8>(p, wr, cta, rank, n, g0, g1, t_o, v_scale, stage, m_a, m_b, l_a, l_b);
+    else if (n <= 4) merge_groups<D, 3, 4>(p, wr, cta, rank, n, g0, g1, t_o, v_scale, stage, m_a, m_b, l_a, l_b);
+    else merge_groups<D, 7, 2>(p, wr, cta, rank, n, g0, g1, t_o, v_scale, stage, m_a, m_b, l_a, l_b);
+    __syncwarp();
+    const int groups = g1 - g0, inv = (65536 + groups - 1) / groups;           // i / groups = i inv / 65536 for i below 128
+    for (int i = lane; i < 16 * groups; i += 32) {
+        const int r = (i * inv) >> 16, k = g0 + i - r * groups, row = 128 * wr.w + wr.first() + r;
+        const uint4 v = ld_shared_v4(tile + (k >> 3) * C::kAtomBytes + (uint32_t)(wr.first() + r) * 128 + ((uint32_t)((k ^ r) & 7) << 4));
+        if (row < s.rows_valid) *reinterpret_cast<uint4 *>(item.out + ((size_t)(s.q0 + row) * p.heads + s.head) * D + 8 * k) = v;
+    }
+    if (rank == 0) store_lse(item, s, wr, m_a, m_b, l_a, l_b);
+    return true;
+}
+
+template <int D, int kForm>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMaps maps)
 {
@@ -440,7 +586,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
     const uint32_t p_smem = smem_base + 2 * C::kTileBytes;              // one 64-key P tile per lane
     const uint32_t kv_smem = p_smem + 2 * C::kPBytes;                   // kStages tiles
     const uint32_t bars = smem_base + C::kSmemTiles;                    // kNumBars x 8 bytes
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_gen + C::kSmemTiles + kNumBars * 8);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_gen + C::kSmemTiles + kNumBarsParts * 8);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
 
@@ -452,7 +598,9 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
 
     // ---- setup ------------------------------------------------------------------
     grid_dep_launch();
+    constexpr bool kParts = kForm == kFormParts;
     if (threadIdx.x == 0) {
+#pragma unroll
         for (int i = 0; i < kNumBars; ++i) {
             uint32_t count = 1;
             if ((i >= kSEmpty && i < kSEmpty + 2) || (i >= kPFull && i < kPFull + 2) || (i >= kOEmpty && i < kOEmpty + 2))
@@ -460,8 +608,11 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
             if (i == kQEmpty || i >= kKvEmpty) count = 2;                      // both MMA warps release Q and every K/V stage
             mbar_init(bar(i), count);
         }
+        if (kParts)
+            for (int i = 0; i < kSlabs; ++i) mbar_init(bar(kPartFull + i), p.cluster_parts - 1);     // the same warp of every other CTA of the cluster
         fence_mbar_init();
     }
+    if (kParts) cluster_arrive();
     if (warp == kTmaWarp) {
         tmem_alloc(smem_u32(tmem_slot), C::kTmemCols);
         tmem_relinquish();
@@ -469,6 +620,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
     grid_dep_wait();
     // an earlier CTA already gave up on a wait: this one does not start (flag value 2)
     if (threadIdx.x == 0) *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
+    if (kParts) cluster_wait();                        // every CTA of the cluster has its barriers
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -497,11 +649,12 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 uint32_t n = 0;                 // K/V tiles issued so far
                 uint32_t seg = 0;
                 Segment s;
-                for (WorkIter<kTiles> it(p, cta); it.next(s); ++seg) {
+                for (WorkIter<kForm> it(p, cta); it.next(s); ++seg) {
                     // Tile order K_0, K_1, V_0, K_2, V_1, ... : the QK of a step is issued a whole
                     // softmax ahead of the step's PV, so K runs one step ahead of V and three stages
                     // (the V in use, the K in use, one in flight) keep both fed.
-                    KeyIter kit_k(&p.g[s.g], s.kt0), kit_v(&p.g[s.g], s.kt0);
+                    KeyIter kit(&p.g[s.g], s.kt0);
+                    int row = kit.row();
                     const int item = p.g[s.g].item;
                     const CUtensorMap *qmap = &maps.q[item], *kmap = &maps.k[item], *vmap = &maps.v[item];
                     auto load_kv = [&](const CUtensorMap *m, int row) -> bool {
@@ -517,7 +670,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                     };
                     // the first key tile goes out before Q: it needs no Q buffer and is in
                     // flight while the previous column's last products drain
-                    if (!load_kv(kmap, kit_k.row())) return;
+                    if (!load_kv(kmap, row)) return;
                     if (seg > 0 && !wait(kQEmpty, seg - 1, (int)seg)) return;
                     for (int w = 0; w < s.n_sub; ++w) {
                         mbar_arrive_expect_tx(bar(kQFull + w), C::kTileBytes);
@@ -526,12 +679,13 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                                         a * 64, s.head, s.q0 + 128 * w);
                     }
                     for (int j = s.kt0; j < s.kt1; ++j) {
+                        const int v_row = row;
                         if (j + 1 < s.kt1) {
-                            kit_k.next();
-                            if (!load_kv(kmap, kit_k.row())) return;
+                            kit.next();
+                            row = kit.row();
+                            if (!load_kv(kmap, row)) return;
                         }
-                        if (!load_kv(vmap, kit_v.row())) return;
-                        kit_v.next();
+                        if (!load_kv(vmap, v_row)) return;
                     }
                 }
             }();
@@ -588,7 +742,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 uint32_t oc = 0;                // columns this lane took part in so far
                 uint32_t seg = 0;
                 Segment s;
-                for (WorkIter<kTiles> it(p, cta); it.next(s); ++seg) {
+                for (WorkIter<kForm> it(p, cta); it.next(s); ++seg) {
                     const int n_steps = s.kt1 - s.kt0;
                     if (w >= s.n_sub) {
                         // not this lane's column: pass every stage on once its tile has landed, and
@@ -661,7 +815,7 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
             constexpr bool kMergeLate = D == 64;
             uint32_t to_merge = 0;                             // which of the CTA's two parts complete a column here
             Segment s;
-            for (WorkIter<kTiles> it(p, cta); it.next(s);) {
+            for (WorkIter<kForm> it(p, cta); it.next(s);) {
                 if (w >= s.n_sub) continue;
                 const AttnGroup &G = p.g[s.g];
                 // keys left in the current run of the visible set (its last tile may be ragged)
@@ -900,7 +1054,12 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                     l_b += __shfl_xor_sync(0xffffffffu, l_b, 2);
                 }
                 const AttnItem &item = p.item[G.item];
-                if (s.kt0 == 0 && s.kt1 == G.n_kt) {
+                if constexpr (kParts) {
+                    const int part_bar = kPartFull + wr.slab();
+                    if (!merge_in_cluster<D>(p, s, wr, cta, t_o, m_a, m_b, l_a, l_b, p_smem, bar(part_bar),
+                                             [&]() { return wait_bar<true>(bar(part_bar), 0, ctx, part_bar, s.kt1); }))
+                        return;
+                } else if (s.kt0 == 0 && s.kt1 == G.n_kt) {
                     // a whole column: normalise and store
                     const float v_scale = item.v_scale ? item.v_scale[s.head] : 1.f;   // 8-bit caches: value codes x scale
                     const float inv_a = v_scale / l_a, inv_b = v_scale / l_b;
@@ -966,10 +1125,10 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 if (lane == 0) mbar_arrive(bar(kOEmpty + w));
                 ++oc;
             }
-            if (kMergeLate && to_merge) {
+            if (!kParts && kMergeLate && to_merge) {
                 __threadfence();                                   // the other parts' slots, seen complete above
                 const int own = p.share_of_cta[cta];
-                for (WorkIter<kTiles> it(p, cta); it.next(s);) {
+                for (WorkIter<kForm> it(p, cta); it.next(s);) {
                     if (w >= s.n_sub || (s.kt0 == 0 && s.kt1 == p.g[s.g].n_kt)) continue;
                     if ((to_merge >> (s.kt0 == 0 ? 1 : 0)) & 1u) merge_column<D>(p, s, own, wr, p_smem, p_at);
                 }
@@ -985,6 +1144,14 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
         // shared and tensor memory go back to the SM
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
+        __syncthreads();
+    }
+    if (kParts && *abort_flag != 0) {
+        // Every warp that merges has waited for the others' arrivals at its barrier.  A CTA that gave up, or did not start, stays until they have
+        // come, or as long as the others may take to give up themselves.
+        const uint64_t t0 = globaltimer_ns(), limit = *abort_flag == 1 ? 2 * kWaitLimitNs : 50000000ull;
+        if (warp < kSlabs && lane == 0)
+            while (!mbar_try_wait_cluster(bar(kPartFull + warp), 0) && globaltimer_ns() - t0 < limit) __nanosleep(1000);
         __syncthreads();
     }
     if (warp == kTmaWarp) {
@@ -1021,7 +1188,7 @@ cudaError_t launch_wait_probe(uint32_t *status, uint64_t limit_ns, cudaStream_t 
 
 namespace {
 
-template <int D, bool kTiles>
+template <int D, int kForm>
 cudaError_t launch_instance(const AttnParams &p, const AttnMaps &maps, dim3 grid, bool early, cudaStream_t stream)
 {
     // Once per device: the in-kernel register reallocation assumes the launch
@@ -1033,14 +1200,15 @@ cudaError_t launch_instance(const AttnParams &p, const AttnMaps &maps, dim3 grid
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices || !prepared[dev].load(std::memory_order_acquire)) {
         cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, attn_sm100_kernel<D, kTiles>);
+        e = cudaFuncGetAttributes(&fa, attn_sm100_kernel<D, kForm>);
         if (e != cudaSuccess) return e;
         if (fa.numRegs != kLaunchRegs) return cudaErrorLaunchOutOfResources;
-        e = cudaFuncSetAttribute(attn_sm100_kernel<D, kTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
+        e = cudaFuncSetAttribute(attn_sm100_kernel<D, kForm>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < kMaxDevices) prepared[dev].store(1, std::memory_order_release);
     }
-    return launch_dependent(early, attn_sm100_kernel<D, kTiles>, grid, kThreads, Cfg<D>::kSmemBytes, stream, p, maps);
+    return launch_dependent(early, -1, kForm == kFormParts ? p.cluster_parts : 1, attn_sm100_kernel<D, kForm>, grid, kThreads, Cfg<D>::kSmemBytes,
+                            stream, p, maps);
 }
 
 }  // namespace
@@ -1053,9 +1221,11 @@ cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps 
     long long steps = 0;
     for (int g = 0; g < p.n_groups; ++g) steps += (long long)p.heads * p.g[g].tiles * p.g[g].n_kt;
     const bool early = steps <= kEarlySteps * p.n_ctas;
-    if (head_dim == 128) e = launch_instance<128, true>(p, maps, grid, early, stream);
-    else if (p.tile_ctas > 0) e = launch_instance<64, true>(p, maps, grid, early, stream);
-    else e = launch_instance<64, false>(p, maps, grid, early, stream);
+    if (p.cluster_parts > 0)
+        e = head_dim == 128 ? launch_instance<128, kFormParts>(p, maps, grid, early, stream) : launch_instance<64, kFormParts>(p, maps, grid, early, stream);
+    else if (head_dim == 128) e = launch_instance<128, kFormTiles>(p, maps, grid, early, stream);
+    else if (p.tile_ctas > 0) e = launch_instance<64, kFormTiles>(p, maps, grid, early, stream);
+    else e = launch_instance<64, kFormColumns>(p, maps, grid, early, stream);
     count_launch();
     return e;
 }

@@ -20,7 +20,8 @@ struct WaitCtx {
     int role;                     // who is waiting (the warp index)
 };
 
-// Returns false when the CTA is aborting.
+// Returns false when the CTA is aborting.  kCluster: other CTAs of the cluster arrive at the barrier too.
+template <bool kCluster = false>
 __device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, const WaitCtx &ctx, int bar_id, int iter,
                                           uint64_t limit_ns = kWaitLimitNs)
 {
@@ -28,7 +29,7 @@ __device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, const W
     const uint64_t t0 = globaltimer_ns();
     uint32_t spins = 0;
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
         if ((++spins & 63u) == 0) {
             if (*ctx.abort_flag) return false;
             if (globaltimer_ns() - t0 > limit_ns) {
@@ -46,11 +47,12 @@ __device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, const W
     }
 }
 
+template <bool kCluster = false>
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const WaitCtx &ctx, int bar_id, int iter,
                                          uint64_t limit_ns = kWaitLimitNs)
 {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    return wait_slow(bar, parity, ctx, bar_id, iter, limit_ns);
+    if (kCluster ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity)) return true;
+    return wait_slow<kCluster>(bar, parity, ctx, bar_id, iter, limit_ns);
 }
 
 }  // namespace ll

@@ -313,16 +313,30 @@ int qkv_tile_width(int n_tokens, int width, int sm_count)
 
 // Fewer columns than CTAs, all equally long: every column in the same number of equal parts, one part per
 // CTA, when that is the cheapest way.  In steps, a part costs its own length; splitting at all costs the trip of
-// the parts through the scratch slots (kTripSteps) and the merge, by four parts (kBatchSteps each).  Against levelled shares it saves a CTA's second column segment
-// (kSegmentSteps: its first loads and its drain) and a part per column.  Over 40 drawn launches of
-// up to 100 GF the split by these costs takes 0.926 of the time of levelled shares (geometric mean; 95 x 662, 40
-// heads of 128: 19.5 -> 12.8 us); with (kTripSteps, kBatchSteps) of (1, 0.75) or (2.5, 1.5) shapes of 10 to 20
-// steps are split that are faster whole.  The benchmark layer's preview grid (17 x 29): 76 -> 70 us.
+// the parts through the scratch slots and the merge.  Up to eight parts are a thread-block cluster's, whose CTAs merge together
+// (cluster_steps), as long as all clusters are on the chip at once; otherwise whichever part arrives last merges (kTripSteps, and
+// kBatchSteps by four parts).  Against levelled shares it saves a CTA's second column segment
+// (kSegmentSteps: its first loads and its drain) and a part per column.
+//   Against whole columns, the merge of 2 / 4 / 8 parts costs 4.2 / 4.9 / 5.6 us in a cluster and 7 / 9.7 / 18 us where the last part does it (12 heads of
+// 128, 154 queries; a step there is 1.75 us).  14 / 22 / 40 steps: 27.5 / 38.5 / 64.4 us whole, 21.8 / 25.0 / 31.3 us in
+// four parts merged by the last, 14.5 / 16.3 / 20.1 us in clusters of eight; 72 columns of 22 / 40 steps (1400 queries) in two parts 33.3 / 47.0 us merged by
+// the last, 30.7 / 46.6 us in clusters.  48 columns in three parts (more than 45 clusters) against clusters of two, head_dim 64: 14 steps
+// 19.6 / 17.6 us, 22 steps 23.3 / 23.1, 40 steps 31.2 / 35.2.  All costs but the lengths are taken a little high (about a step): near
+// the line whole columns, tiles and fewer parts are as fast, and fewer parts round less:
 //   Every part takes its weights against references of its own, and the largest weight of a row and part is exactly 1
 // in bf16: with fewer parts fewer weights are exact.  Against 64 bits the relative error of few short columns is 2.25e-3 to
 // 2.36e-3 where levelled shares of a step or two gave 2.17e-3 to 2.28e-3; that of long columns is up to 2.37e-3 either way.
 //   Returns what the busiest CTA costs that way, in steps; 0 when the launch is not for it.
 constexpr double kTripSteps = 2.5, kBatchSteps = 2.5, kSegmentSteps = 2;
+constexpr int kMaxClusterParts = 8;
+double cluster_steps(long long parts) { return parts == 2 ? 3.5 : parts <= 4 ? 4 : 5; }
+// Clusters of n CTAs with this kernel's shared memory that a B200 holds (cudaOccupancyMaxActiveClusters; more would run one behind another).
+int clusters_at_once(long long n, int sms)
+{
+    static const int held[kMaxClusterParts + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    return n <= kMaxClusterParts ? std::min(held[n], sms / (int)n) : 0;
+}
+
 double even_split(ll::AttnParams *p, int sms, long long all_cols)
 {
     if (all_cols >= sms || all_cols <= 0) return 0;
@@ -331,14 +345,19 @@ double even_split(ll::AttnParams *p, int sms, long long all_cols)
         if (p->g[g].n_kt != n_kt) return 0;
     auto merge = [&](long long parts) { return parts > 1 ? kTripSteps + kBatchSteps * ((parts + 3) / 4) : 0.; };
     long long best = 1;
+    int cluster = 0;
     double cost = (double)n_kt;
+    const double beside = all_cols <= clusters_at_once(2, sms) ? 1 : 0;      // a cluster's merge is taken a step too high: so is the other beside it
     for (long long k = 2; k <= std::min<long long>(sms / all_cols, n_kt); ++k) {
-        const double c = (double)((n_kt + k - 1) / k) + merge(k);
-        if (c < cost) { cost = c; best = k; }
+        const bool together = all_cols <= clusters_at_once(k, sms);
+        const double c = (double)((n_kt + k - 1) / k) + (together ? cluster_steps(k) : merge(k) + beside);
+        if (c < cost) { cost = c; best = k; cluster = together ? (int)k : 0; }
     }
+    if (best > 1 && !cluster) cost = (double)((n_kt + best - 1) / best) + merge(best);
     const double share = (double)((all_cols * n_kt + sms - 1) / sms);
     if (cost > share + kSegmentSteps + merge((long long)((double)n_kt / share) + 2)) return 0;
     p->n_ctas = (int)(all_cols * best);
+    p->cluster_parts = cluster;
     p->n_shares = 0;
     p->share_begin[0] = 0;
     for (int i = 0; i < p->n_ctas; ++i) p->share_of_cta[i] = -1;
@@ -499,6 +518,7 @@ void plan_tiles(ll::AttnParams *p, int sms, double cost, int head_dim)
         }
         if (load >= limit) return;
     }
+    p->cluster_parts = 0;
     p->tile_ctas = ctas;
     p->tiles_each = each;
     p->tiles_extra = extra;
@@ -1322,6 +1342,7 @@ int debug_plan(const AttnCall *calls, int n_calls, int sm_count, ll_attn_plan *o
     out->tile_ctas = p.tile_ctas;
     out->tiles_each = p.tiles_each;
     out->tiles_extra = p.tiles_extra;
+    out->cluster_parts = p.cluster_parts;
     return LL_OK;
 }
 }  // namespace

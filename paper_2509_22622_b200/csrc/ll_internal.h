@@ -116,6 +116,8 @@ struct AttnParams {
     // > 0: everything goes out whole, but by 128-row tiles instead of columns: grid.x = tile_ctas, CTA i takes
     // tiles_each consecutive tiles (one more below tiles_extra), two of one head at a time
     int tile_ctas, tiles_each, tiles_extra;
+    // > 0: every column is split into this many parts, one per CTA of a cluster of this size, which merge them among themselves
+    int cluster_parts;
     long long total_steps;            // shared steps of all groups
     int64_t rows_per_head;            // (S+W)*P
     float scale_log2;                 // log2(e) / sqrt(D)
@@ -204,12 +206,12 @@ cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, int sm
 // layer 1.60 -> 1.63 M, backward of the 21-frame clip 14.85 -> 14.97 M) than the gap in front of them.
 // The projection has no such order to lose and always starts early (40 heads of 128, 4680 tokens, 757 us; 759 with an
 // ordinary start).  `carveout`: percentage of an SM's shared memory and L1 cache that the kernel wants as shared
-// memory, -1 the driver's choice.
+// memory, -1 the driver's choice.  `cluster`: CTAs of a cluster along x.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_dependent(bool early, int carveout, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                    Args &&...args)
+inline cudaError_t launch_dependent(bool early, int carveout, int cluster, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                                    cudaStream_t stream, Args &&...args)
 {
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     memset(attr, 0, sizeof attr);
     unsigned n = 0;
     if (early) {
@@ -219,6 +221,12 @@ inline cudaError_t launch_dependent(bool early, int carveout, void (*kernel)(Par
     if (carveout >= 0) {
         attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
         attr[n++].val.sharedMemCarveout = (unsigned)carveout;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        ++n;
     }
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
@@ -236,7 +244,7 @@ inline cudaError_t launch_dependent(bool early, int carveout, void (*kernel)(Par
 template <typename... Params, typename... Args>
 inline cudaError_t launch_dependent(bool early, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args)
 {
-    return launch_dependent(early, -1, kernel, grid, block, smem, stream, std::forward<Args>(args)...);
+    return launch_dependent(early, -1, 1, kernel, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 
 // How many blocks of a kernel an SM holds, and what that follows from.
@@ -286,7 +294,7 @@ inline cudaError_t launch_spread(unsigned blocks, unsigned threads, cudaStream_t
         if (kept && !known[dev].compare_exchange_strong(none, kept, std::memory_order_acq_rel)) delete kept;
     }
     const Spread s = spread_of(blocks, *r);
-    return launch_dependent(s.early, s.carveout, kKernel, blocks, threads, (size_t)s.smem, stream, std::forward<Args>(args)...);
+    return launch_dependent(s.early, s.carveout, 1, kKernel, blocks, threads, (size_t)s.smem, stream, std::forward<Args>(args)...);
 }
 
 // kernel launchers (each returns the cudaError of the launch)
