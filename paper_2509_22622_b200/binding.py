@@ -92,6 +92,8 @@ class LLError(RuntimeError):
 
 
 _lib = None
+_fast = None             # the marshalling module (csrc/marshal.c), once the library is loaded; None: not built
+_ELSEWHERE = None        # what it returns for arguments that only ctypes takes, or refuses
 
 # name -> (restype, argtypes); also the list of symbols include/llattn.h and include/llattn_debug.h declare
 SIGNATURES = {
@@ -156,7 +158,7 @@ SIGNATURES = {
 
 def lib():
     """Load the shared library (fails loudly when it is missing)."""
-    global _lib
+    global _lib, _fast, _ELSEWHERE
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -167,6 +169,15 @@ def lib():
             fn = getattr(L, name)
             fn.restype = res
             fn.argtypes = args
+        try:
+            from . import _marshal
+        except ImportError:
+            _marshal = None
+        if _marshal is not None:
+            _marshal.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name in SIGNATURES})
+            _fast, _ELSEWHERE = _marshal, _marshal.ELSEWHERE
+            if _torch_c is not None:
+                _marshal.streams(_torch_c._cuda_getDevice, _torch_c._cuda_getCurrentRawStream)
         _lib = L
     return _lib
 
@@ -195,6 +206,8 @@ def _stream(stream):
                 return 0
             torch.cuda.current_stream()            # initialises CUDA
             _torch_c = torch._C
+            if _fast is not None:
+                _fast.streams(_torch_c._cuda_getDevice, _torch_c._cuda_getCurrentRawStream)
         return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
     return stream if isinstance(stream, int) else stream.cuda_stream
 
@@ -240,18 +253,31 @@ def ll_cache_kv_offset(h, layer, which, head) -> int:
 
 def ll_rope_append_kv(h, layer, q, k, v, frame_start, n_frames, grid_h, grid_w, rope_theta=10000.0,
                       q_out=None, stream=None):
+    if _fast is not None:
+        code = _fast.rope_append_kv(h, layer, q, k, v, frame_start, n_frames, grid_h, grid_w, rope_theta, q_out, stream)
+        if code is not _ELSEWHERE:
+            return _check(code)
     _check(lib().ll_rope_append_kv(h, layer, _ptr(q), _ptr(k), _ptr(v), frame_start, n_frames, grid_h, grid_w,
                                    rope_theta, _ptr(q_out), _stream(stream)))
 
 
 def ll_norm_rope_append_kv(h, layer, q, k, v, gain_q, gain_k, eps, frame_start, n_frames, grid_h, grid_w,
                            rope_theta=10000.0, q_out=None, stream=None):
+    if _fast is not None:
+        code = _fast.norm_rope_append_kv(h, layer, q, k, v, gain_q, gain_k, eps, frame_start, n_frames, grid_h, grid_w, rope_theta, q_out,
+                                         stream)
+        if code is not _ELSEWHERE:
+            return _check(code)
     _check(lib().ll_norm_rope_append_kv(h, layer, _ptr(q), _ptr(k), _ptr(v), _ptr(gain_q), _ptr(gain_k), eps,
                                         frame_start, n_frames, grid_h, grid_w, rope_theta, _ptr(q_out),
                                         _stream(stream)))
 
 
 def ll_sink_window_attn(h, layer, q_roped, q_frame_start, n_q_frames, out, lse_out=None, stream=None):
+    if _fast is not None:
+        code = _fast.sink_window_attn(h, layer, q_roped, q_frame_start, n_q_frames, out, lse_out, stream)
+        if code is not _ELSEWHERE:
+            return _check(code)
     _check(lib().ll_sink_window_attn(h, layer, _ptr(q_roped), q_frame_start, n_q_frames, _ptr(out),
                                      _ptr(lse_out), _stream(stream)))
 
@@ -269,6 +295,11 @@ def ll_qkv_proj_workspace_bytes(h) -> int:
 def ll_qkv_proj_append(h, layer, x, w_qkv, bias, gain_q, gain_k, eps, frame_start, n_frames, grid_h, grid_w,
                        rope_theta, q_out, q_row_scale=None, workspace=None, stream=None):
     nbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    if _fast is not None:
+        code = _fast.qkv_proj_append(h, layer, x, x.shape[-1], w_qkv, bias, gain_q, gain_k, eps, frame_start, n_frames, grid_h, grid_w,
+                                     rope_theta, q_out, q_row_scale, workspace, nbytes, stream)
+        if code is not _ELSEWHERE:
+            return _check(code)
     _check(lib().ll_qkv_proj_append(h, layer, _ptr(x), x.shape[-1], _ptr(w_qkv), _ptr(bias), _ptr(gain_q), _ptr(gain_k),
                                     eps, frame_start, n_frames, grid_h, grid_w, rope_theta, _ptr(q_out),
                                     _ptr(q_row_scale), _ptr(workspace), nbytes, _stream(stream)))
@@ -276,6 +307,10 @@ def ll_qkv_proj_append(h, layer, x, w_qkv, bias, gain_q, gain_k, eps, frame_star
 
 def ll_sink_window_attn_batched(items, stream=None):
     """items: sequence of (handle, layer, q_roped, q_frame_start, n_q_frames, out, lse_out or None)."""
+    if _fast is not None:
+        code = _fast.sink_window_attn_batched(items, stream)
+        if code is not _ELSEWHERE:
+            return _check(code)
     def addr(t):
         return None if t is None else t.data_ptr()
     arr = (ll_attn_item * max(len(items), 1))()
@@ -293,6 +328,10 @@ def ll_debug_attn_simt(h, layer, q_roped, q_frame_start, n_q_frames, out, lse_ou
 def ll_cross_attn(h, q, k, v, out, lse_out=None, stream=None, n_q=None, n_k=None):
     n_q = q.shape[0] if n_q is None else n_q
     n_k = k.shape[0] if n_k is None else n_k
+    if _fast is not None:
+        code = _fast.cross_attn(h, q, n_q, k, v, n_k, out, lse_out, stream)
+        if code is not _ELSEWHERE:
+            return _check(code)
     _check(lib().ll_cross_attn(h, _ptr(q), n_q, _ptr(k), _ptr(v), n_k, _ptr(out), _ptr(lse_out), _stream(stream)))
 
 

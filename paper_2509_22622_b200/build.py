@@ -1,14 +1,17 @@
-"""Build ``libllattn.so`` in-tree with nvcc for sm_100a (no torch in the link)."""
+"""Build ``libllattn.so`` in-tree with nvcc for sm_100a (no torch in the link), and the binding's marshalling module with the host compiler."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libllattn.so")
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
+MARSHAL_SOURCE = os.path.join(CSRC, "marshal.c")
 SOURCES = ["ll_host.cu", "rope_append.cu", "attn_sm100.cu", "attn_simt.cu", "rope_static.cu", "qkv_gemm.cu", "attn_bwd.cu"]
 HEADERS = ["ll_internal.h", "ptx.cuh", "bounded_wait.cuh", "exp2_poly.cuh", "rope_math.cuh", os.path.join(ROOT, "include", "llattn.h"),
            os.path.join(ROOT, "include", "llattn_debug.h")]
@@ -35,8 +38,23 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_marshal(force: bool = False) -> None:
+    """The marshalling module.  Without Python's headers there is none and the binding's ctypes functions serve every call."""
+    include = sysconfig.get_paths()["include"]
+    header = os.path.join(ROOT, "include", "llattn.h")
+    if not os.path.exists(os.path.join(include, "Python.h")):
+        return
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) > max(map(os.path.getmtime, (MARSHAL_SOURCE, header, __file__))):
+        return
+    tmp = MARSHAL + ".tmp%d" % os.getpid()
+    subprocess.check_call([os.environ.get("CC") or "gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", include, "-I", os.path.join(ROOT, "include"),
+                           MARSHAL_SOURCE, "-o", tmp])
+    os.replace(tmp, MARSHAL)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every translation unit and link the shared library; returns its path."""
+    build_marshal(force)
     if not force and not _stale():
         return LIB
     objs = []
