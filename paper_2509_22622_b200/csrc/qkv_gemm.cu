@@ -86,13 +86,6 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
     return r;
 }
 
-__device__ __forceinline__ uint32_t ld_shared_cluster(uint32_t addr)
-{
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -256,6 +249,7 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
     grid_dep_launch();
     if (threadIdx.x == 0) {
         for (int i = 0; i < G::kBars; ++i) mbar_init(bar(i), (i >= kAccEmpty) ? 2u * G::kEpiWarps : 1u);   // both CTAs' epilogue warps free a buffer
+        *abort_flag = 0;
         fence_mbar_init();
     }
     if (warp == 0) {
@@ -263,16 +257,28 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
-    grid_dep_wait();
-    if (threadIdx.x == 0) *abort_flag = (rank == 0 && *reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
+    if (warp == 0 && lane == 0) {                      // (the maps are launch parameters)
+        prefetch_tensormap(&xmap);
+        prefetch_tensormap(&wmap);
+    }
     tc_fence_before_sync();
     __syncwarp();
     cluster_sync();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     WaitCtx ctx{abort_flag, p.status, warp};
-    // the leader's look at the status word decides for the pair
-    const bool skip = ld_shared_cluster(map_to_rank(smem_u32(tmem_slot + 1), 0)) == 2u;
+    grid_dep_wait();
+    // An earlier kernel gave up on a wait: the pair does not start (flag value 2).  The load warp does not wait to hear of that, its first
+    // tiles are under way meanwhile; it finds the flag when it runs out of stages.  (In front of the first load stood the read of the
+    // status word, the pair's barrier and a look at the leader's flag: 270 tokens, 256 -> 3 x 1536 with norm 13.3 -> 12.7 us; 312 tokens,
+    // 1024 -> 3 x 192 15.2 -> 14.6; 200 tokens, 2048 -> 3 x 5120 33.3 -> 32.6.)
+    if (warp == 0) {
+        named_arrive(1, G::kThreads);
+    } else {
+        if (threadIdx.x == 32 && *reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) *abort_flag = 2;
+        named_sync(1, G::kThreads);
+    }
+    const bool skip = warp != 0 && *abort_flag != 0;
     auto wait = [&](int bar_id, uint32_t parity, int iter) -> bool {
         return wait_bar(bar(bar_id), parity & 1u, ctx, bar_id, iter);
     };
@@ -284,8 +290,6 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
     } else if (warp == 0 && lane == 0) {
         // ---- TMA producer (each CTA its own halves): tiles in the order all roles walk them; tokens
         // run fastest, so that the last round, whose epilogue nothing hides, is of v: no norm, no rotation ----
-        prefetch_tensormap(&xmap);
-        prefetch_tensormap(&wmap);
         uint32_t n = 0;
         for (int tile = pair; tile < n_tiles; tile += n_pairs) {
             const int m0 = (tile % p.m_tiles) * kTileM + 128 * (int)rank, n0 = (tile / p.m_tiles) * TN + TN / 2 * (int)rank;
@@ -354,7 +358,7 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
 done:
     tc_fence_before_sync();
     __syncthreads();
-    if (*abort_flag == 1) {
+    if (*abort_flag != 0) {
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
     }
