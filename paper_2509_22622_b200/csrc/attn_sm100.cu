@@ -1258,6 +1258,43 @@ cudaError_t launch_instance(const AttnParams &p, const AttnMaps &maps, dim3 grid
 
 }  // namespace
 
+namespace {
+
+// Whether the device holds a cluster of n of this kernel's CTAs (a part of a GPU may not); asked once per device and size.
+template <int D>
+bool cluster_fits(int n)
+{
+    constexpr int kMaxDevices = 64, kMaxParts = 8;
+    static std::atomic<signed char> known[kMaxDevices][kMaxParts + 1];      // 0: not asked, 1: yes, -1: no
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || n > kMaxParts) return false;
+    if (dev < kMaxDevices)
+        if (const int k = known[dev][n].load(std::memory_order_acquire)) return k > 0;
+    cudaLaunchAttribute attr;
+    memset(&attr, 0, sizeof attr);
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)n;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3((unsigned)n);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int held = 0;
+    cudaError_t e = cudaFuncSetAttribute(attn_sm100_kernel<D, kFormParts>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&held, attn_sm100_kernel<D, kFormParts>, &cfg);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        held = 0;
+    }
+    if (dev < kMaxDevices) known[dev][n].store(held > 0 ? 1 : -1, std::memory_order_release);
+    return held > 0;
+}
+
+}  // namespace
+
 cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps &maps, cudaStream_t stream)
 {
     if (p.n_ctas <= 0) return cudaSuccess;
@@ -1266,7 +1303,7 @@ cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps 
     long long steps = 0;
     for (int g = 0; g < p.n_groups; ++g) steps += (long long)p.heads * p.g[g].tiles * p.g[g].n_kt;
     const bool early = steps <= kEarlySteps * p.n_ctas;
-    if (p.cluster_parts > 0)
+    if (p.cluster_parts > 0 && (head_dim == 128 ? cluster_fits<128>(p.cluster_parts) : cluster_fits<64>(p.cluster_parts)))      // else the last part merges
         e = head_dim == 128 ? launch_instance<128, kFormParts>(p, maps, grid, early, stream) : launch_instance<64, kFormParts>(p, maps, grid, early, stream);
     else if (head_dim == 128) e = launch_instance<128, kFormTiles>(p, maps, grid, early, stream);
     else if (p.tile_ctas > 0) e = launch_instance<64, kFormTiles>(p, maps, grid, early, stream);

@@ -119,3 +119,54 @@ def test_cluster_parts_of_a_cache(dim):
         cache.check_device()
         check_attn(f64(out), want(q_out, k, v, one))
         cache.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dim", [64, 128])
+def test_captured_cluster_parts(dim):
+    """A launch of clusters between two others in a captured graph, replayed."""
+    gen = torch.Generator(device="cuda").manual_seed(dim)
+    q, k, v = (torch.randn(n, 8, dim, device="cuda", generator=gen).to(torch.bfloat16) for n in (450, 2300, 2300))
+    cache = B.Cache(1, 8, dim, 16, 1, 1, 1)
+    assert B.ll_debug_attn_plan_cross(cache.h, 450, 2300).cluster_parts > 0
+    a, b, c = (torch.empty_like(q) for _ in range(3))
+    want = []
+    for src, dst in ((q, a), (a, b), (b, c)):
+        cache.cross_attn(src, k, v, dst)
+        torch.cuda.synchronize()
+        want.append(dst.clone())
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):
+        for src, dst in ((q, a), (a, b), (b, c)):
+            cache.cross_attn(src, k, v, dst)
+    for _ in range(3):
+        for t in (a, b, c):
+            t.fill_(float("nan"))
+        graph.replay()
+        assert all(torch.equal(t, w) for t, w in zip((a, b, c), want))
+    cache.check_device()
+    del graph
+    cache.close()
+
+
+@pytest.mark.gpu
+def test_clusters_on_two_streams():
+    """Launches of clusters of two handles side by side: each CTA waits only for those of its own cluster."""
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    work = []
+    for n_q, n_k in ((1479, 5916), (450, 2250)):
+        q, k, v = (torch.randn(n, 12, 128, device="cuda", generator=gen).to(torch.bfloat16) for n in (n_q, n_k, n_k))
+        cache = B.Cache(1, 12, 128, 16, 1, 1, 1)
+        assert B.ll_debug_attn_plan_cross(cache.h, n_q, n_k).cluster_parts > 0
+        want = torch.empty_like(q)
+        cache.cross_attn(q, k, v, want)
+        work.append((cache, q, k, v, torch.empty_like(q), want, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for cache, q, k, v, out, _, stream in work:
+            cache.cross_attn(q, k, v, out, stream=stream)
+    torch.cuda.synchronize()
+    for cache, _, _, _, out, want, stream in work:
+        cache.check_device(stream)
+        assert torch.equal(out, want)
+        cache.close()

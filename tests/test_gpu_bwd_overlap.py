@@ -44,5 +44,12 @@ def test_calls_in_a_row(heads, dim, p, chunks, window):
     for _ in range(3):
         for a, b in zip(run(False), want):
             assert all(torch.equal(x, y) and bool(x.isfinite().all()) for x, y in zip(a, b))
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):     # captured calls, each behind the one before
+        captured = run(False)
+    graph.replay()
+    for a, b in zip(captured, want):
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
     cache.check_device()
+    del graph
     cache.close()
