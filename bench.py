@@ -523,7 +523,7 @@ def run_ours(args):
         own_f = sum(min((g + 1) * C, wl.window_frames) for g in range(clip_chunks))
         bwd_flops = 2.0 * nq * P * D * H * (3 * all_f + 2 * own_f)      # S, dP, dQ over all keys; dK, dV over the clip's
         others["clip_21_frames_backward"] = {"ms": ms, "tflops_algorithmic": bwd_flops / ms / 1e9,
-                                             "note": "S and dP are formed twice (dq kernel and dk/dv kernel): 7 products "
+                                             "note": "S and dP are formed twice (dq blocks and dk/dv blocks): 7 products "
                                                      "run where 5 are counted"}
         big.check_device()
         big.close()

@@ -4,32 +4,31 @@
 // With s_ij = q_i.k_j / sqrt(D) over the keys visible to row i, p_ij = exp(s_ij - lse_i):
 //   delta_i = d_out_i . out_i                                  (delta kernel)
 //   dP_ij = d_out_i . v_j,   dS_ij = p_ij (dP_ij - delta_i)
-//   dq_i = sum_j dS_ij k_j / sqrt(D)                            (dq kernel, one CTA per query tile)
-//   dk_j = sum_i dS_ij q_i / sqrt(D),  dv_j = sum_i p_ij d_out_i   (dkdv kernel, one CTA per key tile)
+//   dq_i = sum_j dS_ij k_j / sqrt(D)                            (dq blocks, one CTA per query tile)
+//   dk_j = sum_i dS_ij q_i / sqrt(D),  dv_j = sum_i p_ij d_out_i   (dk/dv blocks, one CTA per key tile)
 // q, k are the rotated tensors; dq and dk are turned back through the rotation before they are
 // stored.  Only the clip's own keys get dk, dv (the sink and the context are detached).
 //
-// Two kernels instead of one with atomics: every gradient element is accumulated by one CTA in one
-// order, so the result is run-to-run deterministic, at the price of forming S and dP twice.  Both
-// kernels have one warp that issues the MMAs (all its lanes walk the loop so that descriptors are warp-uniform;
+// Two passes over the products instead of one with atomics: every gradient element is accumulated by one CTA in one
+// order, so the result is run-to-run deterministic, at the price of forming S and dP twice.  Both kinds of
+// block have one warp that issues the MMAs (all its lanes walk the loop so that descriptors are warp-uniform;
 // one elected lane issues) and eight compute warps (one thread per tile row and 64-column half, the 32x32b TMEM
-// shape).  The dq kernel's issuer also loads (TMA); its compute warps take S into registers and release its tensor
-// memory at once, so the next step's S is formed while they are in the exponentials.  The dk/dv kernel has a
-// load warp of its own, and forms the next S once P has been read.  dP is read only for the last multiply.
-//   Neither kernel needs what the other writes, so the dk/dv kernel starts as soon as every dq block has: behind a short
-// dq grid on the SMs that it leaves idle, behind a long one in its last wave.  Every dq block lets it start only behind its own wait
-// for delta, and the last dk/dv block waits for the dq kernel before it ends, so that whoever comes next waits for both.
-// 450 rows, 3 heads of 128: 34.1 -> 22.0 us; 3920 rows, 2 of 64: 92.8 -> 59.3; 992 rows, 40 of 128: 105 -> 94; 8000 rows, 1 of 128: 193 -> 115;
-// the 21-frame clip 8850 -> 8800.
+// shape).  The dq blocks' issuer also loads (TMA); their compute warps take S into registers and release its tensor
+// memory at once, so the next step's S is formed while they are in the exponentials.  The dk/dv blocks have a
+// load warp of their own, and form the next S once P has been read.  dP is read only for the last multiply.
+//   Neither kind needs what the other writes, so one launch holds both, the dq blocks in front: the dk/dv blocks fill the SMs that a
+// short dq part leaves idle, or the end of a long one, and every block waits for delta as the kernels of a stream do.
+// Against two kernels one behind the other, in us: 650 rows, 2 heads of 128: 33.1 -> 20.6; 2394 rows, 3 of 128: 71.6 -> 42.7; 3240 rows, 2 of 64:
+// 82.0 -> 49.8; 11628 rows, 1 of 128: 381 -> 261; 768 rows, 16 of 64: 19.1 -> 18.3; the 21-frame clip 8919 and 8908.
 //   What they compute goes back to tensor memory as the A operand of the products that follow: dS over dP, and in
-// the dk/dv kernel P over S (at head_dim 64 beside them, where columns are left).  Through shared memory those tiles
+// the dk/dv blocks P over S (at head_dim 64 beside them, where columns are left).  Through shared memory those tiles
 // cost a store and a read of 32 KB each beside operands of 64 KB per 512 clk of products.
 //   Products run in the order of their issue only if they share accumulator and shape.  One that overwrites columns
 // which an earlier one reads as its A operand is therefore issued behind that one's commit; stores from registers are
 // behind a later product's commit anyway, which covers all products before it.
 //   21-frame clip of the benchmark layer (32760 rows, 12 heads of 128): 9.25 -> 8.80 ms in a loop at the power limit (8.65 without
-// the waits between products).  Serving the two 64-key halves of the dq kernel's steps as chains of their own, half a step
-// apart, was slower (64-wide products: 4.66 ms for the kernel where it took 4.07 without those waits).
+// the waits between products).  Serving the two 64-key halves of the dq blocks' steps as chains of their own, half a step
+// apart, was slower (64-wide products: 4.66 ms for them where they took 4.07 without those waits).
 #include <cuda_bf16.h>
 
 #include "bounded_wait.cuh"
@@ -43,12 +42,13 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kBwdThreads = 288;                       // eight compute warps, one load/issue warp
-constexpr int kIssueWarp = 8;
-constexpr int kDkdvThreads = 320;                      // the dk/dv kernel adds a load warp
-constexpr int kLoadWarp = 9;
+constexpr int kComputeWarps = 8;
+constexpr int kIssueWarp = 8;                          // issues the MMAs; in the dq blocks the loads too
+constexpr int kLoadWarp = 9;                           // of the dk/dv blocks
+constexpr int kBwdThreads = 320;
 constexpr int kTile = 128;
-constexpr int kStatBytes = 2 * kTile * 4;              // a query tile's row statistics in the dk/dv kernel
+constexpr int kStatBytes = 2 * kTile * 4;              // a query tile's row statistics in the dk/dv blocks
+constexpr int kBwdBars = 17;
 
 __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t *r)
 {
@@ -166,6 +166,17 @@ template <int D>
 struct BwdCfg {
     static constexpr int kAtomBytes = 128 * 128;
     static constexpr int kTileBytes = (D / 64) * kAtomBytes;     // 128 rows x D bf16
+    static constexpr int kBarOff = 6 * kTileBytes + 2 * kStatBytes;      // behind the tiles and the dk/dv blocks' statistics
+    static constexpr int kSmemBytes = kBarOff + 2048;            // barriers, tensor memory address, flag; alignment of the tiles
+};
+
+// What a block has once its barriers and its tensor memory are set up and the kernels in front of this one have completed.
+struct BwdSetup {
+    uint32_t base, bars, tmem;                         // shared addresses of the tiles and the barriers; tensor memory
+    uint8_t *gen;                                      // the tiles again
+    volatile int *abort_flag;
+    bool skip;                                         // an earlier kernel gave up on a wait: nothing to do
+    int warp, head;
 };
 
 // MMA helpers: all tiles are 128-byte-swizzled, 128 rows, tile base 1024-byte aligned.  The low
@@ -228,51 +239,40 @@ __device__ __forceinline__ void scores_to_weights(uint32_t (&s)[64], float c, fl
 // three stages; K is needed until the step's dQ product, V only until its dP.
 //   tensor memory columns: S 0..127, dP 128..255, dQ 256..256+D-1, Q 384.., dO 448..; dS of key half h at 128 + 64 h.. or 416 + 64 h..
 template <int D>
-__global__ void __launch_bounds__(kBwdThreads, 1)
-bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMaps maps)
-{
+struct DqBlock {
     using C = BwdCfg<D>;
-    constexpr int kStages = 3;
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
-    const uint32_t k_s = base, v_s = k_s + kStages * C::kTileBytes, bars = v_s + kStages * C::kTileBytes;
     enum { kKFull = 0, kVFull = 3, kKEmpty = 6, kVEmpty = 9, kSFull = 12, kSFree = 13, kDpFull = 14, kDsFull = 15, kDone = 16, kBars = 17 };
-    constexpr int kComputeWarps = 8;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(gen + (bars - base) + kBars * 8);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
-    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int head = blockIdx.y;
-    // which group and tile of it
-    int g = 0, tile = blockIdx.x;
-    while (tile >= (p.g[g].q_rows + kTile - 1) / kTile) { tile -= (p.g[g].q_rows + kTile - 1) / kTile; ++g; }
+    static __device__ uint32_t arrivals(int bar_id) { return bar_id == kSFree || bar_id == kDsFull ? kComputeWarps : 1; }
+
+    int g, tile;                                       // query group, and which tile of it
+    __device__ DqBlock(const BwdParams &p, int t) : g(0), tile(t)
+    {
+        while (tile >= (p.g[g].q_rows + kTile - 1) / kTile) { tile -= (p.g[g].q_rows + kTile - 1) / kTile; ++g; }
+    }
+    __device__ __forceinline__ void run(const BwdParams &p, const BwdMaps &maps, const BwdSetup &b) const;
+};
+
+template <int D>
+__device__ __forceinline__ void DqBlock<D>::run(const BwdParams &p, const BwdMaps &maps, const BwdSetup &b) const
+{
+    constexpr int kStages = 3;
+    const uint32_t k_s = b.base, v_s = k_s + kStages * C::kTileBytes;
+    const int warp = b.warp, lane = threadIdx.x & 31, head = b.head;
+    auto bar = [&](int i) -> uint32_t { return b.bars + 8u * (uint32_t)i; };
     const AttnGroup &G = p.g[g];
     const int q0 = G.q_begin + tile * kTile, rows = min(kTile, G.q_rows - tile * kTile);
     const int n_kt = G.n_kt;
-
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kBars; ++i) mbar_init(bar(i), (i == kSFree || i == kDsFull) ? kComputeWarps : 1);
-        fence_mbar_init();
-    }
-    if (warp == kIssueWarp) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
-    grid_dep_wait();
-    grid_dep_launch();                                 // behind the wait: a dk/dv block that starts now finds delta complete
-    if (threadIdx.x == 0) *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    const uint32_t tmem = *tmem_slot;
-    WaitCtx ctx{abort_flag, p.status, warp};
+    const uint32_t tmem = b.tmem;
+    const WaitCtx ctx{b.abort_flag, p.status, warp};
     auto wait = [&](int bar_id, uint32_t parity, int iter) -> bool { return wait_bar(bar(bar_id), parity & 1u, ctx, bar_id, iter); };
-    const bool skip = *abort_flag != 0;
+    const bool skip = b.skip;
     constexpr bool kOverDp = D == 128;                           // dS takes the place of dP
     const uint32_t t_s = tmem, t_dp = tmem + 128, t_dq = tmem + 256, t_q = tmem + 384, t_do = tmem + 448,
                    t_ds = kOverDp ? t_dp : tmem + 416;
 
     // the tile's Q rows (warps 0-3) and dO rows (warps 4-7) into tensor memory; rows past the
     // group's end become zeros
-    if (!skip && warp != kIssueWarp) {
+    if (!skip && warp < kIssueWarp) {
         const int row = threadIdx.x & 127, half = threadIdx.x >> 7;
         const bool live = row < rows;
         const uint4 *src = reinterpret_cast<const uint4 *>((half ? p.d_out : p.q) + ((size_t)(q0 + (live ? row : 0)) * p.heads + head) * D);
@@ -377,7 +377,7 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
             }
             commit(kDone);
         }();
-    } else {
+    } else if (warp < kIssueWarp) {
         bool alive = true;
         auto wait_c = [&](int bar_id, uint32_t parity, int iter) {
             if (alive && !__all_sync(0xffffffffu, wait(bar_id, parity, iter))) alive = false;
@@ -431,16 +431,7 @@ bwd_dq_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMa
             store_grad_row<D, true>(t_dq + lane_off, p.scale, p.dq + ((size_t)token * p.heads + head) * D, p, frame,
                                     cell / p.grid_w, cell % p.grid_w, live, half);
     }
-    tc_fence_before_sync();
-    __syncthreads();
-    if (*abort_flag == 1) {
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
-        __syncthreads();
-    }
-    if (warp == kIssueWarp) { __syncwarp(); tc_fence_after_sync(); tmem_dealloc(tmem, 512); }
 }
-
 
 // Which of the 128 cache rows starting at r0 a group can see (bit c of word c / 32 = row r0 + c).
 __device__ __forceinline__ bool group_mask(const AttnGroup &G, int r0, uint32_t (&valid)[4])
@@ -505,42 +496,34 @@ struct QTiles {
 //   tensor memory columns: S 0..127, dP 128..255, dK and dV 256..256+2D-1; P (16-query slices 0-3 at 0.., 4-7 at 64.. of it) at 0
 // or 384, dS (likewise) at 128 or 416.
 template <int D>
-__global__ void __launch_bounds__(kDkdvThreads, 1)
-bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMaps maps)
-{
+struct DkdvBlock {
     using C = BwdCfg<D>;
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
-    const uint32_t k_s = base, v_s = k_s + C::kTileBytes, q_s = v_s + C::kTileBytes, do_s = q_s + 2 * C::kTileBytes,
-                   stat_s = do_s + 2 * C::kTileBytes, bars = stat_s + 2 * kStatBytes;
     enum { kKvFull = 0, kQFull = 1, kDoFull = 3, kQEmpty = 5, kDoEmpty = 7, kStatFull = 9, kSFull = 11, kPHalf = 12, kPFull = 13,
            kDpFull = 14, kDsFull = 15, kDone = 16, kBars = 17 };
-    constexpr int kComputeWarps = 8;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(gen + (bars - base) + kBars * 8);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
-    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int head = blockIdx.y;
-    // the tile's first cache row and the end of the run it belongs to
-    int run = 0, t = blockIdx.x;
-    while (t >= (p.krun_len[run] + kTile - 1) / kTile) { t -= (p.krun_len[run] + kTile - 1) / kTile; ++run; }
-    const int r0 = p.krun_start[run] + t * kTile, run_end = p.krun_start[run] + p.krun_len[run];
+    static __device__ uint32_t arrivals(int bar_id) { return bar_id == kPHalf || bar_id == kPFull || bar_id == kDsFull ? kComputeWarps : 1; }
 
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kBars; ++i) mbar_init(bar(i), (i == kPHalf || i == kPFull || i == kDsFull) ? kComputeWarps : 1);
-        fence_mbar_init();
+    int r0, run_end;                                   // the tile's first cache row and the end of the run it belongs to
+    __device__ DkdvBlock(const BwdParams &p, int t)
+    {
+        int run = 0;
+        while (t >= (p.krun_len[run] + kTile - 1) / kTile) { t -= (p.krun_len[run] + kTile - 1) / kTile; ++run; }
+        r0 = p.krun_start[run] + t * kTile;
+        run_end = p.krun_start[run] + p.krun_len[run];
     }
-    if (warp == kIssueWarp) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
-    grid_dep_launch();
-    if (threadIdx.x == 0) *abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    const uint32_t tmem = *tmem_slot;
-    WaitCtx ctx{abort_flag, p.status, warp};
+    __device__ __forceinline__ void run(const BwdParams &p, const BwdMaps &maps, const BwdSetup &b) const;
+};
+
+template <int D>
+__device__ __forceinline__ void DkdvBlock<D>::run(const BwdParams &p, const BwdMaps &maps, const BwdSetup &b) const
+{
+    const uint32_t k_s = b.base, v_s = k_s + C::kTileBytes, q_s = v_s + C::kTileBytes, do_s = q_s + 2 * C::kTileBytes;
+    uint8_t *const stats = b.gen + 6 * C::kTileBytes;            // two slots of kStatBytes
+    const int warp = b.warp, lane = threadIdx.x & 31, head = b.head;
+    auto bar = [&](int i) -> uint32_t { return b.bars + 8u * (uint32_t)i; };
+    const uint32_t tmem = b.tmem;
+    const WaitCtx ctx{b.abort_flag, p.status, warp};
     auto wait = [&](int bar_id, uint32_t parity, int iter) -> bool { return wait_bar(bar(bar_id), parity & 1u, ctx, bar_id, iter); };
-    const bool skip = *abort_flag != 0;
+    const bool skip = b.skip;
     constexpr bool kOver = D == 128;                             // P and dS take the places of S and dP
     const uint32_t t_s = tmem, t_dp = tmem + 128, t_dk = tmem + 256, t_dv = tmem + 256 + D,
                    t_p = kOver ? t_s : tmem + 384, t_ds = kOver ? t_dp : tmem + 416;
@@ -565,8 +548,8 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                 for (int i = 0; i < 4; ++i) {
                     const bool in = lane + 32 * i < live;
                     const size_t stat = (size_t)head * p.nq_total + row + (in ? lane + 32 * i : 0);
-                    nl[i] = in ? -1.4426950408889634f * __ldcg(p.lse + stat) : 0.f;      // (from L2: this kernel has not waited)
-                    nd[i] = in ? -__ldcg(p.delta + stat) : 0.f;
+                    nl[i] = in ? -1.4426950408889634f * p.lse[stat] : 0.f;
+                    nd[i] = in ? -p.delta[stat] : 0.f;
                 }
                 if (j == 0) {
                     if (elected) {
@@ -582,7 +565,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
                 load_tile(q_s + sl * C::kTileBytes, &maps.q, kQFull + sl, row);
                 if (j >= 2 && !wait(kDoEmpty + sl, (j >> 1) - 1, j)) return;     // dV(j-2) has read dO(j-2)
                 load_tile(do_s + sl * C::kTileBytes, &maps.d_out, kDoFull + sl, row);
-                float *st = reinterpret_cast<float *>(gen + (stat_s - base) + sl * kStatBytes);
+                float *st = reinterpret_cast<float *>(stats + sl * kStatBytes);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     st[lane + 32 * i] = nl[i];
@@ -677,7 +660,7 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
             const uint32_t word = row < 32 ? valid[0] : row < 64 ? valid[1] : row < 96 ? valid[2] : valid[3];
             const bool seen = (word >> (row & 31)) & 1u;         // whether the group sees this key
             for (int i = 0; i * kTile < G.q_rows; ++i, ++step) {
-                const float4 *nl = reinterpret_cast<const float4 *>(gen + (stat_s - base) + (step & 1) * kStatBytes) + 16 * half;
+                const float4 *nl = reinterpret_cast<const float4 *>(stats + (step & 1) * kStatBytes) + 16 * half;
                 const float4 *nd = nl + kTile / 4;
                 const int n_live = seen ? G.q_rows - i * kTile - 64 * half : 0;      // live columns of this thread's 64 (or more)
                 wait_c(kStatFull + (step & 1), step >> 1, (int)step);
@@ -751,19 +734,52 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
             store_grad_row<D, false>(t_dv + lane_off, 1.f, p.dv + (token * p.heads + head) * D, p, 0, 0, 0, live, half);
         }
     }
+}
+
+// The dq blocks of the call, tile after tile and head after head, then its dk/dv blocks.
+template <int D>
+__global__ void __launch_bounds__(kBwdThreads, 1)
+bwd_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ BwdMaps maps)
+{
+    using C = BwdCfg<D>;
+    static_assert(DqBlock<D>::kBars <= kBwdBars && DkdvBlock<D>::kBars <= kBwdBars, "more barriers than there is room for");
+    extern __shared__ uint8_t smem_raw[];
+    BwdSetup b;
+    b.base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    b.gen = smem_raw + (b.base - smem_u32(smem_raw));
+    b.bars = b.base + C::kBarOff;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(b.gen + C::kBarOff + kBwdBars * 8);
+    b.abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    b.warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int n_dq = p.n_qtiles * p.heads;
+    const bool is_dq = (int)blockIdx.x < n_dq;
+    const int index = is_dq ? (int)blockIdx.x : (int)blockIdx.x - n_dq, tiles = is_dq ? p.n_qtiles : p.n_ktiles;
+    b.head = index / tiles;
+    const int tile = index - b.head * tiles;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kBwdBars; ++i) mbar_init(b.bars + 8u * (uint32_t)i, is_dq ? DqBlock<D>::arrivals(i) : DkdvBlock<D>::arrivals(i));
+        fence_mbar_init();
+    }
+    if (b.warp == kIssueWarp) { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+    grid_dep_launch();
+    grid_dep_wait();
+    if (threadIdx.x == 0) *b.abort_flag = (*reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) ? 2 : 0;
     tc_fence_before_sync();
     __syncthreads();
-    if (*abort_flag == 1) {
+    tc_fence_after_sync();
+    b.tmem = *tmem_slot;
+    b.skip = *b.abort_flag != 0;
+    if (is_dq) DqBlock<D>(p, tile).run(p, maps, b);
+    else DkdvBlock<D>(p, tile).run(p, maps, b);
+    tc_fence_before_sync();
+    __syncthreads();
+    if (*b.abort_flag == 1) {
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
         __syncthreads();
     }
-    if (warp == kIssueWarp) { __syncwarp(); tc_fence_after_sync(); tmem_dealloc(tmem, 512); }
-    // whoever waits for this kernel waits for dq too (one block does, and holds nothing that a dq block may still need)
-    if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y) {
-        __syncthreads();
-        grid_dep_wait();
-    }
+    if (b.warp == kIssueWarp) { __syncwarp(); tc_fence_after_sync(); tmem_dealloc(b.tmem, 512); }
 }
 
 }  // namespace
@@ -771,16 +787,9 @@ bwd_dkdv_kernel(const __grid_constant__ BwdParams p, const __grid_constant__ Bwd
 cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, int sm_count, cudaStream_t stream)
 {
     const int D = p.head_dim;
-    const size_t tile = (size_t)128 * D * 2;
-    const int smem_dq = (int)(6 * tile + 2048), smem_kv = (int)(6 * tile + 2 * kStatBytes + 2048);
-    cudaError_t e;
-    if (D == 128) {
-        e = cudaFuncSetAttribute(bwd_dq_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_dq);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bwd_dkdv_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_kv);
-    } else {
-        e = cudaFuncSetAttribute(bwd_dq_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_dq);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bwd_dkdv_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_kv);
-    }
+    const int smem = D == 128 ? BwdCfg<128>::kSmemBytes : BwdCfg<64>::kSmemBytes;
+    cudaError_t e = D == 128 ? cudaFuncSetAttribute(bwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                             : cudaFuncSetAttribute(bwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     // D / 8 threads per four rows of a head
     const long long threads = (long long)((p.nq_total + 3) / 4) * p.heads * (D / 8);
@@ -791,13 +800,9 @@ cudaError_t launch_attn_backward(const BwdParams &p, const BwdMaps &maps, int sm
     long long steps = 0;
     for (int g = 0; g < p.n_groups; ++g) steps += (long long)p.heads * ((p.g[g].q_rows + kTile - 1) / kTile) * p.g[g].n_kt;
     const bool early = steps <= kEarlySteps * sm_count;
-    dim3 gq((unsigned)p.n_qtiles, (unsigned)p.heads), gk((unsigned)p.n_ktiles, (unsigned)p.heads);
-    e = D == 128 ? launch_dependent(early, bwd_dq_kernel<128>, gq, kBwdThreads, smem_dq, stream, p, maps)
-                 : launch_dependent(early, bwd_dq_kernel<64>, gq, kBwdThreads, smem_dq, stream, p, maps);
-    count_launch();
-    if (e != cudaSuccess) return e;
-    e = D == 128 ? launch_dependent(true, bwd_dkdv_kernel<128>, gk, kDkdvThreads, smem_kv, stream, p, maps)
-                 : launch_dependent(true, bwd_dkdv_kernel<64>, gk, kDkdvThreads, smem_kv, stream, p, maps);
+    const dim3 grid((unsigned)(p.n_qtiles + p.n_ktiles) * (unsigned)p.heads);
+    e = D == 128 ? launch_dependent(early, bwd_kernel<128>, grid, kBwdThreads, smem, stream, p, maps)
+                 : launch_dependent(early, bwd_kernel<64>, grid, kBwdThreads, smem, stream, p, maps);
     count_launch();
     return e;
 }

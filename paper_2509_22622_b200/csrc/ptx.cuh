@@ -26,8 +26,7 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // A kernel launched with launch_dependent or launch_spread (ll_internal.h) may start while the kernel before it in the stream
 // is still running.  It calls grid_dep_launch() early, which lets the kernel behind it do the same once all its
 // blocks have started, and grid_dep_wait() before its first access to global memory: that returns when the
-// kernels before it have completed and their writes are visible.  (bwd_dkdv_kernel alone waits at its end: what it reads was complete
-// before the kernel in front let it start, and it reads past the L1 cache.)  What can be done without memory (barriers,
+// kernels before it have completed and their writes are visible.  What can be done without memory (barriers,
 // tensor memory, index arithmetic where it pays) comes before the wait.  rope_q_static_kernel, attn_simt_kernel and
 // wait_probe_kernel have neither call and are launched the ordinary way.
 //   What such a kernel reads behind the wait may have been written during its own lifetime, so it is read with

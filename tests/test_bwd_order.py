@@ -1,4 +1,4 @@
-"""CPU-only: no product of the backward kernels overwrites tensor memory that an earlier product may still read, read
+"""CPU-only: no product of the backward kernel overwrites tensor memory that an earlier product may still read, read
 from the order of issue in their source.
 
 Products run in their order of issue only if they share accumulator and shape.  At head_dim 128 the next S (or dP) goes over
@@ -8,7 +8,7 @@ import re
 
 import pytest
 
-from test_early_start import kernels, source
+from test_early_start import source
 
 TOKEN = re.compile(r"(issue_s|issue_dp)\(j \+ 1\)|(?:mma_ts|slice)\((t_dq|t_dv|t_dk),|(commit)\((k\w+)|(wait)\(([^,]*)")
 COMPUTE = {"kSFree": "kSFull", "kPHalf": "kSFull", "kPFull": "kSFull", "kDsFull": "kDpFull"}      # and the commit their arrivals are behind
@@ -16,7 +16,8 @@ COMPUTE = {"kSFree": "kSFull", "kPHalf": "kSFull", "kPFull": "kSFull", "kDsFull"
 
 def issued(name):
     """The issuer's step as (what, barrier or product); a product of S or dP with the waits in front of it."""
-    body = kernels(source("attn_bwd.cu"))[name]
+    text = source("attn_bwd.cu")
+    body = text[text.index("void %s<D>::run(" % name):]
     step = body[body.index("issue_s(0)"):body.index("commit(kDone)")]
     for m in TOKEN.finditer(step):
         issue, product, commit, bar, wait, bars = m.groups()
@@ -33,8 +34,8 @@ def issued(name):
             yield "wait", re.findall(r"k[A-Z]\w+", bars)[0]
 
 
-@pytest.mark.parametrize("name,overwrites", [("bwd_dq_kernel", {"issue_dp": {"t_dq"}}),
-                                             ("bwd_dkdv_kernel", {"issue_s": {"t_dv"}, "issue_dp": {"t_dk"}})])
+@pytest.mark.parametrize("name,overwrites", [("DqBlock", {"issue_dp": {"t_dq"}}),
+                                             ("DkdvBlock", {"issue_s": {"t_dv"}, "issue_dp": {"t_dk"}})])
 def test_operands_are_read_before_they_are_overwritten(name, overwrites):
     pending, covers, checked = set(), {"kSFull": set(), "kDpFull": set()}, []
     for what, x in issued(name):

@@ -38,8 +38,8 @@ EARLY = sorted({k for f in FILES for call in re.findall(r"launch_(?:dependent|sp
 
 
 def test_the_early_kernels_are_found():
-    assert EARLY == sorted(["attn_sm100_kernel", "qkv_gemm_kernel", "qkv_finish_kernel", "bwd_delta_kernel", "bwd_dq_kernel",
-                            "bwd_dkdv_kernel", "rope_table_kernel", "rope_append_kernel", "rope_append_e4m3_kernel",
+    assert EARLY == sorted(["attn_sm100_kernel", "qkv_gemm_kernel", "qkv_finish_kernel", "bwd_delta_kernel", "bwd_kernel",
+                            "rope_table_kernel", "rope_append_kernel", "rope_append_e4m3_kernel",
                             "norm_rope_append_kernel", "stage_e4m3_kernel"])
     assert set(EARLY) <= set(ALL)
 
@@ -47,6 +47,14 @@ def test_the_early_kernels_are_found():
 @pytest.mark.parametrize("name", EARLY)
 def test_an_early_kernel_waits_once(name):
     assert ALL[name][1].count("grid_dep_wait()") == 1 and ALL[name][1].count("grid_dep_launch()") == 1
+
+
+@pytest.mark.parametrize("name", EARLY)
+def test_nothing_is_read_before_the_wait(name):
+    """Neither by a copy or a load that the kernel's own text shows, nor by a function that it calls with the launch's pointers."""
+    before = ALL[name][1].split("grid_dep_wait()")[0]
+    assert not re.search(r"tma_load\w*\(|bulk_\w+\(|__ld\w+\(|atomic\w+\(|\*>\(p\.status|\bp\.(q|k|v|x|out|d_out|lse|delta|counters|partial|[thw]_tab)\b", before)
+    assert not re.search(r"\brun\(|load_tile\(|epilogue_rows[<(]|merge_\w+[<(]", before)
 
 
 @pytest.mark.parametrize("name", sorted(set(ALL) - set(EARLY)))
@@ -61,7 +69,7 @@ def test_no_read_only_loads(name):
     assert "__ldg(" not in text and "global.nc" not in text and "__restrict__" not in text
 
 
-@pytest.mark.parametrize("name", ["attn_sm100_kernel", "qkv_gemm_kernel", "bwd_dq_kernel", "bwd_dkdv_kernel", "norm_rope_append_kernel"])
+@pytest.mark.parametrize("name", ["attn_sm100_kernel", "qkv_gemm_kernel", "bwd_kernel", "norm_rope_append_kernel"])
 def test_barriers_are_set_up_before_the_wait(name):
     body = ALL[name][1]
     assert re.search(r"\b(mbar_init|init_barriers)\(", body[:body.index("grid_dep_wait()")])

@@ -1,7 +1,8 @@
-"""The dk/dv kernel of the backward runs beside its dq kernel: calls in a row equal calls with a wait behind each, bit for bit.
+"""The dk/dv blocks of the backward run beside its dq blocks: calls in a row equal calls with a wait behind each, bit for bit.
 
-Few blocks (both kernels side by side), one kernel short of the chip, both longer than it; every call has inputs of its own but shares
-workspace and statistics buffers with the call before, and its gradients are read by the next kernel in the stream."""
+Few blocks (both kinds side by side), one kind short of the chip, both longer than it; every call has inputs and an angle base of its own (so
+the rotation tables are written anew) but shares workspace, statistics buffers and tables with the call before, and its gradients are
+read by the next kernel in the stream."""
 import pytest
 import torch
 
@@ -34,7 +35,7 @@ def test_calls_in_a_row(heads, dim, p, chunks, window):
             for g in grads:
                 g.fill_(float("nan"))
             shifted = lse + 0.01 * i                 # another call's statistics at another time
-            B.ll_clip_attn_backward(cache.h, 0, q_out, out, d_out, shifted, 0, chunks, window, 1, p, 10000.0, *grads, workspace)
+            B.ll_clip_attn_backward(cache.h, 0, q_out, out, d_out, shifted, 0, chunks, window, 1, p, 10000.0 / (1 + i), *grads, workspace)
             got.append([g.clone() for g in grads])   # the next kernel in the stream
             if wait:
                 torch.cuda.synchronize()

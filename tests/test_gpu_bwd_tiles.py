@@ -1,5 +1,5 @@
 """GPU parity of the clip backward at chunk sizes round its 128-row tiles and their 64-row halves: the query columns
-of the dk/dv kernel that are not live, key rows a group does not see, one step and many."""
+of the dk/dv blocks that are not live, key rows a group does not see, one step and many."""
 import pytest
 
 from paper_2509_22622_b200 import synth
