@@ -539,7 +539,7 @@ __device__ __forceinline__ void merge_groups(const AttnParams &p, const WarpRows
 
 template <int D, class Wait>
 __device__ __forceinline__ bool merge_in_cluster(const AttnParams &p, const Segment &s, const WarpRows &wr, int cta, uint32_t t_o, float m_own_a,
-                                                 float m_own_b, float l_own_a, float l_own_b, uint32_t p_smem, uint32_t part_bar, Wait wait)
+                                                 float m_own_b, float l_own_a, float l_own_b, uint32_t p_smem, uint32_t part_bar, bool &told, Wait wait)
 {
     using C = Cfg<D>;
     constexpr int kGroups = D / 8;
@@ -564,6 +564,7 @@ __device__ __forceinline__ bool merge_in_cluster(const AttnParams &p, const Segm
     fence_cluster();
     __syncwarp();
     if (lane < n && lane != rank) mbar_arrive_remote(part_bar, (uint32_t)lane);
+    told = true;
     if (!__all_sync(0xffffffffu, wait())) return false;
     const AttnItem &item = p.item[p.g[s.g].item];
     const float v_scale = item.v_scale ? item.v_scale[s.head] : 1.f;   // 8-bit caches: value codes x scale
@@ -670,7 +671,9 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
     }
 
     WaitCtx ctx{abort_flag, p.status, warp};
-    const bool skip = warp != kTmaWarp && *abort_flag != 0;
+    // (in a cluster another CTA may set the flag at any time: the lanes of a warp agree on what they saw)
+    const bool skip = warp != kTmaWarp && (kParts ? __any_sync(0xffffffffu, *abort_flag != 0) : *abort_flag != 0);
+    bool told = false;                                 // kParts: this warp has arrived at its peers' barriers
     auto wait = [&](int bar_id, uint32_t parity, int iter) -> bool {
         return wait_bar(bar(bar_id), parity & 1u, ctx, bar_id, iter);
     };
@@ -1101,8 +1104,8 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
                 const AttnItem &item = p.item[G.item];
                 if constexpr (kParts) {
                     const int part_bar = kPartFull + wr.slab();
-                    if (!merge_in_cluster<D>(p, s, wr, cta, t_o, m_a, m_b, l_a, l_b, p_smem, bar(part_bar),
-                                             [&]() { return wait_bar<true>(bar(part_bar), 0, ctx, part_bar, s.kt1); }))
+                    if (!merge_in_cluster<D>(p, s, wr, cta, t_o, m_a, m_b, l_a, l_b, p_smem, bar(part_bar), told,
+                                             [&]() { return wait_bar<true>(bar(part_bar), 0, ctx, part_bar, s.kt1) && *abort_flag == 0; }))
                         return;
                 } else if (s.kt0 == 0 && s.kt1 == G.n_kt) {
                     // a whole column: normalise and store
@@ -1182,6 +1185,15 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
     }
 
     // ---- common exit -------------------------------------------------------------
+    // In a cluster every warp that merges arrives at its peers exactly once, whatever becomes of its CTA, and leaves only when
+    // all of them have arrived: a CTA that did not start, or gave up, sets the others' flags in front of its arrivals (value 3), so that
+    // they neither merge rows that are not there nor wait for them.  A CTA that ends with its flag clear has heard of
+    // every peer, and no peer sets it any more.
+    auto merges = [&]() { return kParts && warp < 8 * first->s.n_sub; };
+    if (kParts && !told && merges() && lane < p.cluster_parts && lane != (int)cluster_rank()) {
+        st_shared_remote(smem_u32(tmem_slot + 1), (uint32_t)lane, 3u);
+        mbar_arrive_remote(bar(kPartFull + WarpRows(warp, lane).slab()), (uint32_t)lane);
+    }
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag != 0) {
@@ -1192,11 +1204,10 @@ attn_sm100_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ 
         __syncthreads();
     }
     if (kParts && *abort_flag != 0) {
-        // Every warp that merges has waited for the others' arrivals at its barrier.  A CTA that gave up, or did not start, stays until they have
-        // come, or as long as the others may take to give up themselves.
-        const uint64_t t0 = globaltimer_ns(), limit = *abort_flag == 1 ? 2 * kWaitLimitNs : 50000000ull;
-        if (warp < kSlabs && lane == 0)
-            while (!mbar_try_wait_cluster(bar(kPartFull + warp), 0) && globaltimer_ns() - t0 < limit) __nanosleep(1000);
+        // (the limit is longer than a peer can take to give up)
+        const uint64_t t0 = globaltimer_ns();
+        if (merges() && lane == 0)
+            while (!mbar_try_wait_cluster(bar(kPartFull + warp), 0) && globaltimer_ns() - t0 < 2 * kWaitLimitNs) __nanosleep(1000);
         __syncthreads();
     }
     if (warp == kTmaWarp) {

@@ -15,7 +15,7 @@ namespace ll {
 constexpr uint64_t kWaitLimitNs = 2000000000ull;    // 2 s
 
 struct WaitCtx {
-    volatile int *abort_flag;     // in shared memory: 0 = running, 1 = a wait of this CTA ran out
+    volatile int *abort_flag;     // in shared memory: 0 = running, 1 = a wait of this CTA ran out, others: the CTA ends early for another reason
     uint32_t *status;             // the aux block's status words
     int role;                     // who is waiting (the warp index)
 };

@@ -142,6 +142,18 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
+// Writes to the word that CTA `rank` of the cluster has at the shared-memory address `addr`.
+__device__ __forceinline__ void st_shared_remote(uint32_t addr, uint32_t rank, uint32_t v)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .b32 a;\n\t"
+        "mapa.shared::cluster.u32 a, %0, %1;\n\t"
+        "st.shared::cluster.u32 [a], %2;\n\t"
+        "}" ::"r"(addr), "r"(rank), "r"(v)
+        : "memory");
+}
+
 // Arrives at the barrier that CTA `rank` of the cluster has at the shared-memory address `bar`.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar, uint32_t rank)
 {

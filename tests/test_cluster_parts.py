@@ -170,3 +170,33 @@ def test_clusters_on_two_streams():
         cache.check_device(stream)
         assert torch.equal(out, want)
         cache.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("heads,dim,n_q,n_k,parts", [s for s in SHAPES if s[4]])
+def test_clusters_behind_a_recorded_timeout(heads, dim, n_q, n_k, parts):
+    """Launches behind a time-out that nobody has read yet write nothing and end at once; the same call works when it has been read."""
+    gen = torch.Generator(device="cuda").manual_seed(n_k)
+    q, k, v = (torch.randn(n, heads, dim, device="cuda", generator=gen).to(torch.bfloat16) for n in (n_q, n_k, n_k))
+    cache = B.Cache(1, heads, dim, 16, 1, 1, 1)
+    assert B.ll_debug_attn_plan_cross(cache.h, n_q, n_k).cluster_parts == parts
+    want = torch.empty_like(q)
+    cache.cross_attn(q, k, v, want)
+    cache.check_device()
+    out = torch.full_like(q, 7.0)
+    begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    B.ll_debug_wait_timeout(cache.h, 20)
+    begin.record()
+    for _ in range(10):
+        cache.cross_attn(q, k, v, out)
+    end.record()
+    torch.cuda.synchronize()
+    assert bool((out == 7.0).all())
+    assert begin.elapsed_time(end) < 40.0                # 0.2 ms each, in which copies under way land
+    with pytest.raises(B.LLError) as e:
+        cache.check_device()
+    assert e.value.code == B.LL_ERR_DEVICE_TIMEOUT
+    cache.cross_attn(q, k, v, out)
+    cache.check_device()
+    assert torch.equal(out, want)
+    cache.close()
