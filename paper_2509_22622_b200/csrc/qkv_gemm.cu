@@ -61,8 +61,9 @@ struct GemmCfg {
     static constexpr int kStaging = kStages * kStageBytes; // 16 rows x 64 bytes per epilogue warp
     static constexpr int kBarOff = kStaging + kEpiWarps * 1024;
     static constexpr int kSmem = kBarOff + 1024 /*barriers*/ + 1024 /*alignment*/;
-    // barrier indices: full and acc-empty are the leader's, empty and acc-full each CTA's own
-    static constexpr int kFull = 0, kEmpty = kStages, kAccFull = 2 * kStages, kAccEmpty = 2 * kStages + 2, kBars = 2 * kStages + 4;
+    // barrier indices: full and acc-empty are the leader's, empty and acc-full each CTA's own, start the other CTA's
+    static constexpr int kFull = 0, kEmpty = kStages, kAccFull = 2 * kStages, kAccEmpty = 2 * kStages + 2, kStart = 2 * kStages + 4,
+                         kBars = 2 * kStages + 5;
 };
 
 // ---- pairs of CTAs ----
@@ -226,13 +227,14 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
 {
     using G = GemmCfg<TN>;
     constexpr int kStages = G::kStages, kStageBytes = G::kStageBytes;
-    constexpr int kFull = G::kFull, kEmpty = G::kEmpty, kAccFull = G::kAccFull, kAccEmpty = G::kAccEmpty;
+    constexpr int kFull = G::kFull, kEmpty = G::kEmpty, kAccFull = G::kAccFull, kAccEmpty = G::kAccEmpty, kStart = G::kStart;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     const uint32_t bars = smem_base + G::kBarOff;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_gen + G::kBarOff + G::kBars * 8);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    volatile uint32_t *verdict = tmem_slot + 2;        // the leader's look at the status word: 1 the pair starts, 2 it does not
     auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
@@ -241,8 +243,9 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
 
     grid_dep_launch();
     if (threadIdx.x == 0) {
-        for (int i = 0; i < G::kBars; ++i) mbar_init(bar(i), (i >= kAccEmpty) ? 2u * G::kEpiWarps : 1u);   // both CTAs' epilogue warps free a buffer
+        for (int i = 0; i < G::kBars; ++i) mbar_init(bar(i), (i >= kAccEmpty && i < kStart) ? 2u * G::kEpiWarps : 1u);   // both CTAs' epilogue warps free a buffer
         *abort_flag = 0;
+        *verdict = 0;
         fence_mbar_init();
     }
     if (warp == 0) {
@@ -261,17 +264,24 @@ qkv_gemm_kernel(const __grid_constant__ QkvParams p, const __grid_constant__ CUt
     const uint32_t tmem = *tmem_slot;
     WaitCtx ctx{abort_flag, p.status, warp};
     grid_dep_wait();
-    // An earlier kernel gave up on a wait: the pair does not start (flag value 2).  The load warp does not wait to hear of that, its first
-    // tiles are under way meanwhile; it finds the flag when it runs out of stages.  (In front of the first load stood the read of the
-    // status word, the pair's barrier and a look at the leader's flag: 270 tokens, 256 -> 3 x 1536 with norm 13.3 -> 12.7 us; 312 tokens,
-    // 1024 -> 3 x 192 15.2 -> 14.6; 200 tokens, 2048 -> 3 x 5120 33.3 -> 32.6.)
-    if (warp == 0) {
-        named_arrive(1, G::kThreads);
-    } else {
-        if (threadIdx.x == 32 && *reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk) *abort_flag = 2;
-        named_sync(1, G::kThreads);
+    // An earlier kernel gave up on a wait: the pair does not start (flag value 2).  The leader's look at the status word decides for both
+    // CTAs.  The load warps do not wait to hear of it: their first tiles are under way meanwhile, and they find the flag when they run out
+    // of stages.  (In front of the first load stood the read of the status word, the pair's barrier and a look at the leader's flag:
+    // 270 tokens, 256 -> 3 x 1536 with norm 13.3 -> 12.7 us; 312 tokens, 1024 -> 3 x 192 15.2 -> 14.6; 200 tokens, 2048 -> 3 x 5120
+    // 33.3 -> 32.6.)
+    if (warp == 2) {                                   // (which has nothing else to do)
+        if (rank == 1) {
+            wait_bar<true>(bar(kStart), 0, ctx, kStart, 0);
+        } else if (lane == 0) {
+            *verdict = *reinterpret_cast<volatile uint32_t *>(p.status) != kStatusOk ? 2u : 1u;
+            st_shared_remote(smem_u32(tmem_slot + 2), 1, *verdict);
+            mbar_arrive_remote(bar(kStart), 1);
+        }
+        if (lane == 0 && *verdict != 1u && *abort_flag == 0) *abort_flag = 2;
+        __syncwarp();
     }
-    const bool skip = warp != 0 && *abort_flag != 0;
+    if (warp != 0) named_sync(1, G::kThreads - 32);
+    const bool skip = warp != 0 && *verdict != 1u;
     auto wait = [&](int bar_id, uint32_t parity, int iter) -> bool {
         return wait_bar(bar(bar_id), parity & 1u, ctx, bar_id, iter);
     };

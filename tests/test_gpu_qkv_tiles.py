@@ -69,3 +69,44 @@ def test_tile_edges(heads, dim, gh, gw, d_model, tile_n, per_pair, with_norm):
         # one rounding to bf16 (2^-8 of the element) on fp32 sums of d_model products (1e-4 covers their order)
         assert ((got.double() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-4).all()
     cache.close()
+
+
+@pytest.mark.parametrize("heads,dim,tokens,d_model,tile_n", [(2, 128, 1, 64, 128), (3, 64, 255, 1544, 192), (12, 128, 4680, 136, 256)])
+def test_behind_a_recorded_timeout(heads, dim, tokens, d_model, tile_n):
+    """Projections behind a time-out that nobody has read yet write nothing and end at once, pairs and all; the same call works
+    when it has been read."""
+    width = heads * dim
+    assert B.ll_debug_qkv_tiles(tokens, width, 148)[0] == tile_n
+    gen = torch.Generator(device="cuda").manual_seed(tokens)
+    x = torch.randn(tokens, d_model, device="cuda", generator=gen).to(torch.bfloat16)
+    w = torch.randn(3 * width, d_model, device="cuda", generator=gen).to(torch.bfloat16)
+    cache = B.Cache(1, heads, dim, tokens, 1, 1, 2)
+    q_out = torch.empty(tokens, heads, dim, device="cuda", dtype=torch.bfloat16)
+
+    def project():
+        B.ll_qkv_proj_append(cache.h, 0, x, w, None, None, None, 1e-6, 0, 1, 1, tokens, 10000.0, q_out)
+
+    def rows():
+        return [q_out] + [cache.kv_view(0, i)[:, :tokens] for i in range(2)]
+
+    project()
+    cache.check_device()
+    want = [t.clone() for t in rows()]
+    for t in rows():
+        t.fill_(7.0)
+    begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    B.ll_debug_wait_timeout(cache.h, 20)
+    begin.record()
+    for _ in range(10):
+        project()
+    end.record()
+    torch.cuda.synchronize()
+    assert all(bool((t == 7.0).all()) for t in rows())
+    assert begin.elapsed_time(end) < 40.0                # 0.2 ms each, in which copies under way land
+    with pytest.raises(B.LLError) as e:
+        cache.check_device()
+    assert e.value.code == B.LL_ERR_DEVICE_TIMEOUT
+    project()
+    cache.check_device()
+    assert all(torch.equal(t, a) for t, a in zip(rows(), want))
+    cache.close()
