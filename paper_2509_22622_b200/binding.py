@@ -174,7 +174,7 @@ def lib():
         except ImportError:
             _marshal = None
         if _marshal is not None:
-            _marshal.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name in SIGNATURES})
+            _marshal.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name in SIGNATURES}, C.c_void_p)
             _fast, _ELSEWHERE = _marshal, _marshal.ELSEWHERE
             if _torch_c is not None:
                 _marshal.streams(_torch_c._cuda_getDevice, _torch_c._cuda_getCurrentRawStream)

@@ -11,6 +11,7 @@
 
 static PyObject *get_device, *get_stream;          // torch._C._cuda_getDevice, _cuda_getCurrentRawStream
 static PyObject *s_data_ptr, *s_value, *s_cuda_stream;
+static PyTypeObject *handle_type;                  // ctypes.c_void_p
 static PyObject *not_here;                         // returned for arguments that only ctypes takes (or refuses)
 
 // One argument list being converted: `bad` once something is not of the plain kind.
@@ -47,13 +48,13 @@ static void *as_ptr(Args *x, int i)
     return p;
 }
 
-// A handle: an integer or a c_void_p.
+// A handle: an integer or a c_void_p.  (Whatever else has a `value` is not one: ctypes says what becomes of it.)
 static ll_cache *as_handle(Args *x, int i)
 {
     PyObject *o = x->a[i], *r;
     void *p;
     if (PyLong_Check(o)) return (ll_cache *)(uintptr_t)as_u64(x, o);
-    r = PyObject_GetAttr(o, s_value);
+    r = Py_TYPE(o) == handle_type ? PyObject_GetAttr(o, s_value) : NULL;
     if (!r) { x->bad = 1; return NULL; }
     p = r == Py_None ? NULL : (void *)(uintptr_t)as_u64(x, r);
     Py_DECREF(r);
@@ -203,10 +204,15 @@ static PyObject *sink_window_attn_batched(PyObject *self, PyObject *const *a, Py
     CALL(L.sink_window_attn_batched(items, count, stream));
 }
 
-// bind({name: address}): the library's functions.
-static PyObject *bind(PyObject *self, PyObject *d)
+// bind({name: address}, c_void_p): the library's functions, and the type of a handle.
+static PyObject *bind(PyObject *self, PyObject *const *a, Py_ssize_t n)
 {
     PyObject *o;
+    if (n != 2 || !PyDict_Check(a[0]) || !PyType_Check(a[1])) {
+        PyErr_SetString(PyExc_TypeError, "bind({name: address}, c_void_p)");
+        return NULL;
+    }
+    PyObject *const d = a[0];
 #define TAKE(name)                                              \
     o = PyDict_GetItemString(d, "ll_" #name);                   \
     if (!o) return PyErr_Format(PyExc_KeyError, "ll_" #name);   \
@@ -218,6 +224,8 @@ static PyObject *bind(PyObject *self, PyObject *d)
     TAKE(cross_attn)
     TAKE(qkv_proj_append)
     TAKE(sink_window_attn_batched)
+    Py_INCREF(a[1]);
+    Py_XSETREF(handle_type, (PyTypeObject *)a[1]);
     Py_RETURN_NONE;
 }
 
@@ -235,7 +243,7 @@ static PyObject *streams(PyObject *self, PyObject *const *a, Py_ssize_t n)
 #define FAST(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, NULL}
 static PyMethodDef methods[] = {
     FAST(rope_append_kv), FAST(norm_rope_append_kv), FAST(sink_window_attn), FAST(cross_attn), FAST(qkv_proj_append),
-    FAST(sink_window_attn_batched), FAST(streams), {"bind", bind, METH_O, NULL}, {NULL, NULL, 0, NULL},
+    FAST(sink_window_attn_batched), FAST(streams), FAST(bind), {NULL, NULL, 0, NULL},
 };
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", "Argument marshalling of the hot calls.", -1, methods};
 

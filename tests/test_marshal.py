@@ -81,6 +81,32 @@ def test_same_answers(monkeypatch):
     assert {type(x[3]) for x in native} == {type(None), tuple, str}           # taken, refused by the library, refused on the way
 
 
+class Value:
+    def __init__(self, value):
+        self.value = value
+
+
+class Handle(ctypes.c_void_p):
+    pass
+
+
+def test_same_handles(way):
+    """A handle is an integer or a c_void_p; other things with an address in them are refused before the library sees it."""
+    for name, args in CALLS.items():
+        fn = getattr(B, name)
+        for kind in (ctypes.c_long, ctypes.c_ulong, ctypes.c_uint64, Value):
+            h = handle()
+            with pytest.raises(ctypes.ArgumentError):
+                fn(kind(h.value), *args)
+            with pytest.raises((TypeError, ctypes.ArgumentError)):
+                B.ll_sink_window_attn_batched([(kind(h.value), 0, X, 0, 2, X, None)], 0)
+            B.ll_cache_destroy(h)
+        for kind in (int, ctypes.c_void_p, Handle):
+            h = handle()
+            assert outcome(lambda: fn(kind(h.value), *args)) != "refused"
+            B.ll_cache_destroy(h)
+
+
 def test_batched(way):
     hs = [handle() for _ in range(9)]
     for h in hs:
