@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import os
+import shlex
 import subprocess
 import sys
 import sysconfig
@@ -39,17 +40,23 @@ def _stale() -> bool:
 
 
 def build_marshal(force: bool = False) -> None:
-    """The marshalling module.  Without Python's headers there is none and the binding's ctypes functions serve every call."""
+    """The marshalling module.  Without Python's headers or a compiler that builds it there is none (nor an older one), and the
+    binding's ctypes functions serve every call."""
     include = sysconfig.get_paths()["include"]
     header = os.path.join(ROOT, "include", "llattn.h")
-    if not os.path.exists(os.path.join(include, "Python.h")):
-        return
     if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) > max(map(os.path.getmtime, (MARSHAL_SOURCE, header, __file__))):
         return
     tmp = MARSHAL + ".tmp%d" % os.getpid()
-    subprocess.check_call([os.environ.get("CC") or "gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", include, "-I", os.path.join(ROOT, "include"),
-                           MARSHAL_SOURCE, "-o", tmp])
-    os.replace(tmp, MARSHAL)
+    try:
+        if not os.path.exists(os.path.join(include, "Python.h")):
+            raise OSError("no Python.h in %s" % include)
+        subprocess.check_call(shlex.split(os.environ.get("CC") or "gcc") + ["-O2", "-Wall", "-shared", "-fPIC", "-I", include, "-I",
+                                                                            os.path.join(ROOT, "include"), MARSHAL_SOURCE, "-o", tmp])
+        os.replace(tmp, MARSHAL)
+    except (OSError, ValueError, subprocess.CalledProcessError) as e:
+        sys.stderr.write("the marshalling module has not been built, calls go through ctypes: %s\n" % e)
+        if os.path.exists(MARSHAL):
+            os.remove(MARSHAL)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

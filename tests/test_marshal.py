@@ -124,6 +124,20 @@ def test_batched(way):
         B.ll_cache_destroy(h)
 
 
+@pytest.mark.parametrize("cc,built", [("gcc -m64", True), ("no-such-compiler", False), ("false", False), ("gcc '", False)])
+def test_the_compiler_of_the_environment(cc, built, monkeypatch, tmp_path, capfd):
+    """CC may come with options; one that does not do leaves the module out, an older one too, and does not end the build."""
+    from paper_2509_22622_b200 import build
+    module = tmp_path / "_marshal.so"
+    module.write_bytes(b"older")
+    monkeypatch.setattr(build, "MARSHAL", str(module))
+    monkeypatch.setenv("CC", cc)
+    build.build_marshal(force=True)
+    assert module.exists() == built and (not built or module.read_bytes() != b"older")
+    assert ("has not been built" in capfd.readouterr().err) != built
+    assert [f.name for f in tmp_path.iterdir()] == ["_marshal.so"] * built
+
+
 def test_errors_are_reported(way):
     h = handle()
     with pytest.raises(B.LLError, match="grid"):
