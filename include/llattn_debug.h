@@ -85,6 +85,10 @@ int ll_debug_attn_plan_batched(const ll_attn_item *items, int n_items, int sm_co
 int ll_debug_attn_plan_clip(ll_cache *cache, int layer, int n_frames, int attn_window_frames, int sm_count, ll_attn_plan *out);
 int ll_debug_attn_plan_cross(ll_cache *cache, int64_t n_q, int64_t n_k, int sm_count, ll_attn_plan *out);
 
+/* Lets the handle's calls count on fewer clusters than its device holds at once: held[n] of n thread blocks, n = 2 to 8
+ * (what a GPU whose SMs are arranged differently, or a part of one, would answer).  Host-only. */
+int ll_debug_attn_clusters(ll_cache *cache, const int32_t *held);
+
 /* The tile_ctas, tiles_each and tiles_extra of ll_debug_attn_plan with recache = 0. */
 int ll_debug_attn_tiles(ll_cache *cache, int layer, int sm_count, int *tile_ctas, int *tiles_each, int *tiles_extra);
 

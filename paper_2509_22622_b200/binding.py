@@ -145,6 +145,7 @@ SIGNATURES = {
     "ll_debug_attn_plan_batched": (C.c_int, [C.POINTER(ll_attn_item), C.c_int, C.c_int, C.POINTER(ll_attn_plan)]),
     "ll_debug_attn_plan_clip": (C.c_int, [C.c_void_p] + [C.c_int] * 4 + [C.POINTER(ll_attn_plan)]),
     "ll_debug_attn_plan_cross": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_int, C.POINTER(ll_attn_plan)]),
+    "ll_debug_attn_clusters": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32)]),
     "ll_debug_attn_tiles": (C.c_int, [C.c_void_p, C.c_int, C.c_int] + [C.POINTER(C.c_int)] * 3),
     "ll_debug_norm_rows": (C.c_int, [C.c_int] * 5 + [C.POINTER(C.c_int)]),
     "ll_debug_qkv_tiles": (C.c_int, [C.c_int] * 3 + [C.POINTER(C.c_int)] * 2),
@@ -425,6 +426,11 @@ def ll_debug_attn_plan_cross(h, n_q, n_k, sm_count=0) -> ll_attn_plan:
     plan = ll_attn_plan()
     _check(lib().ll_debug_attn_plan_cross(h, n_q, n_k, sm_count, C.byref(plan)))
     return plan
+
+
+def ll_debug_attn_clusters(h, held):
+    """held: clusters of 0, 1, ... 8 thread blocks."""
+    _check(lib().ll_debug_attn_clusters(h, (C.c_int32 * 9)(*held)))
 
 
 def ll_debug_attn_tiles(h, layer=0, sm_count=0):

@@ -1271,16 +1271,16 @@ cudaError_t launch_instance(const AttnParams &p, const AttnMaps &maps, dim3 grid
 
 namespace {
 
-// Whether the device holds a cluster of n of this kernel's CTAs (a part of a GPU may not); asked once per device and size.
+// Asked once per device and size.
 template <int D>
-bool cluster_fits(int n)
+int clusters_held(int n)
 {
-    constexpr int kMaxDevices = 64, kMaxParts = 8;
-    static std::atomic<signed char> known[kMaxDevices][kMaxParts + 1];      // 0: not asked, 1: yes, -1: no
+    constexpr int kMaxDevices = 64;
+    static std::atomic<int> known[kMaxDevices][kMaxClusterParts + 1];      // 0: not asked, else one more than are held
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || n > kMaxParts) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (dev < kMaxDevices)
-        if (const int k = known[dev][n].load(std::memory_order_acquire)) return k > 0;
+        if (const int k = known[dev][n].load(std::memory_order_acquire)) return k - 1;
     cudaLaunchAttribute attr;
     memset(&attr, 0, sizeof attr);
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1300,11 +1300,13 @@ bool cluster_fits(int n)
         (void)cudaGetLastError();
         held = 0;
     }
-    if (dev < kMaxDevices) known[dev][n].store(held > 0 ? 1 : -1, std::memory_order_release);
-    return held > 0;
+    if (dev < kMaxDevices) known[dev][n].store(held + 1, std::memory_order_release);
+    return held;
 }
 
 }  // namespace
+
+int attn_clusters(int head_dim, int n) { return n < 1 || n > kMaxClusterParts ? 0 : head_dim == 128 ? clusters_held<128>(n) : clusters_held<64>(n); }
 
 cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps &maps, cudaStream_t stream)
 {
@@ -1314,7 +1316,7 @@ cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps 
     long long steps = 0;
     for (int g = 0; g < p.n_groups; ++g) steps += (long long)p.heads * p.g[g].tiles * p.g[g].n_kt;
     const bool early = steps <= kEarlySteps * p.n_ctas;
-    if (p.cluster_parts > 0 && (head_dim == 128 ? cluster_fits<128>(p.cluster_parts) : cluster_fits<64>(p.cluster_parts)))      // else the last part merges
+    if (p.cluster_parts > 0)
         e = head_dim == 128 ? launch_instance<128, kFormParts>(p, maps, grid, early, stream) : launch_instance<64, kFormParts>(p, maps, grid, early, stream);
     else if (head_dim == 128) e = launch_instance<128, kFormTiles>(p, maps, grid, early, stream);
     else if (p.tile_ctas > 0) e = launch_instance<64, kFormTiles>(p, maps, grid, early, stream);

@@ -314,7 +314,7 @@ int qkv_tile_width(int n_tokens, int width, int sm_count)
 // Fewer columns than CTAs, all equally long: every column in the same number of equal parts, one part per
 // CTA, when that is the cheapest way.  In steps, a part costs its own length; splitting at all costs the trip of
 // the parts through the scratch slots and the merge.  Up to eight parts are a thread-block cluster's, whose CTAs merge together
-// (cluster_steps), as long as all clusters are on the chip at once; otherwise whichever part arrives last merges (kTripSteps, and
+// (cluster_steps), as long as the device holds all clusters at once; otherwise whichever part arrives last merges (kTripSteps, and
 // kBatchSteps by four parts).  Against levelled shares it saves a CTA's second column segment
 // (kSegmentSteps: its first loads and its drain) and a part per column.
 //   Against whole columns, the merge of 2 / 4 / 8 parts costs 4.2 / 4.9 / 5.6 us in a cluster and 7 / 9.7 / 18 us where the last part does it (12 heads of
@@ -328,17 +328,12 @@ int qkv_tile_width(int n_tokens, int width, int sm_count)
 // 2.36e-3 where levelled shares of a step or two gave 2.17e-3 to 2.28e-3; that of long columns is up to 2.37e-3 either way.
 //   Returns what the busiest CTA costs that way, in steps; 0 when the launch is not for it.
 constexpr double kTripSteps = 2.5, kBatchSteps = 2.5, kSegmentSteps = 2;
-constexpr int kMaxClusterParts = 8;
 double cluster_steps(long long parts) { return parts == 2 ? 3.5 : parts <= 4 ? 4 : 5; }
-// Clusters of n CTAs with this kernel's shared memory that a B200 holds (cudaOccupancyMaxActiveClusters; more would run one behind another).
-int clusters_at_once(long long n, int sms)
-{
-    static const int held[kMaxClusterParts + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
-    return n <= kMaxClusterParts ? std::min(held[n], sms / (int)n) : 0;
-}
 
-double even_split(ll::AttnParams *p, int sms, long long all_cols)
+// `clusters`: how many clusters of n CTAs are on the chip at once (more would run one behind another).
+double even_split(ll::AttnParams *p, int sms, const int *clusters, long long all_cols)
 {
+    auto at_once = [&](long long n) { return n <= ll::kMaxClusterParts ? std::min(clusters[n], sms / (int)n) : 0; };
     if (all_cols >= sms || all_cols <= 0) return 0;
     const long long n_kt = p->g[0].n_kt;
     for (int g = 1; g < p->n_groups; ++g)
@@ -347,9 +342,9 @@ double even_split(ll::AttnParams *p, int sms, long long all_cols)
     long long best = 1;
     int cluster = 0;
     double cost = (double)n_kt;
-    const double beside = all_cols <= clusters_at_once(2, sms) ? 1 : 0;      // a cluster's merge is taken a step too high: so is the other beside it
+    const double beside = all_cols <= at_once(2) ? 1 : 0;      // a cluster's merge is taken a step too high: so is the other beside it
     for (long long k = 2; k <= std::min<long long>(sms / all_cols, n_kt); ++k) {
-        const bool together = all_cols <= clusters_at_once(k, sms);
+        const bool together = all_cols <= at_once(k);
         const double c = (double)((n_kt + k - 1) / k) + (together ? cluster_steps(k) : merge(k) + beside);
         if (c < cost) { cost = c; best = k; cluster = together ? (int)k : 0; }
     }
@@ -389,13 +384,13 @@ double even_split(ll::AttnParams *p, int sms, long long all_cols)
 // level T of steps, after its whole columns; CTAs already above T take none.
 // Returns what that costs the busiest CTA, in steps, if the columns are equally long (with shares: a column's parts, a second
 // segment and the merge of up to four parts on top of its level of steps).
-double plan_work(ll::AttnParams *p, int sms, long long all_cols, long long all_steps)
+double plan_work(ll::AttnParams *p, int sms, const int *clusters, long long all_cols, long long all_steps)
 {
     const bool waves = all_cols >= sms;
     p->n_ctas = waves ? sms : (int)std::min<long long>(sms, all_steps);
     p->n_waves = waves ? (int)(all_cols / sms) : 0;
     p->all_cols = (int)all_cols;
-    if (const double cost = even_split(p, sms, all_cols)) return cost;
+    if (const double cost = even_split(p, sms, clusters, all_cols)) return cost;
     // What goes out whole and what is left of it, and the steps each CTA gets as whole columns
     long long load[ll::kMaxCtas] = {}, steps = 0;
     const int n = p->n_ctas;
@@ -595,7 +590,7 @@ int build_attn_params(const AttnCall *calls, int n_calls, ll::AttnParams *p)
     if (all_steps > INT32_MAX) return fail(LL_ERR_UNSUPPORTED_SHAPE, "too much work for one launch");
     p->n_groups = ng;
     p->nq_total = p->item[0].nq_total;
-    plan_tiles(p, sms, plan_work(p, sms, all_cols, all_steps), c0->D);
+    plan_tiles(p, sms, plan_work(p, sms, c0->clusters, all_cols, all_steps), c0->D);
     return LL_OK;
 }
 
@@ -801,11 +796,15 @@ int ll_cache_bind_storage(ll_cache *c, void *dev, size_t bytes, ll_stream stream
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(guard bands)");
     }
     cudaPointerAttributes attr;
-    int sms = 0;
+    int sms = 0, current = 0;
     e = cudaPointerGetAttributes(&attr, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, attr.device);
+    if (e == cudaSuccess) e = cudaGetDevice(&current);
+    if (e == cudaSuccess && current != attr.device) e = cudaSetDevice(attr.device);
     if (e != cudaSuccess) return cuda_fail(e, "query of the storage's device");
     c->sm_count = sms;
+    for (int n = 2; n <= ll::kMaxClusterParts; ++n) c->clusters[n] = ll::attn_clusters(c->D, n);
+    if (current != attr.device) (void)cudaSetDevice(current);
     std::vector<CUtensorMap> km(c->L), vm(c->L);
     char *base = static_cast<char *>(dev) + c->aux_bytes;
     if (c->kv_format == LL_KV_E4M3) {
@@ -1440,6 +1439,16 @@ int ll_debug_qkv_tiles(int n_tokens, int width, int sm_count, int *tile_n, int *
     if (!tn) return fail(LL_ERR_UNSUPPORTED_SHAPE, "no tile width divides %d", width);
     *tile_n = tn;
     *tiles_per_pair = (int)qkv_rounds(n_tokens, width, sm_count, tn);
+    return LL_OK;
+}
+
+int ll_debug_attn_clusters(ll_cache *c, const int32_t *held)
+{
+    if (!c || !held) return fail(LL_ERR_INVALID_ARG, "null argument to ll_debug_attn_clusters");
+    for (int n = 2; n <= ll::kMaxClusterParts; ++n) {
+        if (held[n] < 0 || held[n] > c->clusters[n]) return fail(LL_ERR_INVALID_ARG, "%d clusters of %d", (int)held[n], n);
+        c->clusters[n] = held[n];
+    }
     return LL_OK;
 }
 

@@ -25,6 +25,7 @@ constexpr int kStatusWords = 64;      // uint32 words at the head of the aux blo
 constexpr int kQTileRows = 256;       // query rows of one work column (two 128-row MMA tiles)
 constexpr int kKeyTile = 128;         // keys per MMA tile
 constexpr int kMaxCtas = 160;         // persistent CTAs one attention launch may use
+constexpr int kMaxClusterParts = 8;   // CTAs of a cluster that hold the parts of one column
 constexpr int kSlabs = 16;            // 16-row warp slabs in a work column (2 tiles x 8)
 
 // status word 0 is non-zero when a kernel abandoned a wait; words 1.. hold details
@@ -320,6 +321,8 @@ bool norm_append_streams(int heads, int head_dim, int n_tokens, bool with_q, int
 cudaError_t launch_norm_rope_append(const RopeAppendParams &p, int head_dim, const float *gain_q, const float *gain_k,
                                     float eps, int sm_count, cudaStream_t stream);
 cudaError_t launch_attn_sm100(const AttnParams &p, int head_dim, const AttnMaps &maps, cudaStream_t stream);
+// Clusters of n (up to kMaxClusterParts) CTAs of the attention kernel that the current device holds at once.
+int attn_clusters(int head_dim, int n);
 cudaError_t launch_attn_simt(const AttnParams &p, int head_dim, cudaStream_t stream);
 // what the probe of the bounded-wait machinery records as barrier and iteration
 constexpr int kProbeBarrierId = 99;
@@ -345,6 +348,8 @@ struct ll_cache {
     // aux block layout (byte offsets from storage)
     size_t off_status = 0, off_ttab = 0, off_hwtab = 0, off_counters = 0, off_partial = 0, aux_bytes = 0;
     int sm_count = 0;                 // of the device the storage lives on
+    // attn_clusters of that device by number of CTAs; without storage those of a whole B200
+    int clusters[ll::kMaxClusterParts + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
     size_t kv_bytes = 0;              // one K (or V) matrix set of one layer in bf16: H*rows*D*2
     size_t kv_store_bytes = 0;        // the same as stored: kv_bytes, or half of it for E4M3 codes
     std::vector<CUtensorMap> kmap, vmap;

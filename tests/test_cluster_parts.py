@@ -44,6 +44,41 @@ def test_where_clusters_are_used(heads, dim, n_q, n_k, parts):
         assert list(plan.share_begin[:plan.n_shares + 1]) == cuts
 
 
+# what a device holds of each size; parts of SHAPES[0] (72 columns of 47 steps) and SHAPES[6] (12 columns of 14)
+@pytest.mark.parametrize("held,parts", [([0, 148, 74, 45, 33, 26, 22, 15, 15], (2, 7)), ([0, 148, 71, 45, 33, 26, 22, 11, 15], (0, 8)),
+                                        ([0, 148, 74, 45, 11, 26, 22, 0, 0], (2, 5)), ([0] * 9, (0, 0))])
+def test_the_device_says_how_many_clusters(held, parts):
+    """Clusters that would run one behind another are not planned with."""
+    for (heads, dim, n_q, n_k, _), want in zip((SHAPES[0], SHAPES[6]), parts):
+        h = handle(heads, dim)
+        B.ll_debug_attn_clusters(h, held)
+        assert B.ll_debug_attn_plan_cross(h, n_q, n_k).cluster_parts == want
+        with pytest.raises(B.LLError):
+            B.ll_debug_attn_clusters(h, [0, 0, 75] + [0] * 6)
+        B.ll_cache_destroy(h)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("heads,dim,n_q,n_k,parts", [s for s in SHAPES if s[4]])
+def test_without_clusters(heads, dim, n_q, n_k, parts):
+    """The same launches on a device that holds none: the part that arrives last merges, or nothing is split."""
+    from gpu_util import check_attn, f64
+    gen = torch.Generator(device="cuda").manual_seed(n_q)
+    q, k, v = (torch.randn(n, heads, dim, device="cuda", generator=gen).to(torch.bfloat16) for n in (n_q, n_k, n_k))
+    cache = B.Cache(1, heads, dim, 16, 1, 1, 1)
+    B.ll_debug_attn_clusters(cache.h, [0] * 9)
+    assert B.ll_debug_attn_plan_cross(cache.h, n_q, n_k).cluster_parts == 0
+    s = torch.einsum("qhd,khd->hqk", q.double(), k.double()) * dim ** -0.5
+    want = torch.einsum("hqk,khd->qhd", s.softmax(-1), v.double()).cpu().numpy()
+    for _ in range(2):
+        out, lse = torch.full_like(q, float("nan")), torch.full((heads, n_q), float("nan"), device="cuda")
+        cache.cross_attn(q, k, v, out, lse)
+        cache.check_device()
+        check_attn(f64(out), want)
+        assert (lse.double() - s.logsumexp(-1)).abs().max().item() <= 1e-4
+    cache.close()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("heads,dim,n_q,n_k,parts", [s for s in SHAPES if s[4]])
 def test_cluster_parts(heads, dim, n_q, n_k, parts):
