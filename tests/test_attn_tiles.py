@@ -46,7 +46,10 @@ def check_tiles(plan, rows, dim, sms):
     split = 0.
     if plan.n_shares:
         equal = plan.n_waves == 0 and plan.n_ctas == plan.n_shares and plan.n_shares % plan.all_cols == 0
-        split = 2.5 + 2.5 * ((plan.n_shares // plan.all_cols + 3) // 4) if equal else 8.
+        parts = plan.n_shares // plan.all_cols
+        held = [0, 148, 74, 45, 33, 26, 22, 15, 15][parts] if parts <= 8 else 0          # clusters, whose CTAs merge together
+        together = plan.all_cols <= min(held, sms // max(parts, 1))
+        split = 8. if not equal else (3.5 if parts == 2 else 4. if parts <= 4 else 5.) if together else 2.5 + 2.5 * ((parts + 3) // 4)
     by_columns = max(sum(k1 - k0 for _, _, k0, k1 in cta_work(plan, i)) for i in range(plan.n_ctas)) + split
     assert by_tiles < by_columns
     return segs

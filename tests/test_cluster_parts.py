@@ -67,7 +67,8 @@ def test_without_clusters(heads, dim, n_q, n_k, parts):
     q, k, v = (torch.randn(n, heads, dim, device="cuda", generator=gen).to(torch.bfloat16) for n in (n_q, n_k, n_k))
     cache = B.Cache(1, heads, dim, 16, 1, 1, 1)
     B.ll_debug_attn_clusters(cache.h, [0] * 9)
-    assert B.ll_debug_attn_plan_cross(cache.h, n_q, n_k).cluster_parts == 0
+    plan = B.ll_debug_attn_plan_cross(cache.h, n_q, n_k)
+    assert (plan.cluster_parts, plan.tile_ctas) == (0, 0) and plan.n_shares > plan.all_cols
     s = torch.einsum("qhd,khd->hqk", q.double(), k.double()) * dim ** -0.5
     want = torch.einsum("hqk,khd->qhd", s.softmax(-1), v.double()).cpu().numpy()
     for _ in range(2):

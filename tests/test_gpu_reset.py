@@ -96,8 +96,9 @@ def test_a_reported_timeout_also_clears_the_merge_counters(oracle_mod):
         q_out = torch.empty_like(dq)
         cache.rope_append_kv(0, dq, dev(k), dev(v), chunk * C, wl.grid_h, wl.grid_w, wl.rope_theta, q_out)
         orc.append(0, F64(k), F64(v), chunk * C, wl.grid_h, wl.grid_w, wl.rope_theta)
+    B.ll_debug_attn_clusters(cache.h, [0] * 9)                        # (in clusters nothing is counted)
     plan = B.ll_debug_attn_plan(cache.h, 0, False, 0)
-    assert plan.n_shares > 0                                          # this launch merges split columns
+    assert plan.n_shares > 0 and plan.cluster_parts == 0              # this launch merges split columns and counts the parts
     s_off, s_bytes, c_off, c_bytes = B.ll_debug_aux_layout(cache.h)
     counters = cache.storage[c_off:c_off + c_bytes].view(torch.int32)
     status = cache.storage[s_off:s_off + s_bytes].view(torch.int32)
