@@ -321,11 +321,14 @@ int qkv_tile_width(int n_tokens, int width, int sm_count)
 // 128, 154 queries; a step there is 1.75 us).  14 / 22 / 40 steps: 27.5 / 38.5 / 64.4 us whole, 21.8 / 25.0 / 31.3 us in
 // four parts merged by the last, 14.5 / 16.3 / 20.1 us in clusters of eight; 72 columns of 22 / 40 steps (1400 queries) in two parts 33.3 / 47.0 us merged by
 // the last, 30.7 / 46.6 us in clusters.  48 columns in three parts (more than 45 clusters) against clusters of two, head_dim 64: 14 steps
-// 19.6 / 17.6 us, 22 steps 23.3 / 23.1, 40 steps 31.2 / 35.2.  All costs but the lengths are taken a little high (about a step): near
-// the line whole columns, tiles and fewer parts are as fast, and fewer parts round less:
-//   Every part takes its weights against references of its own, and the largest weight of a row and part is exactly 1
-// in bf16: with fewer parts fewer weights are exact.  Against 64 bits the relative error of few short columns is 2.25e-3 to
-// 2.36e-3 where levelled shares of a step or two gave 2.17e-3 to 2.28e-3; that of long columns is up to 2.37e-3 either way.
+// 19.6 / 17.6 us, 22 steps 23.3 / 23.1, 40 steps 31.2 / 35.2.
+//   All costs but the lengths are taken about a step high, because those of 128-row tiles (plan_tiles) are weighed against them.  Taken as
+// measured (2.4 / 2.8 / 3.2 steps), launches that go out by tiles are split and mostly lose: 8 heads of 128, 192 queries over 736 keys 11.3 us by
+// tiles, 12.9 in six parts; 40 heads, 196 over 1250 16.8 and 18.2; 8 heads, 1880 over 1670 21.0 and 22.2; but 3 heads, 982 over 974 13.4
+// and 12.6.  Against whole columns and fewer parts the line lies too high for that: 3 heads, 27 over 724 10.9 us whole, 9.0 in six
+// parts; 40 heads of 64, 117 over 789 11.8 and 10.2 in three; 12 heads of 128, 26 over 1081 11.4 in three, 10.6 in five.
+//   Every part takes its weights against references of its own and the weights are rounded to bf16, so that results differ by 2e-3 to 3e-3 between
+// numbers of parts; the error against 64 bits is the same, 2.2e-3 to 2.4e-3 with one part or eight.
 //   Returns what the busiest CTA costs that way, in steps; 0 when the launch is not for it.
 constexpr double kTripSteps = 2.5, kBatchSteps = 2.5, kSegmentSteps = 2;
 double cluster_steps(long long parts) { return parts == 2 ? 3.5 : parts <= 4 ? 4 : 5; }
