@@ -90,8 +90,8 @@ static_assert(kSoftmaxWarps * kSoftmaxRegs + (kThreads / 32 - kSoftmaxWarps) * k
 // waits for, and the cubic's ten instructions per pair cost time and power (0.4027 ms against
 // 0.4047 ms with one group in four, 0.4218 ms with two; 0.4664 / 0.4715 / 0.4915 ms in a long
 // loop at the power cap).  head_dim 64 has twice the exponentials per flop and is bound by
-// them: one group in four (0.681 ms against 0.726 ms with none, 0.684 / 0.683 ms with one in
-// eight / three in eight, 24 heads on the same grid; measured when the loop still took half a score tile at a time).
+// them: one group in four (24 heads on the same grid, 605 us in bursts and 672 in a loop; the other 14 of 15 masks of none
+// to half of the groups take 606 to 718 and 671 to 782).
 template <int D> constexpr uint32_t kPolyMask = D == 64 ? 0x8888u : 0x0000u;
 
 template <int D>
