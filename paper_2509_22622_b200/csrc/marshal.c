@@ -1,5 +1,6 @@
 // The calls of a denoising pass without ctypes: a CPython module that takes the arguments of the binding's functions, turns them
-// into those of the C ABI and returns the status code.  Marshalling only, as in binding.py, whose ctypes functions it stands in for.
+// into those of the C ABI and returns the status code.  Marshalling only, as in binding.py, whose ctypes functions it stands in for:
+// what is not of the plain kind (an integer where the ABI has a float, a numpy scalar) is left to them, at their price.
 //   Of an append's 5.2 us of host time 2.1 were the launch and 2.0 the Python functions and ctypes' conversions (0.8 now), where the kernel of
 // a small one runs for 2.1 us: 360 tokens, 2 heads of 128: 5.2 -> 3.65 us a call in a row; append and attention of 16 tokens
 // 10.0 -> 7.5 us; six streams of 115 tokens, 16 heads of 64: 41.4 -> 27.5 us a step.
